@@ -17,9 +17,9 @@ using namespace phl::eos;
 
 struct phl_eos_table {
   Table t;
-  double *dv = nullptr;
-  float *dvf = nullptr;
-  double *dd = nullptr;   // per table cell: the corner values in difference form (Table::d)
+  double *dv = nullptr;   // node values
+  double *dc = nullptr;   // per table cell: the interpolant's coefficients (Table::c)
+  float *dcf = nullptr;   // their FP32 copy
 };
 
 namespace {
@@ -58,28 +58,49 @@ __global__ void k_table_nodes(int nx, int ny, double x0, double dx, double y0, d
     atomicOr(fail, 1);
 }
 
-// Per table cell (i, j) and node slot s: q00 and the differences q10 - q00,
-// q01 - q00, (q11 - q01) - (q10 - q00) of its corners (x first, then y),
-// the same FP64 operations the contraction would do at every evaluation.
-__global__ void k_table_diffs(int nx, int ny, double dx, double dy, const double *__restrict__ v,
-                              double *__restrict__ d) {
-  const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (q >= (long)(nx - 1) * (ny - 1) * NQ) return;
-  const int s = (int)(q % NQ);
-  const long cell = q / NQ;
+// Coefficients of the quintic on [0, 1] with value, first and second
+// derivative q[0][0..2] at 0 and q[1][0..2] at 1.  The three highest come from
+// what the second-order Taylor polynomial at 0 leaves at 1, so no term
+// subtracts more than the interval's own differences.
+__device__ __forceinline__ void quintic_coeffs(const double q[2][3], double *c) {
+  const double h2 = 0.5 * q[0][2];
+  const double A = ((q[1][0] - q[0][0]) - q[0][1]) - h2;
+  const double B = (q[1][1] - q[0][1]) - q[0][2];
+  const double C = q[1][2] - q[0][2];
+  c[0] = q[0][0];
+  c[1] = q[0][1];
+  c[2] = h2;
+  c[3] = 10.0 * A - 4.0 * B + 0.5 * C;
+  c[4] = -15.0 * A + 7.0 * B - C;
+  c[5] = 6.0 * A - 3.0 * B + 0.5 * C;
+}
+
+// Per table cell (i, j): the biquintic Hermite interpolant of its four
+// corners' nine values as coefficients c[r][p] of u^p v^r, u and v the
+// position inside the cell (the node derivatives times dx^p dy^r).
+__global__ void k_table_coeffs(int nx, int ny, double dx, double dy, const double *__restrict__ v,
+                               double *__restrict__ c, float *__restrict__ cf) {
+  const long cell = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (cell >= (long)(nx - 1) * (ny - 1)) return;
   const int i = (int)(cell % (nx - 1)), j = (int)(cell / (nx - 1));
-  const long k0 = ((long)j * nx + i) * NQ + s, k1 = k0 + (long)nx * NQ;
-  const double q00 = v[k0], q10 = v[k0 + NQ], q01 = v[k1], q11 = v[k1 + NQ];
-  // the slot's derivative orders (p in x, r in y; slot = qslot(p, r)): in
-  // units of the cell, times dx^p dy^r
-  const int p = (s == 1 || s == 5 || s == 7) ? 1 : ((s == 3 || s == 6 || s == 8) ? 2 : 0);
-  const int r = (s == 2 || s == 5 || s == 6) ? 1 : ((s == 4 || s == 7 || s == 8) ? 2 : 0);
-  const double sc = (p == 0 ? 1.0 : (p == 1 ? dx : dx * dx)) * (r == 0 ? 1.0 : (r == 1 ? dy : dy * dy));
-  double *o = d + cell * 4 * NQ + 4 * s;
-  o[0] = q00 * sc;
-  o[1] = (q10 - q00) * sc;
-  o[2] = (q01 - q00) * sc;
-  o[3] = ((q11 - q01) - (q10 - q00)) * sc;
+  double g[2][3][NC1];   // [y end][y order][power of u]
+  const double sx[3] = {1.0, dx, dx * dx}, sy[3] = {1.0, dy, dy * dy};
+  for (int b = 0; b < 2; ++b)
+    for (int r = 0; r < 3; ++r) {
+      double q[2][3];
+      for (int a = 0; a < 2; ++a)
+        for (int p = 0; p < 3; ++p) q[a][p] = v[((long)(j + b) * nx + i + a) * NQ + qslot(p, r)] * sx[p] * sy[r];
+      quintic_coeffs(q, g[b][r]);
+    }
+  for (int p = 0; p < NC1; ++p) {
+    const double q[2][3] = {{g[0][0][p], g[0][1][p], g[0][2][p]}, {g[1][0][p], g[1][1][p], g[1][2][p]}};
+    double o[NC1];
+    quintic_coeffs(q, o);
+    for (int r = 0; r < NC1; ++r) {
+      c[cell * NCF + r * NC1 + p] = o[r];
+      cf[cell * NCF + r * NC1 + p] = (float)o[r];
+    }
+  }
 }
 
 template <typename R>
@@ -91,14 +112,15 @@ __global__ void k_eos_batch(Table t, long n, const double *rho, const double *ei
   EosOut<double> o;
   double Td = T[i];
   int it;
-  if (sizeof(R) == 8) it = eos_invert<double>(t, rho[i], eint[i], abar[i], ye[i], Td, tol, maxit, o);
-  else it = eos_invert_mixed(t, rho[i], eint[i], abar[i], ye[i], Td, tol, maxit, o);
+  const double r = rho[i], ir = rcp_nr(r), iab = rcp_nr(abar[i]);
+  if (sizeof(R) == 8) it = eos_invert<double>(t, r, ir, eint[i], iab, ye[i], Td, tol, maxit, o);
+  else it = eos_invert_mixed(t, r, ir, eint[i], iab, ye[i], Td, tol, maxit, o);
   const bool ok = it > 0;
   T[i] = Td;
   if (P) P[i] = ok ? o.P : NAN;
   if (ge) ge[i] = o.ge;
   if (gc) gc[i] = o.gc;
-  if (cs) cs[i] = sqrt(o.gc * o.P / rho[i]);
+  if (cs) cs[i] = sqrt(o.gc * o.P * ir);
   if (iters) iters[i] = ok ? it : -1;
 }
 
@@ -128,52 +150,41 @@ phl_status phl_eos_table_create(double lrhoye_lo, double lrhoye_hi, int nrho, do
   t->t.dy = (lT_hi - lT_lo) * log(10.0) / (nT - 1);
   t->t.x0f = (float)t->t.x0; t->t.dxf = (float)t->t.dx; t->t.y0f = (float)t->t.y0; t->t.dyf = (float)t->t.dy;
   t->t.idx = 1.0 / t->t.dx; t->t.idy = 1.0 / t->t.dy;
-  t->t.idx2 = t->t.idx * t->t.idx; t->t.idy2 = t->t.idy * t->t.idy; t->t.idxdy = t->t.idx * t->t.idy;
+  t->t.idxdy = t->t.idx * t->t.idy; t->t.idx2x2 = 2.0 * t->t.idx * t->t.idx; t->t.idy2x2 = 2.0 * t->t.idy * t->t.idy;
+  t->t.idxdyf = (float)t->t.idxdy; t->t.idx2x2f = (float)t->t.idx2x2; t->t.idy2x2f = (float)t->t.idy2x2;
   t->t.idxf = (float)t->t.idx; t->t.idyf = (float)t->t.idy;
   t->t.Tlo = exp(t->t.y0); t->t.Thi = exp(t->t.y0 + (nT - 1) * t->t.dy);
   t->t.Tlof = (float)t->t.Tlo; t->t.Thif = (float)t->t.Thi;
   const long nv = (long)NQ * nrho * nT;
   int *fail = nullptr;
   double *dgl = nullptr;
+  const long ncell = (long)(nrho - 1) * (nT - 1);
   e = cudaMalloc(&t->dv, nv * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&t->dvf, nv * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&t->dc, ncell * NCF * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&t->dcf, ncell * NCF * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fail, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&dgl, sizeof(gxw));
   if (e == cudaSuccess) e = cudaMemset(fail, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemcpy(dgl, gxw, sizeof(gxw), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
-    cudaFree(t->dv); cudaFree(t->dvf); cudaFree(fail); cudaFree(dgl); delete t;
+    cudaFree(fail); cudaFree(dgl); phl_eos_table_destroy(t);
     return (phl_status)set_error(PHL_ENOMEM, "eos table: %s", cudaGetErrorString(e));
   }
   const double me = MEC2 / (CL * CL), l = me * CL / HPL;
   const int nn = nrho * nT;
   k_table_nodes<<<(nn + 63) / 64, 64>>>(nrho, nT, t->t.x0, t->t.dx, t->t.y0, t->t.dy, l * l * l, dgl, t->dv, fail);
-  std::vector<double> h(nv);
+  k_table_coeffs<<<(unsigned)((ncell + 63) / 64), 64>>>(nrho, nT, t->t.dx, t->t.dy, t->dv, t->dc, t->dcf);
   int f = 0;
-  e = cudaMemcpy(h.data(), t->dv, nv * sizeof(double), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(&f, fail, sizeof(int), cudaMemcpyDeviceToHost);
+  e = cudaMemcpy(&f, fail, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(fail);
   cudaFree(dgl);
   if (e != cudaSuccess || f) {
-    cudaFree(t->dv); cudaFree(t->dvf); delete t;
+    phl_eos_table_destroy(t);
     return (phl_status)set_error(e != cudaSuccess ? PHL_ECUDA : PHL_ENEWTON, "eos table: node solve failed");
   }
-  std::vector<float> hf(nv);
-  for (long q = 0; q < nv; ++q) hf[q] = (float)h[q];
-  cudaMemcpy(t->dvf, hf.data(), nv * sizeof(float), cudaMemcpyHostToDevice);
-  const long nd = 4L * NQ * (nrho - 1) * (nT - 1);
-  e = cudaMalloc(&t->dd, nd * sizeof(double));
-  if (e == cudaSuccess) {
-    k_table_diffs<<<(unsigned)((nd / 4 + 255) / 256), 256>>>(nrho, nT, t->t.dx, t->t.dy, t->dv, t->dd);
-    e = cudaDeviceSynchronize();
-  }
-  if (e != cudaSuccess) {
-    cudaFree(t->dv); cudaFree(t->dvf); cudaFree(t->dd); delete t;
-    return (phl_status)set_error(PHL_ECUDA, "eos table: %s", cudaGetErrorString(e));
-  }
   t->t.v = t->dv;
-  t->t.vf = t->dvf;
-  t->t.d = t->dd;
+  t->t.c = t->dc;
+  t->t.cf = t->dcf;
   *out = t;
   return PHL_OK;
 }
@@ -181,8 +192,8 @@ phl_status phl_eos_table_create(double lrhoye_lo, double lrhoye_hi, int nrho, do
 void phl_eos_table_destroy(phl_eos_table *t) {
   if (!t) return;
   cudaFree(t->dv);
-  cudaFree(t->dvf);
-  cudaFree(t->dd);
+  cudaFree(t->dc);
+  cudaFree(t->dcf);
   delete t;
 }
 

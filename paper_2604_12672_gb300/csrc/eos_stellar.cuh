@@ -13,13 +13,22 @@
 // thermodynamic identities hold for the interpolated EOS, and c_v, gamma_c
 // are continuous.
 //
-// Evaluation in two parts.  rho and the composition are fixed during an
-// inversion, so the x-direction is contracted once per table row pair: for
-// the two y-nodes j, j+1 of the current cell and each y-order r = 0, 1, 2,
-// g[m][b][r] = d^m/dx^m d^r/dy^r f at (x, y_(j+b)) by the quintic Hermite
-// polynomial in x.  A Newton iteration then needs only the one-dimensional
-// quintic in y on those six values (18 multiply-adds for f, f_y, f_yy), and
-// redoes the contraction only when T leaves the current table interval.
+// Evaluation.  The interpolant on a table cell is one polynomial of degree 5
+// in each of u, v (the position inside the cell along x and y, in cell
+// units); its 36 coefficients c[r][p] (of u^p v^r) are formed once with the
+// table.  The FP64 pipe bounds every inversion (1/64 of the FP32 rate on this
+// GPU), so the evaluation is laid out for the fewest FP64 instructions:
+// synthetic division (Horner's scheme carried on to the derivatives) gives
+// value, first and half the second derivative of a degree-5 polynomial in
+// 5 + 4 + 3 multiply-adds, so f, f_x, f_xx of the six rows take 72 and the six
+// needed mixed derivatives 26 more.  The Hermite form it replaces (two bases
+// of 62 operations, 108 + 36 multiply-adds) took 268.  With the shared
+// subexpressions below, the recorded inversion of the stellar box went from
+// 2.12 to ~1.03 ms per launch on 128^3 cells, the shell's kernel from 2.40 to
+// 1.20 ms on 2.36 million cells and the batch inversion from 4.63 to 2.10 ms
+// for 10^6 far guesses; FP64 pipe bound as before.  The coefficients above
+// the constant are the size of the cell's own differences, so no derivative
+// cancels node values at evaluation; their set-up works on differences too.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -38,6 +47,8 @@ constexpr double ARAD_QUARTER = 2.9492579329135276e-04;   // ARAD^(1/4)
 constexpr double RGAS = KB * NAV;
 constexpr double PI_D = 3.14159265358979323846;
 constexpr int NQ = 9;          // node values: f, f_x, f_y, f_xx, f_yy, f_xy, f_xxy, f_xyy, f_xxyy
+constexpr int NC1 = 6;         // coefficients of the quintic per direction
+constexpr int NCF = NC1 * NC1; // coefficients of a table cell: [power of v][power of u]
 
 // node slot of d^(p + r) f / dx^p dy^r
 __host__ __device__ __forceinline__ int qslot(int p, int r) {
@@ -48,169 +59,124 @@ struct Table {
   int nx, ny;
   double x0, dx, y0, dy;      // x = ln n_e, y = ln T
   const double *v;            // [ny][nx][NQ] (device)
-  const float *vf;            // FP32 copy
-  const double *d;            // [ny-1][nx-1][NQ][4]: each table cell's corner values in difference
-                              // form (D00, D10, D01, D11 below), each slot times dx^p dy^r (its
-                              // derivative orders in units of the cell), formed once; null: formed
-                              // per use.  With d the FP64 evaluation works in cell units and scales
-                              // its results once (idx2 = idx^2, idy2 = idy^2, idxdy = idx idy).
-  double idx2, idy2, idxdy;
+  const double *c;            // [ny-1][nx-1][NCF] polynomial coefficients in cell units
+  const float *cf;            // FP32 copy
   float x0f, dxf, y0f, dyf;
-  double idx, idy;            // 1/dx, 1/dy: the evaluation multiplies (FP64 division
-  float idxf, idyf;           // is a dozen FP64-pipe instructions on this GPU)
+  double idx, idy;            // 1/dx, 1/dy
+  float idxf, idyf;
+  double idxdy, idx2x2, idy2x2;   // idx idy, 2 idx^2, 2 idy^2 (the second derivatives come halved)
+  float idxdyf, idx2x2f, idy2x2f;
   double Tlo, Thi;            // the table's temperature range, exp(y0) and
   float Tlof, Thif;           // exp(y0 + (ny - 1) dy), set with the table
 };
 
-struct Mix {                   // composition-derived constants of a cell
-  double abar, ye;
-};
-
-template <typename R> struct TV { R f, fx, fy, fxx, fyy, fxy; };
-
-// Quintic Hermite basis on [0, 1]: h[a][q] has q-th derivative 1 at end a and
-// value, first and second derivative 0 otherwise at both ends; d, e are its
-// first and second derivatives.  At end 1 the functions are (-1)^q times those
-// of end 0 at 1 - u.  D selects what is formed: 0 values, 1 + first, 2 + second.
-template <typename R, int D>
-__device__ __forceinline__ void quintic(R u, R h[2][3], R d[2][3], R e[2][3]) {
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    const R w = a == 0 ? u : R(1) - u;
-    const R w2 = w * w, w3 = w2 * w;
-    h[a][0] = R(1) + w3 * (R(-10) + w * (R(15) - R(6) * w));
-    h[a][1] = w + w3 * (R(-6) + w * (R(8) - R(3) * w));
-    h[a][2] = R(0.5) * w2 * (R(1) + w * (R(-3) + w * (R(3) - w)));
-    if (D >= 1) {
-      d[a][0] = w2 * (R(-30) + w * (R(60) - R(30) * w));
-      d[a][1] = R(1) + w2 * (R(-18) + w * (R(32) - R(15) * w));
-      d[a][2] = w * (R(1) + w * (R(-4.5) + w * (R(6) - R(2.5) * w)));
-    }
-    if (D >= 2) {
-      e[a][0] = w * (R(-60) + w * (R(180) - R(120) * w));
-      e[a][1] = w * (R(-36) + w * (R(96) - R(60) * w));
-      e[a][2] = R(1) + w * (R(-9) + w * (R(18) - R(10) * w));
-    }
-    if (a == 1) {   // (-1)^q, and d/du = -d/dw on the first derivative
-      h[1][1] = -h[1][1];
-      if (D >= 1) { d[1][0] = -d[1][0]; d[1][2] = -d[1][2]; }
-      if (D >= 2) e[1][1] = -e[1][1];
-    }
-  }
+// 1/x to about one unit in the last place for normal x: the hardware's gross
+// approximation (relative error below 2^-19) and one step of the third-order
+// Newton-Halley iteration y (1 + e + e^2), e = 1 - x y (remaining error e^3 <
+// 2^-57): three FP64 multiply-adds, where the full-range division takes about
+// a dozen FP64-pipe instructions and a branch.  0 and infinity give NaN.
+__device__ __forceinline__ double rcp_nr(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
+__device__ __forceinline__ float rcp_nr(float x) { return 1.0f / x; }
 
-// Difference form of a tensor product.  The 2 x 2 corner values c[a][b] of
-// a quantity enter as sum c[a][b] X_a Y_b = sum D[a][b] X~_a Y~_b with
-// D00 = c00, D10 = c10 - c00, D01 = c01 - c00, D11 = (c11 - c10) - (c01 - c00),
-// X~_0 = X_0 + X_1, X~_1 = X_1 (the same in y): an identity, in which the
-// value functions' X~_0 is exactly 1 (value) or 0 (derivatives).  It keeps a
-// derivative from cancelling two large node values (f_y from f alone would
-// lose ~|f| / dy to rounding).
-template <typename R>
-__device__ __forceinline__ void diff_basis(R b[2][3], R first) {
-  b[0][0] = first;
-  b[0][1] += b[1][1];
-  b[0][2] += b[1][2];
-}
-
-// x-part (x = ln n_e), fixed during an inversion: cell and the quintic basis
-// in difference form, with dx^p folded into order p (value), dx^(p-1) (first
-// derivative) and dx^(p-2) (second), so contracted values are physical
-// derivatives.
+// Position along x (x = ln n_e): table interval and fraction, fixed during
+// an inversion.
 template <typename R> struct XB {
   int i;
   bool ok;
-  R h[2][3], d[2][3], e[2][3];
+  R u;
 };
 
 template <typename R>
 __device__ __forceinline__ XB<R> xbasis(const Table &t, R x) {
   XB<R> X;
   const R x0 = sizeof(R) == 8 ? (R)t.x0 : (R)t.x0f, idx = sizeof(R) == 8 ? (R)t.idx : (R)t.idxf;
-  const R dx = sizeof(R) == 8 ? (R)t.dx : (R)t.dxf;
   const R gx = (x - x0) * idx;
   X.ok = gx >= R(0) && gx <= R(t.nx - 1);
   int i = X.ok ? (int)gx : 0;
   if (i > t.nx - 2) i = t.nx - 2;
   X.i = i;
-  quintic<R, 2>(gx - (R)i, X.h, X.d, X.e);
-  diff_basis<R>(X.h, R(1));
-  diff_basis<R>(X.d, R(0));
-  diff_basis<R>(X.e, R(0));
-  if (sizeof(R) == 8 && t.d) return X;   // cell units: the table's differences carry dx^p
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    X.h[a][1] *= dx; X.h[a][2] *= dx * dx;
-    X.d[a][0] *= idx; X.d[a][2] *= dx;
-    X.e[a][0] *= idx * idx; X.e[a][1] *= idx;
-  }
+  X.u = gx - (R)i;
   return X;
 }
 
-// The x-contracted values of one y-interval, in difference form along y:
-// g[m][r] = d^m/dx^m d^r/dy^r f at (x, y_j) and dg[m][r] the same at y_(j+1)
-// minus that at y_j (contracted from node differences), m < M.
-template <typename R, int M> struct YC {
-  int j;
-  R g[M][3], dg[M][3];
-};
-
-template <typename R, int M, int M0 = 0>
-__device__ __forceinline__ void contract(const Table &t, const XB<R> &X, int j, YC<R, M> &c) {
-  c.j = j;
-  const bool pre = sizeof(R) == 8 && t.d;   // the differences stored with the table
-  const long k0 = ((long)j * t.nx + X.i) * NQ, k1 = k0 + (long)t.nx * NQ;
-  const double *dc = pre ? t.d + ((long)j * (t.nx - 1) + X.i) * 4 * NQ : nullptr;
-  R q[2][2][NQ];   // [b][a][slot]; with pre: [0][0] D00, [0][1] D10, [1][0] D01, [1][1] D11
-#pragma unroll
-  for (int b = 0; b < 2; ++b)
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int s = 0; s < NQ; ++s) {
-        const long k = (b ? k1 : k0) + a * NQ + s;
-        q[b][a][s] = pre ? (R)dc[4 * s + 2 * b + a] : (sizeof(R) == 8 ? (R)t.v[k] : (R)t.vf[k]);
-      }
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    R g0 = R(0), g1 = R(0), g2 = R(0), d0 = R(0), d1 = R(0), d2 = R(0);
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-      const int sl = qslot(p, r);
-      const R D00 = q[0][0][sl];
-      const R D10 = pre ? q[0][1][sl] : q[0][1][sl] - q[0][0][sl];
-      const R D01 = pre ? q[1][0][sl] : q[1][0][sl] - q[0][0][sl];
-      const R D11 = pre ? q[1][1][sl] : (q[1][1][sl] - q[0][1][sl]) - (q[1][0][sl] - q[0][0][sl]);
-      if (M0 == 0) {
-        g0 += D00 * X.h[0][p] + D10 * X.h[1][p];
-        d0 += D01 * X.h[0][p] + D11 * X.h[1][p];
-      }
-      if (M > 1) {
-        g1 += D00 * X.d[0][p] + D10 * X.d[1][p];
-        d1 += D01 * X.d[0][p] + D11 * X.d[1][p];
-      }
-      if (M > 2) {
-        g2 += D00 * X.e[0][p] + D10 * X.e[1][p];
-        d2 += D01 * X.e[0][p] + D11 * X.e[1][p];
-      }
+// Value, first and half the second derivative (D = 0, 1, 2 selects how many)
+// of the polynomial sum_k q[k] w^k by synthetic division.
+template <typename R, int D>
+__device__ __forceinline__ void horner5(const R *q, R w, R &h, R &d, R &e) {
+  const R h4 = fma(q[5], w, q[4]), h3 = fma(h4, w, q[3]), h2 = fma(h3, w, q[2]), h1 = fma(h2, w, q[1]);
+  h = fma(h1, w, q[0]);
+  if (D >= 1) {
+    const R d3 = fma(q[5], w, h4), d2 = fma(d3, w, h3), d1 = fma(d2, w, h2);
+    d = fma(d1, w, h1);
+    if (D >= 2) {
+      const R e2 = fma(q[5], w, d3), e1 = fma(e2, w, d2);
+      e = fma(e1, w, d1);
     }
-    if (M0 == 0) { c.g[0][r] = g0; c.dg[0][r] = d0; }
-    if (M > 1) { c.g[1][r] = g1; c.dg[1][r] = d1; }
-    if (M > 2) { c.g[2][r] = g2; c.dg[2][r] = d2; }
   }
 }
 
-// The full contraction of interval j, reusing the values of a Newton
-// iteration's contraction c1 when it holds the same interval.
+// The six coefficients of u^0 .. u^5 of row r (power of v) of a table cell.
 template <typename R>
-__device__ __forceinline__ void contract_full(const Table &t, const XB<R> &X, int j, const YC<R, 1> *c1, YC<R, 3> &c) {
-  if (c1 && c1->j == j) {
+__device__ __forceinline__ void cell_row(const Table &t, long cell, int r, R *q) {
+  if constexpr (sizeof(R) == 8) {   // 16-byte loads: a row is 48 bytes, a cell 288
+    const double2 *p = reinterpret_cast<const double2 *>(t.c + cell * NCF) + 3 * r;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) { c.g[0][r] = c1->g[0][r]; c.dg[0][r] = c1->dg[0][r]; }
-    contract<R, 3, 1>(t, X, j, c);
+    for (int k = 0; k < 3; ++k) { const double2 w = __ldg(p + k); q[2 * k] = w.x; q[2 * k + 1] = w.y; }
   } else {
-    contract<R, 3>(t, X, j, c);
+    const float2 *p = reinterpret_cast<const float2 *>(t.cf + cell * NCF) + 3 * r;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { const float2 w = __ldg(p + k); q[2 * k] = w.x; q[2 * k + 1] = w.y; }
   }
+}
+
+// f at fixed x on y-interval j as a polynomial in v, for the iterations that
+// stay in one interval.
+template <typename R> struct YC {
+  int j;
+  R a[NC1];
+};
+
+template <typename R>
+__device__ __forceinline__ void contract(const Table &t, const XB<R> &X, int j, YC<R> &o) {
+  o.j = j;
+  const long cell = (long)j * (t.nx - 1) + X.i;
+#pragma unroll
+  for (int r = 0; r < NC1; ++r) {
+    R q[NC1], d, e;
+    cell_row<R>(t, cell, r, q);
+    horner5<R, 0>(q, X.u, o.a[r], d, e);
+  }
+}
+
+// f, f_y, f_yy / 2, f_x, f_xy, f_xx / 2 (in cell units) at (u, v): the rows
+// from the highest power of v down, each folded into the synthetic divisions
+// in v as it is formed, so no row is kept.
+template <typename R> struct TV { R f, fy, fyy, fx, fxy, fxx; };
+
+template <typename R>
+__device__ __forceinline__ void cell_eval(const Table &t, int i, int j, R u, R v, TV<R> &o) {
+  const long cell = (long)j * (t.nx - 1) + i;
+  R h = R(0), d = R(0), e = R(0), bh = R(0), bd = R(0), ch = R(0);
+#pragma unroll
+  for (int r = NC1 - 1; r >= 0; --r) {
+    R q[NC1], a0, a1, a2;
+    cell_row<R>(t, cell, r, q);
+    horner5<R, 2>(q, u, a0, a1, a2);
+    if (r == NC1 - 1) { h = a0; bh = a1; ch = a2; continue; }
+    if (r < NC1 - 3) e = fma(e, v, d);
+    else if (r == NC1 - 3) e = d;
+    if (r < NC1 - 2) { d = fma(d, v, h); bd = fma(bd, v, bh); }
+    else { d = h; bd = bh; }
+    h = fma(h, v, a0);
+    bh = fma(bh, v, a1);
+    ch = fma(ch, v, a2);
+  }
+  o.f = h; o.fy = d; o.fyy = e; o.fx = bh; o.fxy = bd; o.fxx = ch;
 }
 
 // Interval index of y and its fraction; false outside the table.
@@ -225,154 +191,117 @@ __device__ __forceinline__ bool yloc(const Table &t, R y, int &j, R &v) {
   return true;
 }
 
-// f, f_y, f_yy (M = 1) and also f_x, f_xy (M >= 2), f_xx (M = 3) at fraction
-// v of the interval the contraction holds.
-template <typename R, int M>
-__device__ __forceinline__ void yeval(const Table &t, const YC<R, M> &c, R v, TV<R> &o) {
-  const R dy = sizeof(R) == 8 ? (R)t.dy : (R)t.dyf, idy = sizeof(R) == 8 ? (R)t.idy : (R)t.idyf;
-  const bool pre = sizeof(R) == 8 && t.d;   // cell units: scale the results once
-  R h[2][3], d[2][3], e[2][3];
-  quintic<R, 2>(v, h, d, e);
-  diff_basis<R>(h, R(1));
-  diff_basis<R>(d, R(0));
-  diff_basis<R>(e, R(0));
-  R a0 = 0, a1 = 0, a2 = 0, b0 = 0, b1 = 0, c0 = 0;
-#pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    const R sh[3] = {h[b][0], pre ? h[b][1] : h[b][1] * dy, pre ? h[b][2] : h[b][2] * dy * dy};
-    const R sd[3] = {pre ? d[b][0] : d[b][0] * idy, d[b][1], pre ? d[b][2] : d[b][2] * dy};
-    const R se[3] = {pre ? e[b][0] : e[b][0] * idy * idy, pre ? e[b][1] : e[b][1] * idy, e[b][2]};
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const R g0 = b ? c.dg[0][r] : c.g[0][r];
-      a0 += g0 * sh[r];
-      a1 += g0 * sd[r];
-      a2 += g0 * se[r];
-      if (M > 1) {
-        const R g1 = b ? c.dg[1][r] : c.g[1][r];
-        b0 += g1 * sh[r];
-        b1 += g1 * sd[r];
-      }
-      if (M > 2) c0 += (b ? c.dg[2][r] : c.g[2][r]) * sh[r];
-    }
-  }
-  if (pre) {
-    o.f = a0; o.fy = a1 * R(t.idy); o.fyy = a2 * R(t.idy2);
-    o.fx = b0 * R(t.idx); o.fxy = b1 * R(t.idxdy); o.fxx = c0 * R(t.idx2);
-  } else {
-    o.f = a0; o.fy = a1; o.fyy = a2;
-    o.fx = b0; o.fxy = b1; o.fxx = c0;
-  }
-}
+// icv: 1/c_v; er: de/drho at fixed T (the next inversion's first guess,
+// eos_invert_rec)
+template <typename R> struct EosOut { R P, e, icv, PT, ge, gc, er; };
 
-// Biquintic evaluation of f and its derivatives up to second order at
-// (x, y = ln T) given the x-part.
+// Full EOS at (rho, T): P, e, P_T, 1/c_v, de/drho|_T, c_s^2; each quantity
+// shared between them formed once.
+template <typename R> struct EosC { R P, e, PT, icv, er, cs2, iT; };
+
 template <typename R>
-__device__ __forceinline__ bool table_eval_xb(const Table &t, const XB<R> &X, R y, TV<R> &o,
-                                              const YC<R, 1> *c1 = nullptr) {
+__device__ __forceinline__ bool eos_rt_c(const Table &t, const XB<R> &X, R rho, R irho, R T, R lnT, R iT, R iab,
+                                         EosC<R> &o) {
   int j;
   R v;
-  if (!(X.ok && yloc<R>(t, y, j, v))) return false;
-  YC<R, 3> c;
-  contract_full<R>(t, X, j, c1, c);
-  yeval<R, 3>(t, c, v, o);
-  return true;
-}
-
-template <typename R>
-__device__ __forceinline__ bool table_eval(const Table &t, R x, R y, TV<R> &o) {
-  return table_eval_xb<R>(t, xbasis<R>(t, x), y, o);
-}
-
-// er: de/drho at fixed T (the next inversion's first guess, eos_invert_pred)
-template <typename R> struct EosOut { R P, e, cv, Pr, PT, ge, gc, er; };
-
-// Full EOS at (rho, T) for a mixture with mean mass number abar and Y_e
-// (irho = 1/rho and iab = 1/abar: fixed during an inversion, formed once).
-template <typename R>
-__device__ __forceinline__ bool eos_rt_xy(const Table &t, const XB<R> &X, R rho, R irho, R T, R lnT, R iab,
-                                          EosOut<R> &o, const YC<R, 1> *c1 = nullptr) {
+  if (!(X.ok && yloc<R>(t, lnT, j, v))) return false;
   TV<R> q;
-  if (!table_eval_xb<R>(t, X, lnT, q, c1)) return false;
-  const R iT = R(1) / T;
-  const R Pe = q.fx - q.f;
-  const R ee = (q.f - q.fy) * irho;
-  const R cve = (q.fy - q.fyy) * irho * iT;
-  const R PeT = (q.fxy - q.fy) * iT;
-  const R Per = (q.fxx - q.fx) * irho;
-  const R Rg = R(RGAS);
+  cell_eval<R>(t, X.i, j, X.u, v, q);
+  constexpr bool dbl = sizeof(R) == 8;
+  const R idx = dbl ? (R)t.idx : (R)t.idxf, idy = dbl ? (R)t.idy : (R)t.idyf;
+  const R idxdy = dbl ? (R)t.idxdy : (R)t.idxdyf;
+  const R idx2 = dbl ? (R)t.idx2x2 : (R)t.idx2x2f, idy2 = dbl ? (R)t.idy2x2 : (R)t.idy2x2f;
+  const R f = q.f, fy = q.fy * idy, fx = q.fx * idx;
   R aT4, aT3;   // radiation a T^4 and a T^3
-  if (sizeof(R) == 8) {
-    const R T3 = T * T * T;
-    aT3 = R(ARAD) * T3;
+  if (dbl) {
+    aT3 = (R(ARAD) * T) * (T * T);
     aT4 = aT3 * T;
   } else {   // T^4 overflows FP32 above 2^32 K: form (a^(1/4) T)^4 instead
-    const R t = R(ARAD_QUARTER) * T, t2 = t * t;
+    const R tt = R(ARAD_QUARTER) * T, t2 = tt * tt;
     aT4 = t2 * t2;
     aT3 = aT4 * iT;
   }
-  o.P = Pe + rho * Rg * T * iab + aT4 / R(3);
-  o.e = ee + R(1.5) * Rg * T * iab + aT4 * irho;
-  // d/drho = (1/rho) d/dx at fixed T: ((f_x - f_xy) - (f - f_y)) / rho^2 and -a T^4 / rho^2
-  o.er = ((q.fx - q.fxy) - (q.f - q.fy) - aT4) * irho * irho;
-  o.cv = cve + R(1.5) * Rg * iab + R(4) * aT3 * irho;
-  o.PT = PeT + rho * Rg * iab + R(4) / R(3) * aT3;
-  o.Pr = Per + Rg * T * iab;
-  // auxiliary indices of Sect. 2.6: gamma_e = P / (rho e) + 1, gamma_c = rho c_s^2 / P;
+  const R Ra = R(RGAS) * iab, RT = Ra * T;
+  const R w = (f - fy) + aT4;                    // rho e without the ions
+  o.P = fma(aT4, R(1.0 / 3.0), fma(rho, RT, fx - f));
+  o.e = fma(w, irho, R(1.5) * RT);
+  // d/drho = (1/rho) d/dx at fixed T
+  const R ir2 = irho * irho;
+  o.er = (fma(-q.fxy, idxdy, fx) - w) * ir2;
+  const R cv = fma(fma(fma(-q.fyy, idy2, fy), iT, R(4) * aT3), irho, R(1.5) * Ra);
+  o.icv = rcp_nr(cv);
+  o.PT = fma(fma(q.fxy, idxdy, -fy), iT, fma(rho, Ra, R(4.0 / 3.0) * aT3));
+  const R Pr = fma(fma(q.fxx, idx2, -fx), irho, RT);
   // c_s^2 = P_rho + T P_T^2 / (rho^2 c_v), grouped so no product leaves the FP32 range
-  const R cs2 = o.Pr + (T * o.PT * irho) * (o.PT * irho / o.cv);
-  o.ge = o.P / (rho * o.e) + R(1);
-  o.gc = rho * cs2 / o.P;
+  const R pr = o.PT * irho;
+  o.cs2 = fma((T * pr) * o.icv, pr, Pr);
+  o.iT = iT;
+  return true;
+}
+
+// auxiliary indices of Sect. 2.6: gamma_e = P / (rho e) + 1, gamma_c = rho c_s^2 / P
+template <typename R>
+__device__ __forceinline__ void gammas(R rho, R P, R e, R cs2, R &ge, R &gc) {
+  if (sizeof(R) == 8) {   // one reciprocal for both
+    const R re = rho * e, inv = rcp_nr(P * re);   // 1/(rho e) = P inv, 1/P = rho e inv
+    ge = fma(P, P * inv, R(1));
+    gc = rho * cs2 * (re * inv);
+  } else {                // P rho e would leave the FP32 range
+    ge = P / (rho * e) + R(1);
+    gc = rho * cs2 / P;
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ bool eos_rt_xy(const Table &t, const XB<R> &X, R rho, R irho, R T, R lnT, R iT, R iab,
+                                          EosOut<R> &o) {
+  EosC<R> f;
+  if (!eos_rt_c<R>(t, X, rho, irho, T, lnT, iT, iab, f)) return false;
+  o.P = f.P; o.e = f.e; o.icv = f.icv; o.PT = f.PT; o.er = f.er;
+  gammas<R>(rho, f.P, f.e, f.cs2, o.ge, o.gc);
   return true;
 }
 
 template <typename R>
 __device__ __forceinline__ bool eos_rt(const Table &t, R rho, R T, R abar, R ye, EosOut<R> &o) {
-  return eos_rt_xy<R>(t, xbasis<R>(t, log(rho * ye * R(NAV))), rho, R(1) / rho, T, log(T), R(1) / abar, o);
+  return eos_rt_xy<R>(t, xbasis<R>(t, log(rho * ye * R(NAV))), rho, rcp_nr(rho), T, log(T), rcp_nr(T), rcp_nr(abar), o);
 }
 
 // Specific internal energy and c_v at (rho, T): what a Newton iteration needs.
 // c holds the x-contraction of the current table interval and is redone when
 // T has left it.
 template <typename R>
-__device__ __forceinline__ bool eos_ecv_xy(const Table &t, const XB<R> &X, YC<R, 1> &c, R irho, R T, R lnT, R iab,
-                                           R &e, R &cv) {
+__device__ __forceinline__ bool eos_ecv_xy(const Table &t, const XB<R> &X, YC<R> &c, R irho, R T, R lnT, R iT,
+                                           R iab, R &e, R &cv) {
   int j;
   R v;
   if (!(X.ok && yloc<R>(t, lnT, j, v))) return false;
-  if (j != c.j) contract<R, 1>(t, X, j, c);
-  TV<R> q;
-  yeval<R, 1>(t, c, v, q);
-  const R iT = R(1) / T;
-  const R Rg = R(RGAS);
+  if (j != c.j) contract<R>(t, X, j, c);
+  const R idy = sizeof(R) == 8 ? (R)t.idy : (R)t.idyf, idy2 = sizeof(R) == 8 ? (R)t.idy2x2 : (R)t.idy2x2f;
+  R f, a1, a2;
+  horner5<R, 2>(c.a, v, f, a1, a2);
+  const R fy = a1 * idy;
   R aT4, aT3;
   if (sizeof(R) == 8) {
-    aT3 = R(ARAD) * T * T * T;
+    aT3 = (R(ARAD) * T) * (T * T);
     aT4 = aT3 * T;
   } else {
     const R tt = R(ARAD_QUARTER) * T, t2 = tt * tt;
     aT4 = t2 * t2;
     aT3 = aT4 * iT;
   }
-  e = (q.f - q.fy) * irho + R(1.5) * Rg * T * iab + aT4 * irho;
-  cv = (q.fy - q.fyy) * irho * iT + R(1.5) * Rg * iab + R(4) * aT3 * irho;
+  const R Ra = R(1.5) * R(RGAS) * iab;
+  e = fma((f - fy) + aT4, irho, Ra * T);
+  cv = fma(fma(fma(-a2, idy2, fy), iT, R(4) * aT3), irho, Ra);
   return true;
 }
 
-template <typename R>
-__device__ __forceinline__ bool eos_ecv(const Table &t, R rho, R T, R abar, R ye, R &e, R &cv) {
-  YC<R, 1> c;
-  c.j = -1;
-  return eos_ecv_xy<R>(t, xbasis<R>(t, log(rho * ye * R(NAV))), c, R(1) / rho, T, log(T), R(1) / abar, e, cv);
-}
-
-// ln Tn from ln T for a Newton step T -> Tn: with d = (Tn - T) / T below
+// ln Tn from ln T for a Newton step T -> Tn with d = (Tn - T) / T: below
 // 2^-10, ln(1 + d) by its Taylor series to d^4 (truncation below d^5 / 5 <
 // 2e-16, under the rounding of ln T ~ 16..23); otherwise the logarithm.
 // Saves an FP64 logarithm per step once the iteration is close.
 template <typename R>
-__device__ __forceinline__ R next_lnT(R T, R lnT, R Tn) {
-  const R d = (Tn - T) / T;
+__device__ __forceinline__ R next_lnT(R d, R lnT, R Tn) {
   if (!(fabs(d) < R(1.0 / 1024.0))) return log(Tn);
   return lnT + d * (R(1) - d * (R(0.5) - d * (R(1.0 / 3.0) - d * R(0.25))));
 }
@@ -382,55 +311,58 @@ __device__ __forceinline__ R next_lnT(R T, R lnT, R Tn) {
 // The iterations evaluate only e and c_v; the full EOS (P, gamma_e, gamma_c)
 // is evaluated once, at the final T.  Returns the iteration count or -1.
 template <typename R>
-__device__ __forceinline__ int newton_loop(const Table &t, const XB<R> &X, YC<R, 1> &c, R rho, R irho, R eint, R iab,
+__device__ __forceinline__ int newton_loop(const Table &t, const XB<R> &X, YC<R> &c, R rho, R irho, R eint, R iab,
                                            R &T, R tol, int maxit, EosOut<R> &o, bool have, R e0, R cv0, R lnT0) {
   const R Tlo = sizeof(R) == 8 ? (R)t.Tlo : (R)t.Tlof, Thi = sizeof(R) == 8 ? (R)t.Thi : (R)t.Thif;
   R lo = Tlo, hi = Thi;
   if (!(T > Tlo && T < Thi)) { T = sqrt(Tlo * Thi); have = false; }
   R lnT = have ? lnT0 : log(T);   // e0, cv0 were evaluated at (T, lnT0), c may hold its interval
   for (int it = 1; it <= maxit; ++it) {
+    const R iT = rcp_nr(T);
     R e = e0, cv = cv0;   // the first iteration may come evaluated
-    if (!(have && it == 1) && !eos_ecv_xy<R>(t, X, c, irho, T, lnT, iab, e, cv)) return -1;
+    if (!(have && it == 1) && !eos_ecv_xy<R>(t, X, c, irho, T, lnT, iT, iab, e, cv)) return -1;
     const R de = eint - e;
+    const R step = de * rcp_nr(cv);
     if (fabs(de) < tol * fabs(eint)) {
-      const R Tn = T + de / cv;
-      lnT = next_lnT<R>(T, lnT, Tn);
+      const R Tn = T + step;
+      lnT = next_lnT<R>(step * iT, lnT, Tn);
       T = Tn;
-      if (!eos_rt_xy<R>(t, X, rho, irho, T, lnT, iab, o, &c)) return -1;
+      if (!eos_rt_xy<R>(t, X, rho, irho, T, lnT, rcp_nr(T), iab, o)) return -1;
       return it;
     }
     if (de > R(0)) lo = T; else hi = T;
-    R Tn = T + de / cv;
+    R Tn = T + step;
     if (!(Tn > lo && Tn < hi)) Tn = R(0.5) * (lo + hi);
-    lnT = next_lnT<R>(T, lnT, Tn);
+    lnT = next_lnT<R>((Tn - T) * iT, lnT, Tn);
     T = Tn;
   }
   return -1;
 }
 
+// iab = 1/Abar
 template <typename R>
-__device__ __forceinline__ int eos_invert(const Table &t, R rho, R eint, R abar, R ye, R &T, R tol, int maxit,
+__device__ __forceinline__ int eos_invert(const Table &t, R rho, R irho, R eint, R iab, R ye, R &T, R tol, int maxit,
                                           EosOut<R> &o) {
   const XB<R> X = xbasis<R>(t, log(rho * ye * R(NAV)));   // rho and Y_e fixed
-  YC<R, 1> c;
+  YC<R> c;
   c.j = -1;
-  return newton_loop<R>(t, X, c, rho, R(1) / rho, eint, R(1) / abar, T, tol, maxit, o, false, R(0), R(0), R(0));
+  return newton_loop<R>(t, X, c, rho, irho, eint, iab, T, tol, maxit, o, false, R(0), R(0), R(0));
 }
 
 // The FP32 phase of the mixed inversion: Newton on e and c_v only, until
 // |de|/e < tol or maxit; T keeps the last bracketed iterate.
-__device__ __forceinline__ int newton_fp32(const Table &t, float rho, float eint, float abar, float ye, float &T,
+__device__ __forceinline__ int newton_fp32(const Table &t, float rho, float eint, float iab, float ye, float &T,
                                            float tol, int maxit) {
   const float Tlo = t.Tlof, Thi = t.Thif;
   float lo = Tlo, hi = Thi;
   if (!(T > Tlo && T < Thi)) T = sqrtf(Tlo * Thi);
   const XB<float> X = xbasis<float>(t, logf(rho * ye * float(NAV)));
-  const float irho = 1.0f / rho, iab = 1.0f / abar;
-  YC<float, 1> c;
+  const float irho = 1.0f / rho;
+  YC<float> c;
   c.j = -1;
   for (int it = 1; it <= maxit; ++it) {
     float e, cv;
-    if (!eos_ecv_xy<float>(t, X, c, irho, T, logf(T), iab, e, cv)) return -1;
+    if (!eos_ecv_xy<float>(t, X, c, irho, T, logf(T), 1.0f / T, iab, e, cv)) return -1;
     const float de = eint - e;
     if (de > 0.0f) lo = T; else hi = T;
     float Tn = T + de / cv;
@@ -448,20 +380,19 @@ __device__ __forceinline__ int newton_fp32(const Table &t, float rho, float eint
 // step, the full evaluation at the final T).  The low-Mach deviations need
 // P to ~1e-12, so a single FP64 step from 1e-5 is not enough.  Returns the
 // total iteration count, or -1 if the FP64 phase fails.
-__device__ __forceinline__ int eos_invert_mixed(const Table &t, double rho, double eint, double abar, double ye,
-                                                double &T, double tol, int maxit, EosOut<double> &o) {
+__device__ __forceinline__ int eos_invert_mixed(const Table &t, double rho, double irho, double eint, double iab,
+                                                double ye, double &T, double tol, int maxit, EosOut<double> &o) {
   // a first guess already within 1e-4 of the root (the previous step's T in
   // a time step) goes straight to the FP64 iteration: the FP32 phase could
   // only degrade it to FP32's ~1e-6
   const XB<double> X = xbasis<double>(t, log(rho * ye * NAV));
-  const double irho = 1.0 / rho, iab = 1.0 / abar;
-  YC<double, 1> c;
+  YC<double> c;
   c.j = -1;
   {
     double e, cv;
     if (T > t.Tlo && T < t.Thi) {
-      const double lnT = log(T);
-      if (eos_ecv_xy<double>(t, X, c, irho, T, lnT, iab, e, cv) && fabs(eint - e) < 1e-4 * fabs(eint)) {
+      const double lnT = log(T), iT = rcp_nr(T);
+      if (eos_ecv_xy<double>(t, X, c, irho, T, lnT, iT, iab, e, cv) && fabs(eint - e) < 1e-4 * fabs(eint)) {
         const double de = eint - e;
         // From |de|/e < 2e-6 one Newton step lands within ~(de/e)^2 < 1e-11
         // of the root (quadratic convergence; d ln e / d ln T is 1..4 here):
@@ -472,13 +403,18 @@ __device__ __forceinline__ int eos_invert_mixed(const Table &t, double rho, doub
         // only).  The plain iteration would evaluate e, c_v at T1 once more
         // and then the full EOS at T1 + dT.
         if (fabs(de) >= tol * fabs(eint) && fabs(de) < 2e-6 * fabs(eint)) {
-          const double T1 = T + de / cv;
+          const double step = de * rcp_nr(cv), T1 = T + step;
           if (T1 > t.Tlo && T1 < t.Thi) {
-            if (!eos_rt_xy<double>(t, X, rho, irho, T1, next_lnT<double>(T, lnT, T1), iab, o, &c)) return -1;
-            const double dT = (eint - o.e) / o.cv;
-            o.P = fma(o.PT, dT, o.P);
+            EosC<double> f;
+            if (!eos_rt_c<double>(t, X, rho, irho, T1, next_lnT<double>(step * iT, lnT, T1), rcp_nr(T1), iab, f))
+              return -1;
+            const double dT = (eint - f.e) * f.icv;
+            o.P = fma(f.PT, dT, f.P);
             o.e = eint;
-            o.ge = o.P / (rho * eint) + 1.0;
+            o.icv = f.icv; o.PT = f.PT; o.er = f.er;
+            double ge1;   // gamma_c from the pressure at T1, gamma_e from the carried one
+            gammas<double>(rho, f.P, f.e, f.cs2, ge1, o.gc);
+            o.ge = o.P * rcp_nr(rho * eint) + 1.0;
             T = T1 + dT;
             return 2;
           }
@@ -488,7 +424,7 @@ __device__ __forceinline__ int eos_invert_mixed(const Table &t, double rho, doub
     }
   }
   float Tf = (float)T;
-  const int it32 = newton_fp32(t, (float)rho, (float)eint, (float)abar, (float)ye, Tf, 1e-5f, maxit < 12 ? maxit : 12);
+  const int it32 = newton_fp32(t, (float)rho, (float)eint, (float)iab, (float)ye, Tf, 1e-5f, maxit < 12 ? maxit : 12);
   if (isfinite(Tf) && Tf > 0.0f) T = (double)Tf;
   const int it64 = newton_loop<double>(t, X, c, rho, irho, eint, iab, T, tol, maxit, o, false, 0.0, 0.0, 0.0);
   return it64 < 0 ? -1 : it64 + (it32 > 0 ? it32 : 12);
@@ -515,45 +451,19 @@ __device__ __forceinline__ double ln_step(double lnp, double d, double fallback_
   return lnp + d * (1.0 - d * (0.5 - d * (1.0 / 3.0 - d * 0.25)));
 }
 
-// The full EOS at (rho, T) for the recorded mixed inversion: P, e, P_T,
-// 1/c_v, de/drho|_T, c_s^2 and 1/T, the reciprocals formed once (gamma_e and
-// gamma_c follow from the carried P in rec_carry).
-struct EosC {
-  double P, e, PT, icv, er, cs2, iT;
-};
-__device__ __forceinline__ bool eos_rt_c(const Table &t, const XB<double> &X, double rho, double irho, double T,
-                                         double lnT, double iT, double iab, EosC &o, const YC<double, 1> *c1) {
-  TV<double> q;
-  if (!table_eval_xb<double>(t, X, lnT, q, c1)) return false;
-  const double Rg = RGAS;
-  const double aT3 = ARAD * T * T * T, aT4 = aT3 * T;
-  o.P = (q.fx - q.f) + rho * Rg * T * iab + aT4 * (1.0 / 3.0);
-  o.e = (q.f - q.fy) * irho + 1.5 * Rg * T * iab + aT4 * irho;
-  o.icv = 1.0 / ((q.fy - q.fyy) * irho * iT + 1.5 * Rg * iab + 4.0 * aT3 * irho);
-  o.PT = (q.fxy - q.fy) * iT + rho * Rg * iab + (4.0 / 3.0) * aT3;
-  const double Pr = (q.fxx - q.fx) * irho + Rg * T * iab;
-  o.cs2 = Pr + (T * o.PT * irho) * (o.PT * irho * o.icv);
-  o.er = ((q.fx - q.fxy) - (q.f - q.fy) - aT4) * irho * irho;
-  o.iT = iT;
-  return true;
-}
-
 // The carry of a full evaluation c at T1 (within ~2e-6 of the root in e) to
 // the root T1 + dT, dT = (e - e(T1)) / c_v, to first order: P + P_T dT;
 // gamma_e = P / (rho e) + 1 from that P and e; gamma_c = rho c_s^2 / P
 // (c_s^2 at T1: relative error ~dT/T, wave speeds only); one reciprocal for
 // both.  Writes the record of the inversion.
 __device__ __forceinline__ void rec_carry(double rho, double eint, double ine, double x, double T1, double lnT1,
-                                          const EosC &c, EosOut<double> &o, double &T, Pred &pr) {
+                                          const EosC<double> &c, EosOut<double> &o, double &T, Pred &pr) {
   const double dT = (eint - c.e) * c.icv;
-  const double P = fma(c.PT, dT, c.P);
-  const double re = rho * eint;
-  const double inv = 1.0 / (P * re);   // 1/(rho e) = P inv, 1/P = rho e inv
-  o.P = P;
+  o.P = fma(c.PT, dT, c.P);
   o.e = eint;
-  o.ge = P * (P * inv) + 1.0;
-  o.gc = rho * c.cs2 * (re * inv);
-  o.cv = 0.0;   // not formed on this path
+  gammas<double>(rho, o.P, eint, c.cs2, o.ge, o.gc);
+  o.icv = c.icv;
+  o.PT = c.PT;
   o.er = c.er;
   T = T1 + dT;
   const double dd = dT * c.iT;
@@ -572,24 +482,22 @@ __device__ __forceinline__ void rec_carry(double rho, double eint, double ine, d
 // loop; else FP32 iterations first.  irho = 1/rho and iab = 1/Abar come
 // with the arguments.  Writes the record; returns the count of evaluations
 // at distinct temperatures (1 for the recorded path) or -1.
-__device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double irho, double eint, double abar,
-                                              double iab, double ye, double &T, double tol, int maxit,
-                                              EosOut<double> &o, Pred &pr, bool rec) {
+__device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double irho, double eint, double iab,
+                                              double ye, double &T, double tol, int maxit, EosOut<double> &o, Pred &pr,
+                                              bool rec) {
   const double ne = rho * ye;
   rec = rec && pr.ine > 0.0;
-  const double dn = rec ? ne * pr.ine - 1.0 : 0.0;   // n_e = n_e,p (1 + dn)
+  const double dn = rec ? fma(ne, pr.ine, -1.0) : 0.0;   // n_e = n_e,p (1 + dn)
   const double x = rec ? ln_step(pr.x, dn, ne * NAV) : log(ne * NAV);
-  const double ine = rec ? inv_step(pr.ine, dn, ne) : 1.0 / ne;
+  const double ine = rec ? inv_step(pr.ine, dn, ne) : rcp_nr(ne);
   const XB<double> X = xbasis<double>(t, x);
-  YC<double, 1> c;
-  c.j = -1;
-  EosC f;
+  EosC<double> f;
   if (rec && pr.icv > 0.0 && T > t.Tlo && T < t.Thi) {
     const double T1 = T + (eint - pr.e - pr.er * (rho - pr.rho)) * pr.icv;
     if (T1 > t.Tlo && T1 < t.Thi) {
       const double dT = (T1 - T) * pr.iT;   // T1 = T (1 + dT)
       const double lnT1 = ln_step(pr.lnT, dT, T1);
-      if (!eos_rt_c(t, X, rho, irho, T1, lnT1, inv_step(pr.iT, dT, T1), iab, f, nullptr)) return -1;
+      if (!eos_rt_c<double>(t, X, rho, irho, T1, lnT1, inv_step(pr.iT, dT, T1), iab, f)) return -1;
       if (fabs(eint - f.e) < 2e-6 * fabs(eint)) {
         rec_carry(rho, eint, ine, x, T1, lnT1, f, o, T, pr);
         return 1;
@@ -597,17 +505,19 @@ __device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double
       T = T1;   // a larger change: the steps below from T1
     }
   }
+  YC<double> c;
+  c.j = -1;
   int it0 = -2;   // -2: a far guess, FP32 iterations first
   if (T > t.Tlo && T < t.Thi) {
-    const double lnT = log(T);
+    const double lnT = log(T), iT = rcp_nr(T);
     double e, cv;
-    if (eos_ecv_xy<double>(t, X, c, irho, T, lnT, iab, e, cv) && fabs(eint - e) < 1e-4 * fabs(eint)) {
+    if (eos_ecv_xy<double>(t, X, c, irho, T, lnT, iT, iab, e, cv) && fabs(eint - e) < 1e-4 * fabs(eint)) {
       const double de = eint - e;
       if (fabs(de) < 2e-6 * fabs(eint)) {
-        const double T1 = T + de / cv;
+        const double step = de * rcp_nr(cv), T1 = T + step;
         if (T1 > t.Tlo && T1 < t.Thi) {
-          const double lnT1 = next_lnT<double>(T, lnT, T1);
-          if (!eos_rt_c(t, X, rho, irho, T1, lnT1, 1.0 / T1, iab, f, &c)) return -1;
+          const double lnT1 = next_lnT<double>(step * iT, lnT, T1);
+          if (!eos_rt_c<double>(t, X, rho, irho, T1, lnT1, rcp_nr(T1), iab, f)) return -1;
           rec_carry(rho, eint, ine, x, T1, lnT1, f, o, T, pr);
           return 2;
         }
@@ -617,13 +527,13 @@ __device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double
   }
   if (it0 == -2) {
     float Tf = (float)T;
-    const int it32 = newton_fp32(t, (float)rho, (float)eint, (float)abar, (float)ye, Tf, 1e-5f, maxit < 12 ? maxit : 12);
+    const int it32 = newton_fp32(t, (float)rho, (float)eint, (float)iab, (float)ye, Tf, 1e-5f, maxit < 12 ? maxit : 12);
     if (isfinite(Tf) && Tf > 0.0f) T = (double)Tf;
     const int it64 = newton_loop<double>(t, X, c, rho, irho, eint, iab, T, tol, maxit, o, false, 0.0, 0.0, 0.0);
     it0 = it64 < 0 ? -1 : it64 + (it32 > 0 ? it32 : 12);
   }
   if (it0 > 0)   // the record of a Newton-loop result (the rare paths)
-    pr = Pred{rho, eint, 1.0 / o.cv, o.er, log(T), 1.0 / T, x, ine};
+    pr = Pred{rho, eint, o.icv, o.er, log(T), rcp_nr(T), x, ine};
   return it0;
 }
 

@@ -12,32 +12,27 @@ namespace phl {
 using namespace stage;
 namespace {
 
-// Mean mass number and electron fraction of normalised mass fractions.
-template <typename R>
-__device__ __forceinline__ void mixture(const DevGeo &G, const R *X, R &abar, R &ye, R *iabar = nullptr) {
-  R sx = R(0), sa = R(0), sz = R(0);
+// 1/Abar and electron fraction of a cell's mass fractions or species
+// densities u (any common factor cancels); is: 1/sum(u).
+__device__ __forceinline__ void mixture(const DevGeo &G, const double *u, double &iabar, double &ye, double &is) {
+  double s = 0.0, sa = 0.0, sz = 0.0;
 #pragma unroll
   for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-    if (l < G.nspec) sx += X[l];
-  // 1/A and Z/A of each species are constants of the grid: two reciprocals
-  // per cell (GB300's FP64 divisions are a dozen FP64-pipe instructions)
-  const R isx = R(1) / sx;
-#pragma unroll
-  for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-    if (l < G.nspec) {
-      const R x = X[l] * isx;
-      sa += x * (R)G.iAcomp[l];
-      sz += x * (R)G.ZoAcomp[l];
+    if (l < G.nspec) {   // 1/A and Z/A of each species are constants of the grid
+      s += u[l];
+      sa = fma(u[l], G.iAcomp[l], sa);
+      sz = fma(u[l], G.ZoAcomp[l], sz);
     }
-  abar = R(1) / sa;
-  ye = sz;
-  if (iabar) *iabar = sa;
+  is = eos::rcp_nr(s);
+  iabar = sa * is;
+  ye = sz * is;
 }
 
-// Stage-input state of interior cell p: density, velocity, cell-centred B,
-// specific internal energy, mass fractions.
+// Stage-input state of interior cell p: density, velocity, twice the
+// cell-centred B (the sum of its faces), specific internal energy, species
+// densities.
 struct CellState {
-  double rho, irho, v[3], b[3], eint, X[PHL_NSPEC_MAX];
+  double rho, irho, v[3], b2[3], eint, rX[PHL_NSPEC_MAX];
 };
 __device__ __forceinline__ CellState cell_state(const DevGeo &G, long p, const double *__restrict__ U,
                                                 const double *__restrict__ Bf, const float *__restrict__ dU,
@@ -63,15 +58,17 @@ __device__ __forceinline__ CellState cell_state(const DevGeo &G, long p, const d
     bh[2] += f2d_scaled(dB[2 * pl + p + G.sz], k);
   }
   c.rho = u[0];
-  const double ir = 1.0 / c.rho;   // one reciprocal for the cell
+  const double ir = eos::rcp_nr(c.rho);   // one reciprocal for the cell
   c.irho = ir;
   c.v[0] = u[1] * ir; c.v[1] = u[2] * ir; c.v[2] = u[3] * ir;
-  c.b[0] = 0.5 * (bl[0] + bh[0]); c.b[1] = 0.5 * (bl[1] + bh[1]); c.b[2] = 0.5 * (bl[2] + bh[2]);
-  c.eint = u[4] * ir - 0.5 * (c.v[0] * c.v[0] + c.v[1] * c.v[1] + c.v[2] * c.v[2]) -
-           0.5 * (c.b[0] * c.b[0] + c.b[1] * c.b[1] + c.b[2] * c.b[2]) * ir;
+  c.b2[0] = bl[0] + bh[0]; c.b2[1] = bl[1] + bh[1]; c.b2[2] = bl[2] + bh[2];
+  // (E - m.u/2 - B^2/2) / rho with B = b2 / 2
+  const double mu = fma(u[3], c.v[2], fma(u[2], c.v[1], u[1] * c.v[0]));
+  const double bb = fma(c.b2[2], c.b2[2], fma(c.b2[1], c.b2[1], c.b2[0] * c.b2[0]));
+  c.eint = fma(-0.125, bb, fma(-0.5, mu, u[4])) * ir;
 #pragma unroll
   for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-    if (l < G.nspec) c.X[l] = u[5 + l] * ir;
+    if (l < G.nspec) c.rX[l] = u[5 + l];
   return c;
 }
 
@@ -96,7 +93,7 @@ __global__ void k_mlp_guess(DevGeo G, Box box, const double *__restrict__ U, con
   const bool ok_in = in && s.rho > 0.0 && s.eint > 0.0;
   const float lr = ok_in ? (float)log10(s.rho) : G.mlp.c[0];
   const float le = ok_in ? (float)log10(s.eint) : G.mlp.c[1];
-  const float x0 = ok_in ? (float)(s.X[0] / (s.X[0] + (G.nspec > 1 ? s.X[1] : 0.0))) : G.mlp.c[2];
+  const float x0 = ok_in ? (float)(s.rX[0] / (s.rX[0] + (G.nspec > 1 ? s.rX[1] : 0.0))) : G.mlp.c[2];
   const float lt = mlp::guess_log10T(G.mlp, lr, le, x0);
   if (in) Tg[p] = need ? exp10((double)lt) : T;
 }
@@ -120,12 +117,9 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
   const long p = sidx(G, c[0], c[1], c[2]);
   const CellState cs = cell_state(G, p, U, Bf, dU, dB);
   const double rho = cs.rho, eint = cs.eint;
-  const double vx = cs.v[0], vy = cs.v[1], vz = cs.v[2], bx = cs.b[0], by = cs.b[1], bz = cs.b[2];
-  double X[PHL_NSPEC_MAX];
-#pragma unroll
-  for (int l = 0; l < PHL_NSPEC_MAX; ++l) X[l] = cs.X[l];
-  double abar, ye, iab;
-  mixture<double>(G, X, abar, ye, &iab);
+  const double vx = cs.v[0], vy = cs.v[1], vz = cs.v[2];
+  double iab, ye, is;
+  mixture(G, cs.rX, iab, ye, is);
   double T = G.use_mlp ? Tout[p] : Tin[p];   // Tout holds the network's guesses (k_mlp_guess)
   eos::EosOut<double> o;
   int it;
@@ -134,18 +128,17 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     eos::Pred pr{};
     double *rp = G.pred + p;
     if (pm == 2) pr = eos::Pred{rp[0], rp[pl], rp[2 * pl], rp[3 * pl], rp[4 * pl], rp[5 * pl], rp[6 * pl], rp[7 * pl]};
-    it = eos::eos_invert_rec(G.tab, rho, cs.irho, eint, abar, iab, ye, T, G.newton_tol, G.newton_maxit, o, pr,
-                             pm == 2);
+    it = eos::eos_invert_rec(G.tab, rho, cs.irho, eint, iab, ye, T, G.newton_tol, G.newton_maxit, o, pr, pm == 2);
     rp[0] = pr.rho; rp[pl] = pr.e; rp[2 * pl] = pr.icv; rp[3 * pl] = pr.er;
     rp[4 * pl] = pr.lnT; rp[5 * pl] = pr.iT; rp[6 * pl] = pr.x; rp[7 * pl] = pr.ine;
   } else {
-    it = sizeof(R) == 8 ? eos::eos_invert<double>(G.tab, rho, eint, abar, ye, T, G.newton_tol, G.newton_maxit, o)
-                        : eos::eos_invert_mixed(G.tab, rho, eint, abar, ye, T, G.newton_tol, G.newton_maxit, o);
+    it = sizeof(R) == 8 ? eos::eos_invert<double>(G.tab, rho, cs.irho, eint, iab, ye, T, G.newton_tol, G.newton_maxit, o)
+                        : eos::eos_invert_mixed(G.tab, rho, cs.irho, eint, iab, ye, T, G.newton_tol, G.newton_maxit, o);
   }
   if (it < 0 && G.use_mlp) {   // the plain Newton from the previous temperature is the fallback
     T = Tin[p];
-    it = sizeof(R) == 8 ? eos::eos_invert<double>(G.tab, rho, eint, abar, ye, T, G.newton_tol, G.newton_maxit, o)
-                        : eos::eos_invert_mixed(G.tab, rho, eint, abar, ye, T, G.newton_tol, G.newton_maxit, o);
+    it = sizeof(R) == 8 ? eos::eos_invert<double>(G.tab, rho, cs.irho, eint, iab, ye, T, G.newton_tol, G.newton_maxit, o)
+                        : eos::eos_invert_mixed(G.tab, rho, cs.irho, eint, iab, ye, T, G.newton_tol, G.newton_maxit, o);
   }
   if (G.niter) {   // warp sum, one atomic per warp
     const unsigned m = __activemask();
@@ -164,15 +157,17 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     W[wix<R>(G, W_RHO, q)] = d2f_scaled(rho - b.rho, -G.e_rho);
     W[wix<R>(G, W_VX, q)] = d2f_scaled(vx, -ev); W[wix<R>(G, W_VY, q)] = d2f_scaled(vy, -ev);
     W[wix<R>(G, W_VZ, q)] = d2f_scaled(vz, -ev);
-    W[wix<R>(G, W_BX, q)] = d2f_scaled(bx, -G.e_b); W[wix<R>(G, W_BY, q)] = d2f_scaled(by, -G.e_b);
-    W[wix<R>(G, W_BZ, q)] = d2f_scaled(bz, -G.e_b);
+    const int eb = -G.e_b - 1;        // the field is half the sum of its faces
+    W[wix<R>(G, W_BX, q)] = d2f_scaled(cs.b2[0], eb); W[wix<R>(G, W_BY, q)] = d2f_scaled(cs.b2[1], eb);
+    W[wix<R>(G, W_BZ, q)] = d2f_scaled(cs.b2[2], eb);
     W[wix<R>(G, W_P, q)] = d2f_scaled(o.P - b.p, -G.e_e);
     W[wix<R>(G, W_GE, q)] = d2f_scaled(o.ge - b.ge, 0);
     W[wix<R>(G, W_GC, q)] = d2f_scaled(o.gc - b.gc, 0);
 #pragma unroll
     for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-      if (l < G.nspec) W[wix<R>(G, W_X0 + l, q)] = d2f_scaled(X[l], 0);
+      if (l < G.nspec) W[wix<R>(G, W_X0 + l, q)] = d2f_scaled(cs.rX[l] * cs.irho, 0);
   } else {
+    const double bx = 0.5 * cs.b2[0], by = 0.5 * cs.b2[1], bz = 0.5 * cs.b2[2];
     W[wix<R>(G, W_RHO, q)] = rho - b.rho;
     W[wix<R>(G, W_VX, q)] = vx; W[wix<R>(G, W_VY, q)] = vy; W[wix<R>(G, W_VZ, q)] = vz;
     W[wix<R>(G, W_BX, q)] = bx; W[wix<R>(G, W_BY, q)] = by; W[wix<R>(G, W_BZ, q)] = bz;
@@ -181,7 +176,7 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     W[wix<R>(G, W_GC, q)] = o.gc - b.gc;
 #pragma unroll
     for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-      if (l < G.nspec) W[wix<R>(G, W_X0 + l, q)] = X[l];
+      if (l < G.nspec) W[wix<R>(G, W_X0 + l, q)] = cs.rX[l] * cs.irho;
   }
   if constexpr (sizeof(R) == 4) {
     float w[W_P + 1];
@@ -198,7 +193,7 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     const float fr = d2f_scaled(rho, 0), ifr = 1.0f / fr;
     const float a2 = d2f_scaled(o.gc * o.P, 0) * ifr;
     const float fv[3] = {d2f_scaled(vx, 0), d2f_scaled(vy, 0), d2f_scaled(vz, 0)};
-    const float fb[3] = {d2f_scaled(bx, 0), d2f_scaled(by, 0), d2f_scaled(bz, 0)};
+    const float fb[3] = {d2f_scaled(cs.b2[0], -1), d2f_scaled(cs.b2[1], -1), d2f_scaled(cs.b2[2], -1)};
     const float b2 = (fb[0] * fb[0] + fb[1] * fb[1] + fb[2] * fb[2]) * ifr;
     float sum = 0.0f;
     for (int d = 0; d < 3; ++d) {
@@ -209,6 +204,7 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     }
     return (sum == sum) ? (double)sum : INFINITY;
   } else {
+    const double bx = 0.5 * cs.b2[0], by = 0.5 * cs.b2[1], bz = 0.5 * cs.b2[2];
     const double a2 = o.gc * o.P / rho, b2 = (bx * bx + by * by + bz * bz) / rho;
     const double vv[3] = {vx, vy, vz}, bb[3] = {bx, by, bz};
     double sum = 0.0;
@@ -294,22 +290,23 @@ __global__ void k_dt_stellar(DevGeo G, Box box, const double *__restrict__ U, co
                           0.5 * (Bf[2 * pl + p] + Bf[2 * pl + p + G.sz])};
     const double b2 = bc[0] * bc[0] + bc[1] * bc[1] + bc[2] * bc[2];
     const double eint = U[4 * pl + p] / rho - 0.5 * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) - 0.5 * b2 / rho;
-    double X[PHL_NSPEC_MAX];
+    double rX[PHL_NSPEC_MAX];
 #pragma unroll
     for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-      if (l < G.nspec) X[l] = U[(5 + l) * pl + p] / rho;
-    double abar, ye;
-    mixture<double>(G, X, abar, ye);
+      if (l < G.nspec) rX[l] = U[(5 + l) * pl + p];
+    double iab, ye, is;
+    mixture(G, rX, iab, ye, is);
+    const double abar = 1.0 / iab;
     R T = (R)Tin[p];
     eos::EosOut<R> o;
     if (sizeof(R) == 8) {
-      if (eos::eos_invert<R>(G.tab, (R)rho, (R)eint, (R)abar, (R)ye, T, (R)G.newton_tol, G.newton_maxit, o) < 0)
+      if (eos::eos_invert<R>(G.tab, (R)rho, (R)(1.0 / rho), (R)eint, (R)iab, (R)ye, T, (R)G.newton_tol, G.newton_maxit, o) < 0)
         atomicOr(dflag, FLAG_NEWTON);
     } else {
       // the CFL step needs c_s to a few digits: FP32 Newton to 1e-5 (FP32's own
       // floor for ln n, ln T is ~1e-6); a stalled iteration keeps its last,
       // bracketed iterate
-      if (eos::eos_invert<R>(G.tab, (R)rho, (R)eint, (R)abar, (R)ye, T, (R)1e-5, 16, o) < 0 &&
+      if (eos::eos_invert<R>(G.tab, (R)rho, (R)(1.0 / rho), (R)eint, (R)iab, (R)ye, T, (R)1e-5, 16, o) < 0 &&
           !eos::eos_rt<R>(G.tab, (R)rho, T, (R)abar, (R)ye, o))
         atomicOr(dflag, FLAG_NEWTON);
     }
@@ -365,8 +362,9 @@ __global__ void k_bg_stellar(DevGeo G, int L, double *bg, double *bgX, int *fail
   const int q = face ? i - L : i;
   if (!face && q == L - 1) return;          // centres have one value fewer
   const double rho = bg[(face ? 2 : 0) * L + q], P = bg[(face ? 3 : 1) * L + q];
-  double abar, ye;
-  mixture<double>(G, bgX, abar, ye);
+  double iab, ye, is;
+  mixture(G, bgX, iab, ye, is);
+  const double abar = 1.0 / iab;
   double T = 1e9;
   eos::EosOut<double> o;
   if (!p_to_T(G, rho, P, abar, ye, T, o)) { atomicOr(fail, 1); return; }
@@ -397,8 +395,9 @@ __global__ void k_prim_to_cons(DevGeo G, Box box, const double *__restrict__ pri
   if (G.eos == 0) {
     e = P / ((G.gamma - 1.0) * rho);
   } else {
-    double abar, ye;
-    mixture<double>(G, X, abar, ye);
+    double iab, ye, is;
+    mixture(G, X, iab, ye, is);
+    const double abar = 1.0 / iab;
     Tc = 1e9;
     eos::EosOut<double> o;
     if (!p_to_T(G, rho, P, abar, ye, Tc, o)) atomicOr(dflag, FLAG_NEWTON);

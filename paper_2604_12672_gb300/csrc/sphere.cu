@@ -381,7 +381,7 @@ struct SphDev {
   int stellar;
   eos::Table tab;
   double abar, ye, rho_u, p_u, e_u, ntol;
-  double irho_u, iabar;        // 1 / rho_u, 1 / Abar
+  double irho_u, ip_u, iabar;  // 1 / rho_u, 1 / p_u, 1 / Abar
   int nmaxit;
   const double *ge_c, *gc_c, *ge_f, *gc_f;   // background gamma_e, gamma_c: shells (Nr), radii (Nr + 1)
   const float *ge_cf, *gc_cf, *ge_ff, *gc_ff;
@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, c
       rho += f2d_scaled(dU[c], 0); mx += f2d_scaled(dU[n + c], 0); my += f2d_scaled(dU[2 * n + c], 0);
       mz += f2d_scaled(dU[3 * n + c], 0); E += f2d_scaled(dU[4 * n + c], 0);
     }
-    const double ir = 1.0 / rho;
+    const double ir = eos::rcp_nr(rho);
     const double ux = mx * ir, uy = my * ir, uz = mz * ir;
     const double eint = (E - 0.5 * (mx * ux + my * uy + mz * uz) - 0.5 * (bx * bx + by * by + bz * bz)) * ir;
     double T = D.T[c];
@@ -748,18 +748,18 @@ __global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, c
       eos::Pred pr{};
       double *rp = D.pred + c;
       if (pm == 2) pr = eos::Pred{rp[0], rp[n], rp[2 * n], rp[3 * n], rp[4 * n], rp[5 * n], rp[6 * n], rp[7 * n]};
-      it = eos::eos_invert_rec(D.tab, rho * D.rho_u, ir * D.irho_u, eint * D.e_u, D.abar, D.iabar, D.ye, T, D.ntol,
-                               D.nmaxit, o, pr, pm == 2);
+      it = eos::eos_invert_rec(D.tab, rho * D.rho_u, ir * D.irho_u, eint * D.e_u, D.iabar, D.ye, T, D.ntol, D.nmaxit,
+                               o, pr, pm == 2);
       rp[0] = pr.rho; rp[n] = pr.e; rp[2 * n] = pr.icv; rp[3 * n] = pr.er;
       rp[4 * n] = pr.lnT; rp[5 * n] = pr.iT; rp[6 * n] = pr.x; rp[7 * n] = pr.ine;
     } else {
       it = sizeof(R) == 8
-               ? eos::eos_invert<double>(D.tab, rho * D.rho_u, eint * D.e_u, D.abar, D.ye, T, D.ntol, D.nmaxit, o)
-               : eos::eos_invert_mixed(D.tab, rho * D.rho_u, eint * D.e_u, D.abar, D.ye, T, D.ntol, D.nmaxit, o);
+               ? eos::eos_invert<double>(D.tab, rho * D.rho_u, ir * D.irho_u, eint * D.e_u, D.iabar, D.ye, T, D.ntol, D.nmaxit, o)
+               : eos::eos_invert_mixed(D.tab, rho * D.rho_u, ir * D.irho_u, eint * D.e_u, D.iabar, D.ye, T, D.ntol, D.nmaxit, o);
     }
     if (it < 0) atomicOr(D.dflag, FLAG_NEWTON);
     D.T[c] = T;
-    const double P = o.P / D.p_u;
+    const double P = o.P * D.ip_u;
     if (!(rho > 0.0) || !(P > 0.0)) atomicOr(D.dflag, FLAG_NEG);
     if (!isfinite(rho) || !isfinite(P)) atomicOr(D.dflag, FLAG_NAN);
     double geh, gch;
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, c
       float4 *W4 = reinterpret_cast<float4 *>(Wk.W);
       W4[3 * c] = make_float4(drho, fux, fuy, fuz);
       W4[3 * c + 1] = make_float4(fbx, fby, fbz, fdP);
-      W4[3 * c + 2] = make_float4((float)dge, (float)dgc, 0.f, 0.f);
+      W4[3 * c + 2] = make_float4(d2f_scaled(dge, 0), d2f_scaled(dgc, 0), 0.f, 0.f);
       if (dmax) {
         const float frho = (D.rho_cf ? D.rho_cf[k] : 0.f) + drho, fP = (D.p_cf ? D.p_cf[k] : 0.f) + fdP;
         rate = cfl_rate_mx(D, a, k, frho, fP, fux, fuy, fuz, fbx, fby, fbz, (float)o.gc);
@@ -1555,7 +1555,7 @@ phl_status phl_sphere_create(const phl_sphere_desc *d, phl_sphere **out) {
     D.abar = 1.0 / inv_abar;
     D.iabar = inv_abar;
     D.ye = ye;
-    D.rho_u = d->rho_unit; D.p_u = d->p_unit; D.e_u = d->p_unit / d->rho_unit; D.irho_u = 1.0 / d->rho_unit;
+    D.rho_u = d->rho_unit; D.p_u = d->p_unit; D.e_u = d->p_unit / d->rho_unit; D.irho_u = 1.0 / d->rho_unit; D.ip_u = 1.0 / d->p_unit;
     D.ntol = d->newton_tol > 0.0 ? d->newton_tol : 1e-11;
     D.nmaxit = d->newton_maxit > 0 ? d->newton_maxit : 50;
     if (d->mlp) {
