@@ -133,25 +133,84 @@ phl_status copy_field(phl_grid *g, double *dev, const double *abi_src, double *a
   return PHL_OK;
 }
 
-// Dense (ABI) <-> padded device layout of one field with extents (ex, ey, ez):
-// one CTA per x-row, consecutive threads on consecutive elements.
-__global__ void k_repitch(const double *__restrict__ src, double *__restrict__ dst, int ex, int ey, long sy, long sz,
-                          int to_dev) {
-  const long row = blockIdx.x;   // j + ey * k
-  const long j = row % ey, k = row / ey;
-  const long dense = row * ex, padded = j * sy + k * sz;
-  for (int i = threadIdx.x; i < ex; i += blockDim.x) {
-    if (to_dev) dst[padded + i] = src[dense + i];
-    else dst[dense + i] = src[padded + i];
+// Dense (ABI) <-> padded device layout of every state field in one launch: a
+// field's elements in dense order, in units of two doubles where its x extent
+// is even and both pointers sit on 16 bytes (all fields but the x-faces when
+// n_x is even), else of one; IO_U units per thread, loaded before the first
+// is stored.  HBM bound; one launch per field with one row per block moved
+// 4.2 TB/s at 256^3 (eight launches, 512 us a direction) and was mostly launch
+// cost on small boxes.
+constexpr int IO_T = 256, IO_U = 4;
+struct IoField {
+  double *dense, *padded;
+  unsigned units, blk0;   // units of the field, first block
+  int vec;
+  FastDiv fx, fy;         // by the units of a row and the rows of a plane
+};
+struct IoFields {
+  IoField f[5 + PHL_MAXSPEC + 3];   // conserved variables, face fields
+  int n;
+  long sy, sz;
+};
+template <bool TO_DEV>
+__global__ void __launch_bounds__(IO_T) k_state_io(const __grid_constant__ IoFields A) {
+  int k = 0;
+  while (k + 1 < A.n && blockIdx.x >= A.f[k + 1].blk0) ++k;
+  const IoField &F = A.f[k];
+  const unsigned e0 = (blockIdx.x - F.blk0) * (IO_T * IO_U) + threadIdx.x;
+  auto padded = [&](unsigned e) {
+    const unsigned row = fastdiv(e, F.fx), i = e - row * F.fx.d;
+    const unsigned z = fastdiv(row, F.fy), y = row - z * F.fy.d;
+    return (long)(F.vec ? 2 * i : i) + A.sy * y + A.sz * z;
+  };
+  if (F.vec) {
+    double2 v[IO_U];
+#pragma unroll
+    for (int u = 0; u < IO_U; ++u) {
+      const unsigned e = e0 + u * IO_T;
+      if (e < F.units)
+        v[u] = TO_DEV ? reinterpret_cast<const double2 *>(F.dense)[e]
+                      : *reinterpret_cast<const double2 *>(F.padded + padded(e));
+    }
+#pragma unroll
+    for (int u = 0; u < IO_U; ++u) {
+      const unsigned e = e0 + u * IO_T;
+      if (e < F.units)
+        (TO_DEV ? *reinterpret_cast<double2 *>(F.padded + padded(e)) : reinterpret_cast<double2 *>(F.dense)[e]) = v[u];
+    }
+  } else {
+    double v[IO_U];
+#pragma unroll
+    for (int u = 0; u < IO_U; ++u) {
+      const unsigned e = e0 + u * IO_T;
+      if (e < F.units) v[u] = TO_DEV ? F.dense[e] : F.padded[padded(e)];
+    }
+#pragma unroll
+    for (int u = 0; u < IO_U; ++u) {
+      const unsigned e = e0 + u * IO_T;
+      if (e < F.units) (TO_DEV ? F.padded[padded(e)] : F.dense[e]) = v[u];
+    }
   }
+}
+void io_add(IoFields &A, unsigned &blocks, double *dense, double *padded, int ex, int ey, int ez) {
+  IoField &F = A.f[A.n++];
+  F.dense = dense;
+  F.padded = padded;
+  F.vec = ex % 2 == 0 && (((uintptr_t)dense | (uintptr_t)padded) & 15) == 0;
+  const int xu = F.vec ? ex / 2 : ex;
+  F.units = (unsigned)((long)xu * ey * ez);
+  F.fx = make_fastdiv((unsigned)xu);
+  F.fy = make_fastdiv((unsigned)ey);
+  F.blk0 = blocks;
+  blocks += (F.units + IO_T * IO_U - 1) / (IO_T * IO_U);
 }
 
 // The state (nv cell fields and three face fields) between ABI arrays and the
-// device layout.  Device arrays: one repitch kernel per field, straight from
-// or into the caller's buffers.  Host arrays: one linear copy per array
-// through the grid's work arrays (dead between steps), at full link bandwidth,
-// plus the repitch kernels; pitched 3-D copies only when the work arrays are
-// too small to hold the dense state.
+// device layout.  Device arrays: one kernel straight from or into the
+// caller's buffers.  Host arrays: one linear copy per array through the grid's
+// work arrays (dead between steps), at full link bandwidth, plus that kernel;
+// pitched 3-D copies only when the work arrays are too small to hold the
+// dense state.
 phl_status state_io(phl_grid *g, double *cons, double *bx, double *by, double *bz, bool to_dev, bool host) {
   const DevGeo &G = g->G;
   const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
@@ -187,18 +246,16 @@ phl_status state_io(phl_grid *g, double *cons, double *bx, double *by, double *b
     for (int d = 0; d < 3; ++d)
       CK(cudaMemcpyAsync(fa[d], face_abi[d], nf[d] * sizeof(double), cudaMemcpyHostToDevice, g->stream), "copy B");
   }
-  for (int v = 0; v < G.nv; ++v) {
-    double *dev = g->U + v * G.plane;
-    if (to_dev) k_repitch<<<(unsigned)((long)ny * nz), 256, 0, g->stream>>>(ca + v * nc, dev, nx, ny, G.sy, G.sz, 1);
-    else k_repitch<<<(unsigned)((long)ny * nz), 256, 0, g->stream>>>(dev, ca + v * nc, nx, ny, G.sy, G.sz, 0);
-  }
-  for (int d = 0; d < 3; ++d) {
-    double *dev = g->B + d * G.plane;
-    const unsigned rows = (unsigned)((long)ext[d][1] * ext[d][2]);
-    if (to_dev) k_repitch<<<rows, 256, 0, g->stream>>>(fa[d], dev, ext[d][0], ext[d][1], G.sy, G.sz, 1);
-    else k_repitch<<<rows, 256, 0, g->stream>>>(dev, fa[d], ext[d][0], ext[d][1], G.sy, G.sz, 0);
-  }
-  CK(cudaGetLastError(), "repitch");
+  IoFields A;
+  A.n = 0;
+  A.sy = G.sy;
+  A.sz = G.sz;
+  unsigned blocks = 0;
+  for (int v = 0; v < G.nv; ++v) io_add(A, blocks, ca + v * nc, g->U + v * G.plane, nx, ny, nz);
+  for (int d = 0; d < 3; ++d) io_add(A, blocks, fa[d], g->B + d * G.plane, ext[d][0], ext[d][1], ext[d][2]);
+  if (to_dev) k_state_io<true><<<blocks, IO_T, 0, g->stream>>>(A);
+  else k_state_io<false><<<blocks, IO_T, 0, g->stream>>>(A);
+  CK(cudaGetLastError(), "state layout");
   if (staged && !to_dev) {
     CK(cudaMemcpyAsync(cons, ca, cons_bytes, cudaMemcpyDeviceToHost, g->stream), "copy state");
     for (int d = 0; d < 3; ++d)
