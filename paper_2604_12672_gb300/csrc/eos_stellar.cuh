@@ -33,6 +33,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "fp64_math.cuh"
+
 namespace phl {
 namespace eos {
 
@@ -69,19 +71,6 @@ struct Table {
   double Tlo, Thi;            // the table's temperature range, exp(y0) and
   float Tlof, Thif;           // exp(y0 + (ny - 1) dy), set with the table
 };
-
-// 1/x to about one unit in the last place for normal x: the hardware's gross
-// approximation (relative error below 2^-19) and one step of the third-order
-// Newton-Halley iteration y (1 + e + e^2), e = 1 - x y (remaining error e^3 <
-// 2^-57): three FP64 multiply-adds, where the full-range division takes about
-// a dozen FP64-pipe instructions and a branch.  0 and infinity give NaN.
-__device__ __forceinline__ double rcp_nr(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ float rcp_nr(float x) { return 1.0f / x; }
 
 // Position along x (x = ln n_e): table interval and fraction, fixed during
 // an inversion.

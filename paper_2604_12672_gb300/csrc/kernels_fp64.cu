@@ -5,16 +5,22 @@
 //                 deviations from the background (Sects. 2.2, 2.8); ghost
 //                 cells are produced by mapping to their interior source cell
 //                 (Table bcs) -- no ghost storage in the state.
-//   k_flag_raw    shock indicator of Sect. 2.7 on interior cells.
-//   k_flag_dilate 5^d dilation of the indicator (Sect. 2.7).
-//   k_flux<D>     van Leer PLM of the deviations (Sect. 2.5), background added
+//   k_flag_raw    shock indicator of Sect. 2.7 on interior cells, then its 5^d
+//                 dilation (launch_flags).
+//   k_flux_walk   van Leer PLM of the deviations (Sect. 2.5), background added
 //                 at the face, LHLLD / HLL flux minus F_hat (Eqs. flux-hlld,
-//                 pstar, wb1).
-//   k_emf<D>      Contact-CT edge EMFs (Sect. 2.4).
+//                 pstar, wb1), several faces per thread; k_flux for the other
+//                 reconstructions.
+//   k_emf_all     Contact-CT edge EMFs (Sect. 2.4).
 //   k_update_*    residual with sources (Eqs. fv, spatres, wb2) and the SSP-RK
 //                 combination for cells and faces (Sect. 2.9).
-//   k_dt          CFL condition (Eq. cfl): warp-shuffle / block max, one
-//                 atomic per block, finalised on the device.
+//   k_dt          CFL condition (Eq. cfl) for phl_compute_dt; a step takes it
+//                 from its first stage's k_prim.
+//
+// The FP64 pipe bounds the stage: 128 x 96 x 112 cells take 3.6 ms, 2.8 of
+// them in the faces (6.5 and 5.1 ms with full-range divisions and roots,
+// every slope formed twice, a CFL pass of its own and three launches for each
+// of the EMFs and face updates).
 #include <math.h>
 
 #include "phl_internal.cuh"
@@ -32,13 +38,13 @@ __device__ __forceinline__ bool cell_prims(const DevGeo &G, const double *__rest
   const long p = sidx(G, i, j, k);
   const long pl = G.plane;
   const double rho = U[p];
-  const double vx = U[pl + p] / rho, vy = U[2 * pl + p] / rho, vz = U[3 * pl + p] / rho;
+  const double ir = rcp_nr(rho);
+  const double mx = U[pl + p], my = U[2 * pl + p], mz = U[3 * pl + p];
+  const double vx = mx * ir, vy = my * ir, vz = mz * ir;
   const double bx = 0.5 * (Bf[p] + Bf[p + 1]);
   const double by = 0.5 * (Bf[pl + p] + Bf[pl + p + G.sy]);
   const double bz = 0.5 * (Bf[2 * pl + p] + Bf[2 * pl + p + G.sz]);
-  const double eint = U[4 * pl + p] / rho - 0.5 * (vx * vx + vy * vy + vz * vz) -
-                      0.5 * (bx * bx + by * by + bz * bz) / rho;
-  const double P = (G.gamma - 1.0) * rho * eint;
+  const double P = (G.gamma - 1.0) * (U[4 * pl + p] - 0.5 * (mx * vx + my * vy + mz * vz) - 0.5 * (bx * bx + by * by + bz * bz));
   const Bg b = bg_cell(G, k);
   w[W_RHO] = rho - b.rho;
   w[W_VX] = vx; w[W_VY] = vy; w[W_VZ] = vz;
@@ -48,32 +54,72 @@ __device__ __forceinline__ bool cell_prims(const DevGeo &G, const double *__rest
   w[W_GC] = G.gamma - b.gc;
 #pragma unroll
   for (int l = 0; l < PHL_NSPEC_MAX; ++l)
-    if (l < G.nspec) w[W_X0 + l] = U[(U_X0 + l) * pl + p] / rho;
+    if (l < G.nspec) w[W_X0 + l] = U[(U_X0 + l) * pl + p] * ir;
   bool ok = true;
   if (!(rho > 0.0) || !(P > 0.0)) { atomicOr(dflag, FLAG_NEG); ok = false; }
   if (!isfinite(P) || !isfinite(rho)) { atomicOr(dflag, FLAG_NAN); ok = false; }
   return ok;
 }
 
-__global__ void k_prim(DevGeo G, Box box, const double *__restrict__ U, const double *__restrict__ Bf,
-                       double *__restrict__ W, int *dflag) {
-  {
-    int c[3], s[3];
-    bool fl[3];
-    if (!cell3(box, c)) return;
+// CFL sum of a cell from its deviations w at height k (Eq. cfl).
+__device__ __forceinline__ double dt_rate(const DevGeo &G, const double *w, int k) {
+  const Bg b = bg_cell(G, k);
+  const double ir = rcp_nr(w[W_RHO] + b.rho), P = w[W_P] + b.p, gc = w[W_GC] + b.gc;
+  const double a2 = gc * P * ir;
+  const double ab = a2 + (w[W_BX] * w[W_BX] + w[W_BY] * w[W_BY] + w[W_BZ] * w[W_BZ]) * ir;
+  double s = 0.0;
+  for (int d = 0; d < 3; ++d) {
+    if (!G.act[d]) continue;
+    double disc = ab * ab - 4.0 * a2 * (w[W_BX + d] * w[W_BX + d] * ir);
+    if (disc < 0.0) disc = 0.0;
+    s += (fabs(w[W_VX + d]) + sqrt_nr(0.5 * (ab + sqrt_nr(disc)))) * G.idx[d];
+  }
+  return (s == s) ? s : INFINITY;
+}
+
+__device__ __forceinline__ void atomic_max_pos(unsigned long long *addr, double v) {
+  // non-negative doubles order like their bit patterns
+  atomicMax(addr, (unsigned long long)__double_as_longlong(v));
+}
+// Block maximum of m into *dmax (every thread of the block calls).
+__device__ __forceinline__ void block_dmax(double m, unsigned long long *dmax) {
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  __shared__ double red[TPB / 32];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = red[0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, red[w]);
+    atomic_max_pos(dmax, v);
+  }
+}
+
+// dmax (the step's first stage with the device CFL step; else null): the CFL
+// maximum of the interior cells from the deviations just formed, instead of a
+// second pass over the state.
+__global__ void __launch_bounds__(256) k_prim(DevGeo G, Box box, const double *__restrict__ U,
+                                              const double *__restrict__ Bf, double *__restrict__ W, int *dflag,
+                                              unsigned long long *dmax) {
+  int c[3], s[3];
+  double rate = 0.0;
+  if (cell3(box, c)) {
+    bool fl[3], in = true;
     for (int d = 0; d < 3; ++d) {
       fl[d] = false;
       s[d] = G.act[d] ? cell_src(c[d], G.n[d], G.bc[d][0], G.bc[d][1], fl[d]) : 0;
+      in = in && c[d] >= 0 && c[d] < G.n[d];
     }
     double w[NW_MAX];
     cell_prims(G, U, Bf, s[0], s[1], s[2], w, dflag);
+    if (dmax && in) rate = dt_rate(G, w, c[2]);
     for (int d = 0; d < 3; ++d)
       if (fl[d]) { w[W_VX + d] = -w[W_VX + d]; w[W_BX + d] = -w[W_BX + d]; }
     const long q = widx(G, c[0], c[1], c[2]);
 #pragma unroll
-    for (int v = 0; v < NW_MAX; ++v)
-      if (v < G.nw) W[v * G.wtot + q] = w[v];
+    for (int v = 0; v < NW_MAX; ++v)   // an ideal gas reconstructs no gamma deviations
+      if (v < G.nw && v != W_GE && v != W_GC) W[v * G.wtot + q] = w[v];
   }
+  if (dmax) block_dmax(rate, dmax);
 }
 
 __global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
@@ -93,7 +139,7 @@ __global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
       for (int d = 0; d < 3; ++d) {
         if (!G.act[d]) continue;
         const double *f = S.F[d] + fc * wt;
-        s += (f[p + wstride(G, d)] - f[p]) / G.dx[d];
+        s += (f[p + wstride(G, d)] - f[p]) * G.idx[d];
       }
       r[v] = s;
     }
@@ -116,27 +162,29 @@ __global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
 }
 
 template <int D>
-__global__ void k_update_faces(DevGeo G, Box box, StageBufs S) {
+__device__ __forceinline__ void face_update_fp64(const DevGeo &G, const int *c, const StageBufs &S, double dt) {
   constexpr int A = (D + 1) % 3, B = (D + 2) % 3;
-  const double dt = *S.dt;
-  {
-    int c[3];
-    if (!cell3(box, c)) return;
-    int e[3] = {c[0], c[1], c[2]};
-    if (!G.act[D]) e[D] = 0;
-    const long p = widx(G, e[0], e[1], e[2]);
-    const long wt = G.wtot;
-    double r = 0.0;
-    if (G.act[A]) r += (S.E[(long)B * wt + p + wstride(G, A)] - S.E[(long)B * wt + p]) / G.dx[A];
-    if (G.act[B]) r -= (S.E[(long)A * wt + p + wstride(G, B)] - S.E[(long)A * wt + p]) / G.dx[B];
-    const long q = (long)D * G.plane + sidx(G, c[0], c[1], c[2]);
-    S.Bout[q] = S.a * S.Bbase[q] + S.b * S.Bin[q] - S.b * dt * r;
-  }
+  int e[3] = {c[0], c[1], c[2]};
+  if (!G.act[D]) e[D] = 0;
+  const long p = widx(G, e[0], e[1], e[2]);
+  const long wt = G.wtot;
+  double r = 0.0;
+  if (G.act[A]) r += (S.E[(long)B * wt + p + wstride(G, A)] - S.E[(long)B * wt + p]) * G.idx[A];
+  if (G.act[B]) r -= (S.E[(long)A * wt + p + wstride(G, B)] - S.E[(long)A * wt + p]) * G.idx[B];
+  const long q = (long)D * G.plane + sidx(G, c[0], c[1], c[2]);
+  S.Bout[q] = S.a * S.Bbase[q] + S.b * S.Bin[q] - S.b * dt * r;
 }
-
-__device__ __forceinline__ void atomic_max_pos(unsigned long long *addr, double v) {
-  // non-negative doubles order like their bit patterns
-  atomicMax(addr, (unsigned long long)__double_as_longlong(v));
+// The three face components of a site (box: [0, n] along every axis).  Every
+// face array is written: a field with no active curl direction still takes
+// the RK combination a * base + b * in.
+__global__ void k_update_faces(DevGeo G, Box box, StageBufs S) {
+  int c[3];
+  if (!cell3(box, c)) return;
+  const double dt = *S.dt;
+  const bool in[3] = {c[0] < G.n[0], c[1] < G.n[1], c[2] < G.n[2]};
+  if (in[1] && in[2]) face_update_fp64<0>(G, c, S, dt);
+  if (in[0] && in[2]) face_update_fp64<1>(G, c, S, dt);
+  if (in[0] && in[1]) face_update_fp64<2>(G, c, S, dt);
 }
 
 __global__ void k_dt(DevGeo G, Box box, const double *__restrict__ U, const double *__restrict__ Bf,
@@ -147,30 +195,10 @@ __global__ void k_dt(DevGeo G, Box box, const double *__restrict__ U, const doub
     unflat(box, t, c);
     double w[NW_MAX];
     cell_prims(G, U, Bf, c[0], c[1], c[2], w, dflag);
-    const Bg b = bg_cell(G, c[2]);
-    const double rho = w[W_RHO] + b.rho, P = w[W_P] + b.p, gc = w[W_GC] + b.gc;
-    const double a2 = gc * P / rho;
-    const double b2 = (w[W_BX] * w[W_BX] + w[W_BY] * w[W_BY] + w[W_BZ] * w[W_BZ]) / rho;
-    double s = 0.0;
-    for (int d = 0; d < 3; ++d) {
-      if (!G.act[d]) continue;
-      const double bd2 = w[W_BX + d] * w[W_BX + d] / rho;
-      double disc = (a2 + b2) * (a2 + b2) - 4.0 * a2 * bd2;
-      if (disc < 0.0) disc = 0.0;
-      const double cf = sqrt(0.5 * (a2 + b2 + sqrt(disc)));
-      s += (fabs(w[W_VX + d]) + cf) / G.dx[d];
-    }
-    if (s > m || !(s == s)) m = (s == s) ? s : INFINITY;
+    const double r = dt_rate(G, w, c[2]);
+    if (r > m) m = r;
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  __shared__ double red[TPB / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) atomic_max_pos(dmax, v);
-  }
+  block_dmax(m, dmax);
 }
 
 __global__ void k_dt_finalize(double cfl, unsigned long long *dmax, double *dt) {
@@ -209,16 +237,17 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
       launch_eos_cells<double>(G, S.Uin, S.Bin, nullptr, nullptr, S.Tin, S.Tout, S.W, S.dflag, s, &nl, prof,
                                S.cfl_dmax, const_cast<double *>(S.dt));
     } else {
-      PHL_LAUNCH(KC_PRIM, prof, s, k_prim<<<grid3(b), block3(b), 0, s>>>(G, b, S.Uin, S.Bin, S.W, S.dflag));
+      const unsigned t = tpb_for(b.n);
+      PHL_LAUNCH(KC_PRIM, prof, s, k_prim<<<gridt(b, t), t, 0, s>>>(G, b, S.Uin, S.Bin, S.W, S.dflag, S.cfl_dmax));
+      if (S.cfl_dmax) {
+        PHL_LAUNCH(KC_DT, prof, s, k_dt_finalize<<<1, 1, 0, s>>>(G.cfl, S.cfl_dmax, const_cast<double *>(S.dt)));
+        ++nl;
+      }
       ++nl;
     }
   }
   // (2) shock flags
-  if (G.eps_sf > 0.0) {
-    Box bx = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-    PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw<double><<<grid3(bx), block3(bx), 0, s>>>(G, bx, S.W, S.raw));
-    nl += 1 + launch_flags(G, S.raw, S.raw + (long)G.n[0] * G.n[1] * G.n[2], S.flag, s, prof);
-  }
+  if (G.eps_sf > 0.0) nl += launch_flags<double>(G, S.W, S.raw, S.raw + (long)G.n[0] * G.n[1] * G.n[2], S.flag, S.any, s, prof);
   // (3) fluxes: normal faces [0, n], one transverse ghost row each side
   for (int D = 0; D < 3; ++D) {
     if (!G.act[D]) continue;
@@ -232,35 +261,20 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
     ++nl;
   }
   // (4) edge EMFs
-  for (int D = 0; D < 3; ++D) {
-    const int A = (D + 1) % 3, B = (D + 2) % 3;
-    if (!G.act[A] && !G.act[B]) continue;
-    int l[3] = {0, 0, 0}, h[3];
-    h[D] = G.n[D];
-    h[A] = G.act[A] ? G.n[A] + 1 : 1;
-    h[B] = G.act[B] ? G.n[B] + 1 : 1;
-    Box b = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
-    if (D == 0) PHL_LAUNCH(KC_EMF, prof, s, k_emf<0, double><<<grid3(b), block3(b), 0, s>>>(G, b, S.W, S.F[1], S.F[2], S.E));
-    if (D == 1) PHL_LAUNCH(KC_EMF, prof, s, k_emf<1, double><<<grid3(b), block3(b), 0, s>>>(G, b, S.W, S.F[2], S.F[0], S.E));
-    if (D == 2) PHL_LAUNCH(KC_EMF, prof, s, k_emf<2, double><<<grid3(b), block3(b), 0, s>>>(G, b, S.W, S.F[0], S.F[1], S.E));
+  {
+    const Box b = site_box(G);
+    const unsigned t = tpb_for(b.n);
+    PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<double><<<gridt(b, t), t, 0, s>>>(G, b, S.W, S.F[0], S.F[1], S.F[2], S.E));
     ++nl;
   }
   // (5) updates
   {
     Box b = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-    PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells<<<grid3(b), block3(b), 0, s>>>(G, b, S));
-    ++nl;
-  }
-  for (int D = 0; D < 3; ++D) {
-    // every face array is written: a field with no active curl direction still
-    // takes the RK combination a * base + b * in
-    int h[3] = {G.n[0], G.n[1], G.n[2]};
-    h[D] += 1;
-    Box b = make_box(0, h[0], 0, h[1], 0, h[2]);
-    if (D == 0) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<0><<<grid3(b), block3(b), 0, s>>>(G, b, S));
-    if (D == 1) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<1><<<grid3(b), block3(b), 0, s>>>(G, b, S));
-    if (D == 2) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<2><<<grid3(b), block3(b), 0, s>>>(G, b, S));
-    ++nl;
+    const unsigned t = tpb_for(b.n);
+    PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells<<<gridt(b, t), t, 0, s>>>(G, b, S));
+    Box bf = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
+    PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<<<gridt(bf, t), t, 0, s>>>(G, bf, S));
+    nl += 2;
   }
   if (nlaunch) *nlaunch += nl;
 }

@@ -63,9 +63,14 @@ __global__ void k_update_cells_mx(DevGeo G, Box box, StageMx S) {
   k_update_cells_mx_at(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, S);
 }
 
-template <int D>
+// The three face components of a site (box: [0, n] along every axis).
 __global__ void k_update_faces_mx(DevGeo G, Box box, StageMx S) {
-  k_update_faces_mx_at<D>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, S);
+  int c[3];
+  if (!cell3(box, c)) return;
+  const bool in[3] = {c[0] < G.n[0], c[1] < G.n[1], c[2] < G.n[2]};
+  if (in[1] && in[2]) face_update_mx<0>(G, c, S);
+  if (in[0] && in[2]) face_update_mx<1>(G, c, S);
+  if (in[0] && in[1]) face_update_mx<2>(G, c, S);
 }
 
 // CFL condition in FP32 from U^n (Eq. cfl); non-negative floats order like
@@ -188,11 +193,7 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
       ++nl;
     }
   }
-  if (G.eps_sf > 0.0 && !fused) {
-    Box bx = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-    PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw<float><<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.W, M.raw));
-    nl += 1 + launch_flags(G, M.raw, M.raw + (long)G.n[0] * G.n[1] * G.n[2], M.flag, s, prof);
-  }
+  if (G.eps_sf > 0.0 && !fused) nl += launch_flags<float>(G, M.W, M.raw, M.raw + (long)G.n[0] * G.n[1] * G.n[2], M.flag, M.anyraw, s, prof);
   if (fused) launch_fused_tail(G, M, first, last, b, s, &nl, prof);   // flags, faces, cells, EMFs, faces B
   for (int D = 0; D < 3 && !fused; ++D) {
     if (!G.act[D]) continue;
@@ -205,17 +206,10 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
     launch_flux<float>(D, G, bx, M.W, M.B, dB, M.flag, M.F[D], M.dflag, s, prof);
     ++nl;
   }
-  for (int D = 0; D < 3 && !fused; ++D) {
-    const int A = (D + 1) % 3, B = (D + 2) % 3;
-    if (!G.act[A] && !G.act[B]) continue;
-    int l[3] = {0, 0, 0}, h[3];
-    h[D] = G.n[D];
-    h[A] = G.act[A] ? G.n[A] + 1 : 1;
-    h[B] = G.act[B] ? G.n[B] + 1 : 1;
-    Box bx = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
-    if (D == 0) PHL_LAUNCH(KC_EMF, prof, s, k_emf<0, float><<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.W, M.F[1], M.F[2], M.E));
-    if (D == 1) PHL_LAUNCH(KC_EMF, prof, s, k_emf<1, float><<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.W, M.F[2], M.F[0], M.E));
-    if (D == 2) PHL_LAUNCH(KC_EMF, prof, s, k_emf<2, float><<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.W, M.F[0], M.F[1], M.E));
+  if (!fused) {
+    const Box bs = site_box(G);
+    const unsigned t = tpb_for(bs.n);
+    PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<float><<<gridt(bs, t), t, 0, s>>>(G, bs, M.W, M.F[0], M.F[1], M.F[2], M.E));
     ++nl;
   }
   StageMx S;
@@ -227,13 +221,10 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
     PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells_mx<<<grid3(bx), block3(bx), 0, s>>>(G, bx, S));
     ++nl;
   }
-  for (int D = 0; D < 3 && !fused; ++D) {
-    int h[3] = {G.n[0], G.n[1], G.n[2]};
-    h[D] += 1;
-    Box bx = make_box(0, h[0], 0, h[1], 0, h[2]);
-    if (D == 0) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces_mx<0><<<grid3(bx), block3(bx), 0, s>>>(G, bx, S));
-    if (D == 1) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces_mx<1><<<grid3(bx), block3(bx), 0, s>>>(G, bx, S));
-    if (D == 2) PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces_mx<2><<<grid3(bx), block3(bx), 0, s>>>(G, bx, S));
+  if (!fused) {
+    const Box bf = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
+    const unsigned t = tpb_for(bf.n);
+    PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces_mx<<<gridt(bf, t), t, 0, s>>>(G, bf, S));
     ++nl;
   }
   if (nlaunch) *nlaunch += nl;

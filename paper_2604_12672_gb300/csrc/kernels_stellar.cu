@@ -23,7 +23,7 @@ __device__ __forceinline__ void mixture(const DevGeo &G, const double *u, double
       sa = fma(u[l], G.iAcomp[l], sa);
       sz = fma(u[l], G.ZoAcomp[l], sz);
     }
-  is = eos::rcp_nr(s);
+  is = rcp_nr(s);
   iabar = sa * is;
   ye = sz * is;
 }
@@ -58,7 +58,7 @@ __device__ __forceinline__ CellState cell_state(const DevGeo &G, long p, const d
     bh[2] += f2d_scaled(dB[2 * pl + p + G.sz], k);
   }
   c.rho = u[0];
-  const double ir = eos::rcp_nr(c.rho);   // one reciprocal for the cell
+  const double ir = rcp_nr(c.rho);   // one reciprocal for the cell
   c.irho = ir;
   c.v[0] = u[1] * ir; c.v[1] = u[2] * ir; c.v[2] = u[3] * ir;
   c.b2[0] = bl[0] + bh[0]; c.b2[1] = bl[1] + bh[1]; c.b2[2] = bl[2] + bh[2];

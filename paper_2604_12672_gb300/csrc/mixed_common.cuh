@@ -293,12 +293,10 @@ __device__ __forceinline__ void k_update_cells_mx_at(long tl, const DevGeo &G, c
 }
 
 template <int D>
-__device__ __forceinline__ void k_update_faces_mx_at(long tl, const DevGeo &G, const Box &box, StageMx S) {
+__device__ __forceinline__ void face_update_mx(const DevGeo &G, const int *c, const StageMx &S) {
   constexpr int A = (D + 1) % 3, B = (D + 2) % 3;
   const float dt = d2f_scaled(*S.dt, -G.e_t);
   {
-    int c[3];
-    if (!cell_at(box, tl, c)) return;
     int e[3] = {c[0], c[1], c[2]};
     if (!G.act[D]) e[D] = 0;
     const long p = widx(G, e[0], e[1], e[2]);
@@ -314,6 +312,12 @@ __device__ __forceinline__ void k_update_faces_mx_at(long tl, const DevGeo &G, c
   }
 }
 
+
+template <int D>
+__device__ __forceinline__ void k_update_faces_mx_at(long tl, const DevGeo &G, const Box &box, StageMx S) {
+  int c[3];
+  if (cell_at(box, tl, c)) face_update_mx<D>(G, c, S);
+}
 
 // CFL rate of one interior cell of U^n, in scaled units.
 __device__ __forceinline__ float dt_rate_mx(const DevGeo &G, const double *__restrict__ U,

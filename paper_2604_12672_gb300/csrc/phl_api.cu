@@ -293,7 +293,7 @@ void do_stage(phl_grid *g, const double *Uin, const double *Bin, double *Uout, d
   S.Uin = Uin; S.Bin = Bin; S.Ubase = g->U; S.Bbase = g->B;
   S.Uout = Uout; S.Bout = Bout; S.a = a; S.b = b; S.dt = g->dt;
   S.W = g->W; S.F[0] = g->F[0]; S.F[1] = g->F[1]; S.F[2] = g->F[2]; S.E = g->E;
-  S.raw = g->raw; S.flag = g->flag; S.Tin = g->T; S.Tout = g->T2; S.dflag = g->dflag;
+  S.raw = g->raw; S.flag = g->flag; S.any = g->anyraw; S.Tin = g->T; S.Tout = g->T2; S.dflag = g->dflag;
   launch_stage_fp64(g->G, S, g->stream, nl, g->prof.on ? &g->prof : nullptr);
   if (g->T) std::swap(g->T, g->T2);   // this stage's temperatures are the next guesses
 }
@@ -393,6 +393,7 @@ phl_status phl_create_grid(const phl_grid_desc *d, phl_grid **out) {
   G.nf = 8 + d->nspec;
   G.eos = d->eos;
   G.gamma = d->gamma;
+  G.igm1 = 1.0 / (d->gamma - 1.0);
   G.riemann = d->riemann;
   G.recon = d->recon;
   G.eps_sf = d->eps_sf;
@@ -703,16 +704,17 @@ phl_status phl_step(phl_grid *g, double dt, int nsteps) {
         launch_set_scalar(g->dt, dt, g->stream, g->prof.on ? &g->prof : nullptr);
         ++nl;
       }
-    } else if (g->G.eos != PHL_EOS_STELLAR && !(g->mixed && !three)) {
+    } else if (three) {
       launch_dt(g, &nl);
-      if (three) CK(cudaMemsetAsync(g->fmax, 0, sizeof(unsigned int), g->stream), "clear CFL maximum");
+      CK(cudaMemsetAsync(g->fmax, 0, sizeof(unsigned int), g->stream), "clear CFL maximum");
     }
     // ideal-gas mixed form (six launches per stage) with the device CFL step:
     // the first stage's primitives of U^n give it
     unsigned int *cfl_fmax = (g->mixed && !three && g->G.eos != PHL_EOS_STELLAR && !(dt > 0.0)) ? g->fmax + 1
                                                                                                  : nullptr;
-    // stellar EOS with the device CFL step: the first stage's inversion gives it
-    unsigned long long *cfl_dmax = (g->G.eos == PHL_EOS_STELLAR && !(dt > 0.0)) ? g->dmax : nullptr;
+    // stellar EOS and FP64 form with the device CFL step: the first stage's
+    // inversion or primitives give it
+    unsigned long long *cfl_dmax = ((g->G.eos == PHL_EOS_STELLAR || !g->mixed) && !(dt > 0.0)) ? g->dmax : nullptr;
     if (g->mixed) {
       const double bs3[3] = {1.0, 0.25, 2.0 / 3.0}, bs2[2] = {1.0, 0.5};
       const int ns = g->desc.rk == 2 ? 2 : 3;

@@ -49,7 +49,7 @@ struct DevGeo {
   double dx[3], idx[3];
   int nspec, nv, nw, nf;
   int eos;
-  double gamma;
+  double gamma, igm1;          // gamma, 1/(gamma - 1)
   int has_bg;
   const double *bg_rho_c, *bg_p_c, *bg_rho_f, *bg_p_f;   // device profiles
   const double *bg_ge_c, *bg_gc_c, *bg_ge_f, *bg_gc_f;   // may be null
@@ -283,7 +283,8 @@ struct StageBufs {
   const double *Tin;           // temperature guesses (stellar), state layout
   double *Tout;                // temperatures found by this stage
   int *dflag;                  // device error word
-  unsigned long long *cfl_dmax = nullptr;   // stellar: the CFL step from this stage's inversion into dt
+  unsigned long long *cfl_dmax = nullptr;   // the CFL step from this stage's primitives into dt
+  unsigned int *any = nullptr; // the raw-flag kernel's vote
 };
 
 // Buffers of the mixed-precision stage (kernels_mixed.cu): FP64 U^n, FP32
@@ -313,8 +314,7 @@ struct MixedBufs {
   // ideal gas, device CFL step: the first stage's primitives of U^n also
   // fold the CFL rate into this maximum and set dt (no separate CFL pass)
   unsigned int *cfl_fmax = nullptr;
-  // fused six-launch path: the raw-flag kernel's "some cell is flagged" vote
-  // (zeroed before it); null = always dilate and load the flags
+  // the raw-flag kernel's "some cell is flagged" vote (zeroed before it)
   unsigned int *anyraw = nullptr;
 };
 void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nstages, double b, cudaStream_t s,

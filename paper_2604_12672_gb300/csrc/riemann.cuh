@@ -21,6 +21,8 @@
 //         normal-momentum flux and its pressure work in the energy flux take
 //         the scaled value.
 //   HLL   two-wave solver used on shock-flagged faces (Sect. 2.7).
+// The templates here serve the FP32 forms; riemann_dev<double> is in
+// riemann_fp64.cuh.
 // Species: mass fractions are rescaled by their sum (Sect. 2.9, consistent
 // multi-fluid advection) and advected with the mass flux of the side of the
 // contact the flux is taken from.
@@ -38,7 +40,6 @@ enum { RD_RHO = 0, RD_UN, RD_UT1, RD_UT2, RD_BT1, RD_BT2, RD_P, RD_GE, RD_GC, RD
 enum { RF_RHO = 0, RF_MN, RF_MT1, RF_MT2, RF_E, RF_BT1, RF_BT2, RF_X0 };
 enum { SOLVER_LHLLD = 0, SOLVER_HLLD = 1, SOLVER_HLL = 2 };
 
-__device__ __forceinline__ double rsqrt_t(double x) { return sqrt(x); }
 __device__ __forceinline__ float rsqrt_t(float x) { return sqrtf(x); }
 
 template <typename R>
@@ -150,6 +151,11 @@ __device__ __forceinline__ int contact_dir(R frho, R rhol, R rhor, R SL, R SR) {
   return frho > scale ? 1 : (frho < -scale ? -1 : 0);
 }
 
+template <int NS, bool IDEAL>
+__device__ __forceinline__ void riemann_fp64(const double *wl, const double *wr, double bn, double rh, double ph,
+                                             double geh, double gch, int nspec, int solver, double mthr, double *f,
+                                             int &up, const GasK<double> &K);
+
 // wl, wr: normal-frame deviation states (RD_* order) with nspec mass fractions.
 // Background at the face: rh, ph, geh, gch (all 0 without a background).
 // f: F - F_hat in RF_* order (7 + nspec values).
@@ -157,6 +163,9 @@ __device__ __forceinline__ int contact_dir(R frho, R rhol, R rhor, R SL, R SR) {
 template <typename R, int NS, bool IDEAL = false>
 __device__ __forceinline__ void riemann_dev(const R *wl, const R *wr, R bn, R rh, R ph, R geh, R gch, int nspec,
                                             int solver, R mthr, R *f, int &up, const GasK<R> &K = GasK<R>{}) {
+  if constexpr (sizeof(R) == 8) {
+    riemann_fp64<NS, IDEAL>(wl, wr, bn, rh, ph, geh, gch, nspec, solver, mthr, f, up, K);
+  } else {
   Side<R> L, R_;
   side_init<R, IDEAL>(L, wl, bn, rh, ph, geh, gch, K);
   side_init<R, IDEAL>(R_, wr, bn, rh, ph, geh, gch, K);
@@ -267,6 +276,9 @@ __device__ __forceinline__ void riemann_dev(const R *wl, const R *wr, R bn, R rh
   for (int l = 0; l < NS; ++l)
     if (l < nspec) f[RF_X0 + l] = F[RF_RHO] * (left ? xl[l] : xr[l]);
   up = contact_dir(F[RF_RHO], L.rho, R_.rho, SL, SR);
+  }
 }
 
 }  // namespace phl
+
+#include "riemann_fp64.cuh"

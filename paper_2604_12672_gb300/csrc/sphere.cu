@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, c
       rho += f2d_scaled(dU[c], 0); mx += f2d_scaled(dU[n + c], 0); my += f2d_scaled(dU[2 * n + c], 0);
       mz += f2d_scaled(dU[3 * n + c], 0); E += f2d_scaled(dU[4 * n + c], 0);
     }
-    const double ir = eos::rcp_nr(rho);
+    const double ir = rcp_nr(rho);
     const double ux = mx * ir, uy = my * ir, uz = mz * ir;
     const double eint = (E - 0.5 * (mx * ux + my * uy + mz * uz) - 0.5 * (bx * bx + by * by + bz * bz)) * ir;
     double T = D.T[c];

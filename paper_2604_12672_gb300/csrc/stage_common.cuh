@@ -78,7 +78,10 @@ template <typename R>
 __device__ __forceinline__ R vl_slope(R a, R b, R c) {
   const R dm = b - a, dp = c - b;
   if constexpr (sizeof(R) == 4) return (dm * dp > R(0)) ? __fdividef(R(2) * dm * dp, dm + dp) : R(0);
-  else return (dm * dp > R(0)) ? R(2) * dm * dp / (dm + dp) : R(0);
+  else {
+    const R pr = dm * dp;
+    return positive(pr) ? R(2) * pr * rcp_nr(dm + dp) : R(0);
+  }
 }
 
 // PPH (Sect. 2.5, item ii): the parabola whose averages over cells i-1, i,
@@ -237,11 +240,6 @@ __device__ __forceinline__ void k_dilate_axis_at(long tl, const DevGeo &G, const
     out[c[0] + (long)G.n[0] * (c[1] + (long)G.n[1] * c[2])] = f;
   }
 }
-template <int D>
-__global__ void k_dilate_axis(DevGeo G, Box box, const uint8_t *__restrict__ in, uint8_t *__restrict__ out) {
-  k_dilate_axis_at<D>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, in, out);
-}
-
 // Flags of the cells the face stencils touch ([-1, n] on active axes): a ghost
 // cell carries the flag of the interior cell its data comes from.
 __device__ __forceinline__ void k_flag_expand_at(long tl, const DevGeo &G, const Box &box, const uint8_t *__restrict__ dil, uint8_t *__restrict__ flag) {
@@ -255,30 +253,257 @@ __device__ __forceinline__ void k_flag_expand_at(long tl, const DevGeo &G, const
     flag[widx(G, c[0], c[1], c[2])] = dil[s[0] + (long)G.n[0] * (s[1] + (long)G.n[1] * s[2])];
   }
 }
-__global__ void k_flag_expand(DevGeo G, Box box, const uint8_t *__restrict__ dil, uint8_t *__restrict__ flag) {
-  k_flag_expand_at(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, dil, flag);
+constexpr int DF = 8, DH = DF + 2 * NGW;   // cells of a dilation tile and its staged rows along an axis
+
+// 5^3 dilation of the raw shock flags (Sect. 2.7) for one 8^3 tile of
+// interior cells in one pass, eight flags (one byte each) per 64-bit word: the
+// raw flags of x0-4 .. x0+11 for every row of the tile and its two neighbour
+// rows on each side are staged in shared memory as two words, then ORed along
+// x (byte shifts of the 16-byte window), y and z (word ORs) in turn -- the OR
+// over a box is the nested ORs over its axes.  Beyond a periodic boundary the
+// flags wrap; beyond any other boundary they count as unflagged.
+// The dilation of the tile at (x0, y0, z0) with the CTA's threads; r0, r1, r2:
+// shared scratch of DH DH 2, DH DH and DH DF words.
+__device__ __forceinline__ void dilate_tile(const DevGeo &G, const uint8_t *__restrict__ raw, uint8_t *__restrict__ dil,
+                                            int x0, int y0, int z0, unsigned long long (*r0)[2],
+                                            unsigned long long *r1, unsigned long long *r2) {
+  const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
+  const int xs = x0 - 4;
+  const bool wide = (nx % 8) == 0 && xs >= 0 && xs + 16 <= nx;   // aligned window inside the row
+  const bool px = G.bc[0][0] == 0, py = G.bc[1][0] == 0, pz = G.bc[2][0] == 0;
+  for (int q = threadIdx.x; q < DH * DH * 4; q += blockDim.x) {
+    const int w = q & 3, row = q >> 2;
+    int y = y0 - NGW + row % DH, z = z0 - NGW + row / DH;
+    bool in = true;
+    if (y < 0 || y >= ny) { if (py) y = (y % ny + ny) % ny; else in = false; }
+    if (z < 0 || z >= nz) { if (pz) z = (z % nz + nz) % nz; else in = false; }
+    unsigned v = 0u;
+    if (in) {
+      const uint8_t *rr = raw + (long)nx * (y + (long)ny * z);
+      if (wide) {
+        v = *reinterpret_cast<const unsigned *>(rr + xs + 4 * w);
+      } else {
+        for (int bb = 0; bb < 4; ++bb) {
+          int x = xs + 4 * w + bb;
+          bool ok = true;
+          if (x < 0 || x >= nx) { if (px) x = (x % nx + nx) % nx; else ok = false; }
+          if (ok) v |= (unsigned)rr[x] << (8 * bb);
+        }
+      }
+    }
+    reinterpret_cast<unsigned *>(&r0[row][0])[w] = v;
+  }
+  __syncthreads();
+  for (int row = threadIdx.x; row < DH * DH; row += blockDim.x) {
+    // output byte j (x = x0 + j) ORs window bytes j+2 .. j+6
+    const unsigned long long lo = r0[row][0], hi = r0[row][1];
+    unsigned long long o = 0ull;
+#pragma unroll
+    for (int sh = 2; sh <= 6; ++sh) o |= (lo >> (8 * sh)) | (hi << (64 - 8 * sh));
+    r1[row] = o;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < DH * DF; q += blockDim.x) {
+    const int y = q % DF, z = q / DF;
+    const unsigned long long *c = &r1[z * DH + y];
+    r2[q] = c[0] | c[1] | c[2] | c[3] | c[4];
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < DF * DF; q += blockDim.x) {
+    const int y = q % DF, z = q / DF;
+    const int c1 = y0 + y, c2 = z0 + z;
+    if (c1 >= ny || c2 >= nz) continue;
+    const unsigned long long o = r2[z * DF + y] | r2[(z + 1) * DF + y] | r2[(z + 2) * DF + y] |
+                                 r2[(z + 3) * DF + y] | r2[(z + 4) * DF + y];
+    uint8_t *d = dil + x0 + (long)nx * (c1 + (long)ny * c2);
+    if ((nx % 8) == 0 && x0 + 8 <= nx) {
+      *reinterpret_cast<unsigned long long *>(d) = o;
+    } else {
+      for (int j = 0; j < 8 && x0 + j < nx; ++j) d[j] = (uint8_t)(o >> (8 * j));
+    }
+  }
 }
 
-// raw -> dilated (interior) -> flags on the work layout; tmp: one interior byte field.
-inline int launch_flags(const DevGeo &G, uint8_t *raw, uint8_t *tmp, uint8_t *flag, cudaStream_t s, Prof *prof) {
-  Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-  uint8_t *a = raw, *b = tmp;
-  int nl = 0;
-  for (int D = 0; D < 3; ++D) {
-    if (!G.act[D]) continue;
-    if (D == 0) PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_dilate_axis<0><<<grid3(bi), block3(bi), 0, s>>>(G, bi, a, b));
-    if (D == 1) PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_dilate_axis<1><<<grid3(bi), block3(bi), 0, s>>>(G, bi, a, b));
-    if (D == 2) PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_dilate_axis<2><<<grid3(bi), block3(bi), 0, s>>>(G, bi, a, b));
-    uint8_t *t = a; a = b; b = t;
-    ++nl;
+// any (optional): the raw-flag kernel's vote; zero means no cell is flagged,
+// the dilation is all zero and the tile kernel, reading the same vote, loads
+// none of it -- nothing is written.
+__global__ void __launch_bounds__(256) k_flag_dilate3(DevGeo G, const uint8_t *__restrict__ raw,
+                                                     uint8_t *__restrict__ dil, int ntx, int nty,
+                                                     const unsigned int *__restrict__ any) {
+  __shared__ unsigned long long r0[DH * DH][2];
+  __shared__ unsigned long long r1[DH * DH], r2[DH * DF];
+  if (any && *any == 0u) return;
+  const int nb = ntx * nty * ((G.n[2] + DF - 1) / DF);
+  for (int t0 = blockIdx.x; t0 < nb; t0 += gridDim.x) {   // the block's tiles; the grid fills the SMs once
+    int t = t0;
+    const int tx = t % ntx;
+    t /= ntx;
+    const int ty = t % nty, tz = t / nty;
+    dilate_tile(G, raw, dil, tx * DF, ty * DF, tz * DF, r0, r1, r2);
   }
+}
+
+// The dilated flags expanded onto the work layout's cells [-1, n]; zeros where
+// no cell is flagged (*any == 0).
+__global__ void __launch_bounds__(256) k_flag_expand(DevGeo G, Box box, const uint8_t *__restrict__ dil,
+                                                     uint8_t *__restrict__ flag, const unsigned int *__restrict__ any) {
+  const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (*any == 0u) {
+    int c[3];
+    if (cell_at(box, t, c)) flag[widx(G, c[0], c[1], c[2])] = 0;
+    return;
+  }
+  k_flag_expand_at(t, G, box, dil, flag);
+}
+
+// The dilation and its expansion in one pass, for grids with at most two
+// active dimensions: each cell ORs the raw flags (5 or 25) around the interior
+// cell its data comes from.  In three dimensions the 125 loads per cell cost
+// more than the tiled dilation and a second pass (249 against 30 us on the
+// stellar box at 128^3); in two, one launch is saved.
+__global__ void __launch_bounds__(256) k_flag_box(DevGeo G, Box box, const uint8_t *__restrict__ raw,
+                                                  uint8_t *__restrict__ flag, const unsigned int *__restrict__ any) {
+  int c[3], s[3];
+  if (!cell3(box, c)) return;
+  const long q = widx(G, c[0], c[1], c[2]);
+  if (*any == 0u) { flag[q] = 0; return; }
+  for (int d = 0; d < 3; ++d) {
+    bool fl;
+    s[d] = G.act[d] ? cell_src(c[d], G.n[d], G.bc[d][0], G.bc[d][1], fl) : 0;
+  }
+  const int r[3] = {G.act[0] ? 2 : 0, G.act[1] ? 2 : 0, G.act[2] ? 2 : 0};
+  auto nb = [&](int d, int x) {   // neighbour x along axis d: wrapped, or -1 beyond a side that is not periodic
+    if (x >= 0 && x < G.n[d]) return x;
+    return G.bc[d][0] == 0 ? (x + G.n[d]) % G.n[d] : -1;
+  };
+  uint8_t f = 0;
+  for (int dz = -r[2]; dz <= r[2]; ++dz) {
+    const int z = nb(2, s[2] + dz);
+    if (z < 0) continue;
+    for (int dy = -r[1]; dy <= r[1]; ++dy) {
+      const int y = nb(1, s[1] + dy);
+      if (y < 0) continue;
+      const uint8_t *row = raw + (long)G.n[0] * (y + (long)G.n[1] * z);
+      for (int dx = -r[0]; dx <= r[0]; ++dx) {
+        const int x = nb(0, s[0] + dx);
+        if (x >= 0) f |= row[x];
+      }
+    }
+  }
+  flag[q] = f;
+}
+
+// Block size of the one-thread-per-element kernels: 256, or 64 where 256
+// would leave SMs without a block (the FP64 kernels of a 128^2 grid: 65 blocks
+// on 152 SMs, each SM's FP64 pipe serving eight warps while others idle).
+inline unsigned tpb_for(long n) { return n < 2L * 152 * 256 ? 64u : 256u; }
+inline dim3 gridt(const Box &b, unsigned t) { return dim3((unsigned)((b.n + t - 1) / t), 1, 1); }
+
+// Raw flags (W holds the stage input), then the flags of the cells the face
+// stencils touch; tmp: one interior byte field, any: one device word.  Returns
+// the launches.
+template <typename R>
+inline int launch_flags(const DevGeo &G, const R *W, uint8_t *raw, uint8_t *tmp, uint8_t *flag, unsigned int *any, cudaStream_t s,
+                        Prof *prof) {
+  Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
+  cudaMemsetAsync(any, 0, sizeof(unsigned int), s);
+  const unsigned t = tpb_for(bi.n);
+  PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw<R><<<gridt(bi, t), t, 0, s>>>(G, bi, W, raw, any));
   int l[3], h[3];
   for (int d = 0; d < 3; ++d) {
     if (G.act[d]) { l[d] = -1; h[d] = G.n[d] + 1; } else { l[d] = 0; h[d] = 1; }
   }
   Box be = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
-  PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_flag_expand<<<grid3(be), block3(be), 0, s>>>(G, be, a, flag));
-  return nl + 1;
+  if (!(G.act[0] && G.act[1] && G.act[2])) {
+    PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_flag_box<<<gridt(be, 256), 256, 0, s>>>(G, be, raw, flag, any));
+    return 2;
+  }
+  const int ntx = (G.n[0] + DF - 1) / DF, nty = (G.n[1] + DF - 1) / DF, ntz = (G.n[2] + DF - 1) / DF;
+  const long nt = (long)ntx * nty * ntz;
+  PHL_LAUNCH(KC_FLAG_DILATE, prof, s,
+             k_flag_dilate3<<<(unsigned)(nt < 8L * 152 ? nt : 8L * 152), 256, 0, s>>>(G, raw, tmp, ntx, nty, any));
+  PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_flag_expand<<<gridt(be, 256), 256, 0, s>>>(G, be, tmp, flag, any));
+  return 3;
+}
+
+// The flux of the D-face of work cell c (index pR) from its reconstructed
+// left and right states: F - F_hat and the contact direction into F.
+template <int D, typename R, int NS>
+__device__ __forceinline__ void flux_finish(const DevGeo &G, const int *c, long pR, R *ql, R *qr,
+                                            const double *__restrict__ Bf, const R *__restrict__ dB,
+                                            const uint8_t *__restrict__ flag, R *__restrict__ F, int *dflag) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  const long pL = pR - wstride(G, D);
+  constexpr int NWC = W_X0 + NS;   // components this instantiation can hold
+  R wl[NWC], wr[NWC];
+  const bool ideal = G.eos == 0;
+  if (ideal) {   // not used by the ideal-gas solver (constant gamma)
+    ql[W_GE] = qr[W_GE] = R(0);
+    ql[W_GC] = qr[W_GC] = R(0);
+  }
+  wl[RD_RHO] = ql[W_RHO];        wr[RD_RHO] = qr[W_RHO];
+  wl[RD_UN] = ql[W_VX + D];      wr[RD_UN] = qr[W_VX + D];
+  wl[RD_UT1] = ql[W_VX + T1];    wr[RD_UT1] = qr[W_VX + T1];
+  wl[RD_UT2] = ql[W_VX + T2];    wr[RD_UT2] = qr[W_VX + T2];
+  wl[RD_BT1] = ql[W_BX + T1];    wr[RD_BT1] = qr[W_BX + T1];
+  wl[RD_BT2] = ql[W_BX + T2];    wr[RD_BT2] = qr[W_BX + T2];
+  wl[RD_P] = ql[W_P];            wr[RD_P] = qr[W_P];
+  wl[RD_GE] = ql[W_GE];          wr[RD_GE] = qr[W_GE];
+  wl[RD_GC] = ql[W_GC];          wr[RD_GC] = qr[W_GC];
+#pragma unroll
+  for (int l = 0; l < NS; ++l)
+    if (l < G.nspec) { wl[RD_X0 + l] = ql[W_X0 + l]; wr[RD_X0 + l] = qr[W_X0 + l]; }
+  const BgT<R> bf = (D == 2) ? bg_zface_t<R>(G, c[2]) : bg_cell_t<R>(G, c[2]);
+  if (!(positive(bf.rho + wl[RD_RHO]) && positive(bf.rho + wr[RD_RHO]) && positive(bf.p + wl[RD_P]) &&
+        positive(bf.p + wr[RD_P])))
+    atomicOr(dflag, FLAG_NEG);
+  // normal field on this face; transverse ghost rows map to their source rows
+  int s[3];
+  s[D] = c[D];
+  {
+    bool fl;
+    s[T1] = G.act[T1] ? cell_src(c[T1], G.n[T1], G.bc[T1][0], G.bc[T1][1], fl) : 0;
+    s[T2] = G.act[T2] ? cell_src(c[T2], G.n[T2], G.bc[T2][0], G.bc[T2][1], fl) : 0;
+  }
+  const long qb = (long)D * G.plane + sidx(G, s[0], s[1], s[2]);
+  R bn;
+  if constexpr (sizeof(R) == 4) {   // B^n + dB in scaled units
+    const float b0 = d2f_scaled(Bf[qb], -G.e_b);
+    bn = dB ? b0 + dB[qb] : b0;
+  }
+  else bn = (R)Bf[qb];
+  const int solver = (flag[pL] | flag[pR]) ? SOLVER_HLL : G.riemann;
+  R f[7 + NS];
+  int up;
+  if (G.eos == 0) {   // ideal gas: gamma constant
+    GasK<R> K;
+    K.g = sizeof(R) == 4 ? (R)G.gammaf : (R)G.gamma;
+    K.igm1 = sizeof(R) == 4 ? R(1) / (K.g - R(1)) : (R)G.igm1;
+    K.ggm1 = K.g * K.igm1;
+    riemann_dev<R, NS, true>(wl, wr, bn, bf.rho, bf.p, bf.ge, bf.gc, G.nspec, solver, mach_thr_t<R>(G), f, up, K);
+  } else {
+    riemann_dev<R, NS, false>(wl, wr, bn, bf.rho, bf.p, bf.ge, bf.gc, G.nspec, solver, mach_thr_t<R>(G), f, up);
+  }
+  // reflecting wall face: a symmetry plane (Table bcs, u_n = 0, B_n = 0); only
+  // the normal-momentum flux survives, the others are exactly zero
+  if ((c[D] == 0 && G.bc[D][0] == 1) || (c[D] == G.n[D] && G.bc[D][1] == 1)) {
+#pragma unroll
+    for (int q = 0; q < 7 + NS; ++q)
+      if (q != RF_MN) f[q] = R(0);
+    up = 0;
+  }
+  const long wt = G.wtot;
+  F[F_RHO * wt + pR] = f[RF_RHO];
+  F[(F_MX + D) * wt + pR] = f[RF_MN];
+  F[(F_MX + T1) * wt + pR] = f[RF_MT1];
+  F[(F_MX + T2) * wt + pR] = f[RF_MT2];
+  F[F_E * wt + pR] = f[RF_E];
+  F[(F_BX + T1) * wt + pR] = f[RF_BT1];
+  F[(F_BX + T2) * wt + pR] = f[RF_BT2];
+#pragma unroll
+  for (int l = 0; l < NS; ++l)
+    if (l < G.nspec) F[(F_X0 + l) * wt + pR] = f[RF_X0 + l];
+  F[(long)G.nf * wt + pR] = (R)up;   // contact direction for Contact-CT
 }
 
 // Flux at the D-face of work cell c (index pR, left neighbour pR - sd).
@@ -288,11 +513,9 @@ template <int D, typename R, int NS, typename Fetch>
 __device__ __forceinline__ void flux_face(const DevGeo &G, const int *c, long pR, Fetch fetch,
                                           const double *__restrict__ Bf, const R *__restrict__ dB,
                                           const uint8_t *__restrict__ flag, R *__restrict__ F, int *dflag) {
-  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   const long sd = wstride(G, D);
   const long pL = pR - sd;
   constexpr int NWC = W_X0 + NS;   // components this instantiation can hold
-  R wl[NWC], wr[NWC];
   const bool ideal = G.eos == 0;   // ideal gas: gamma_e = gamma_c = gamma (not reconstructed)
   // shock flattening (Sect. 2.7): a flagged cell reconstructs with van Leer
   const bool vlL = G.recon == PHL_RECON_VANLEER || flag[pL], vlR = G.recon == PHL_RECON_VANLEER || flag[pR];
@@ -324,73 +547,7 @@ __device__ __forceinline__ void flux_face(const DevGeo &G, const int *c, long pR
       qr[v] = w2 - R(0.5) * vl_slope(w1, w2, w3);
     }
   }
-  if (ideal) {   // not used by the ideal-gas solver (constant gamma)
-    ql[W_GE] = qr[W_GE] = R(0);
-    ql[W_GC] = qr[W_GC] = R(0);
-  }
-  wl[RD_RHO] = ql[W_RHO];        wr[RD_RHO] = qr[W_RHO];
-  wl[RD_UN] = ql[W_VX + D];      wr[RD_UN] = qr[W_VX + D];
-  wl[RD_UT1] = ql[W_VX + T1];    wr[RD_UT1] = qr[W_VX + T1];
-  wl[RD_UT2] = ql[W_VX + T2];    wr[RD_UT2] = qr[W_VX + T2];
-  wl[RD_BT1] = ql[W_BX + T1];    wr[RD_BT1] = qr[W_BX + T1];
-  wl[RD_BT2] = ql[W_BX + T2];    wr[RD_BT2] = qr[W_BX + T2];
-  wl[RD_P] = ql[W_P];            wr[RD_P] = qr[W_P];
-  wl[RD_GE] = ql[W_GE];          wr[RD_GE] = qr[W_GE];
-  wl[RD_GC] = ql[W_GC];          wr[RD_GC] = qr[W_GC];
-#pragma unroll
-  for (int l = 0; l < NS; ++l)
-    if (l < G.nspec) { wl[RD_X0 + l] = ql[W_X0 + l]; wr[RD_X0 + l] = qr[W_X0 + l]; }
-  const BgT<R> bf = (D == 2) ? bg_zface_t<R>(G, c[2]) : bg_cell_t<R>(G, c[2]);
-  if (!(bf.rho + wl[RD_RHO] > R(0) && bf.rho + wr[RD_RHO] > R(0) && bf.p + wl[RD_P] > R(0) &&
-        bf.p + wr[RD_P] > R(0)))
-    atomicOr(dflag, FLAG_NEG);
-  // normal field on this face; transverse ghost rows map to their source rows
-  int s[3];
-  s[D] = c[D];
-  {
-    bool fl;
-    s[T1] = G.act[T1] ? cell_src(c[T1], G.n[T1], G.bc[T1][0], G.bc[T1][1], fl) : 0;
-    s[T2] = G.act[T2] ? cell_src(c[T2], G.n[T2], G.bc[T2][0], G.bc[T2][1], fl) : 0;
-  }
-  const long qb = (long)D * G.plane + sidx(G, s[0], s[1], s[2]);
-  R bn;
-  if constexpr (sizeof(R) == 4) {   // B^n + dB in scaled units
-    const float b0 = d2f_scaled(Bf[qb], -G.e_b);
-    bn = dB ? b0 + dB[qb] : b0;
-  }
-  else bn = (R)Bf[qb];
-  const int solver = (flag[pL] | flag[pR]) ? SOLVER_HLL : G.riemann;
-  R f[7 + NS];
-  int up;
-  if (G.eos == 0) {   // ideal gas: gamma constant
-    GasK<R> K;
-    K.g = sizeof(R) == 4 ? (R)G.gammaf : (R)G.gamma;
-    K.igm1 = R(1) / (K.g - R(1));
-    K.ggm1 = K.g * K.igm1;
-    riemann_dev<R, NS, true>(wl, wr, bn, bf.rho, bf.p, bf.ge, bf.gc, G.nspec, solver, mach_thr_t<R>(G), f, up, K);
-  } else {
-    riemann_dev<R, NS, false>(wl, wr, bn, bf.rho, bf.p, bf.ge, bf.gc, G.nspec, solver, mach_thr_t<R>(G), f, up);
-  }
-  // reflecting wall face: a symmetry plane (Table bcs, u_n = 0, B_n = 0); only
-  // the normal-momentum flux survives, the others are exactly zero
-  if ((c[D] == 0 && G.bc[D][0] == 1) || (c[D] == G.n[D] && G.bc[D][1] == 1)) {
-#pragma unroll
-    for (int q = 0; q < 7 + NS; ++q)
-      if (q != RF_MN) f[q] = R(0);
-    up = 0;
-  }
-  const long wt = G.wtot;
-  F[F_RHO * wt + pR] = f[RF_RHO];
-  F[(F_MX + D) * wt + pR] = f[RF_MN];
-  F[(F_MX + T1) * wt + pR] = f[RF_MT1];
-  F[(F_MX + T2) * wt + pR] = f[RF_MT2];
-  F[F_E * wt + pR] = f[RF_E];
-  F[(F_BX + T1) * wt + pR] = f[RF_BT1];
-  F[(F_BX + T2) * wt + pR] = f[RF_BT2];
-#pragma unroll
-  for (int l = 0; l < NS; ++l)
-    if (l < G.nspec) F[(F_X0 + l) * wt + pR] = f[RF_X0 + l];
-  F[(long)G.nf * wt + pR] = (R)up;   // contact direction for Contact-CT
+  flux_finish<D, R, NS>(G, c, pR, ql, qr, Bf, dB, flag, F, dflag);
 }
 
 template <int D, typename R, int NS>
@@ -412,14 +569,57 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_flux(DevGeo G, 
   k_flux_at<D, R, NS>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, W, Bf, dB, flag, F, dflag);
 }
 
+// van Leer faces, `step` consecutive D-faces per thread: a cell's slope gives
+// its right face value to one face and its left one to the next, so a thread
+// that walks along D forms step + 1 slopes for step faces instead of 2 step.
+// In the FP64 form the slopes are a fifth of the face's FP64 instructions.
+// box: the faces with the D extent divided by step (rounded up); nD: number
+// of D-faces.
+template <int D, typename R, int NS>
+__global__ void __launch_bounds__(128, NS ? 3 : 4)
+    k_flux_walk(DevGeo G, Box box, int nD, int step, const R *__restrict__ W, const double *__restrict__ Bf,
+                const R *__restrict__ dB, const uint8_t *__restrict__ flag, R *__restrict__ F, int *dflag) {
+  int c[3];
+  if (!cell3(box, c)) return;
+  c[D] *= step;
+  const long sd = wstride(G, D);
+  constexpr int NWC = W_X0 + NS;
+  const bool ideal = G.eos == 0;
+  long p = widx(G, c[0], c[1], c[2]);
+  auto used = [&](int v) { return v < G.nw && !(ideal && (v == W_GE || v == W_GC)) && v != W_BX + D; };
+  R ql[NWC];
+#pragma unroll
+  for (int v = 0; v < NWC; ++v) {
+    if (!used(v)) continue;
+    const long q = p - 2 * sd;
+    const R w0 = W[wix<R>(G, v, q)], w1 = W[wix<R>(G, v, q + sd)], w2 = W[wix<R>(G, v, q + 2 * sd)];
+    ql[v] = w1 + R(0.5) * vl_slope(w0, w1, w2);
+  }
+#pragma unroll 1
+  for (int k = 0; k < step && c[D] < nD; ++k, ++c[D], p += sd) {
+    R qr[NWC], qn[NWC];
+#pragma unroll
+    for (int v = 0; v < NWC; ++v) {
+      if (!used(v)) continue;
+      const R w0 = W[wix<R>(G, v, p - sd)], w1 = W[wix<R>(G, v, p)], w2 = W[wix<R>(G, v, p + sd)];
+      const R sl = vl_slope(w0, w1, w2);
+      qr[v] = w1 - R(0.5) * sl;
+      qn[v] = w1 + R(0.5) * sl;
+    }
+    ql[W_BX + D] = qr[W_BX + D] = R(0);   // the normal field is not reconstructed
+    flux_finish<D, R, NS>(G, c, p, ql, qr, Bf, dB, flag, F, dflag);
+#pragma unroll
+    for (int v = 0; v < NWC; ++v)
+      if (used(v)) ql[v] = qn[v];
+  }
+}
+
 // Edge EMF along D at the lower corner (a-1/2, b-1/2), (D, A, B) cyclic.
 template <int D, typename R>
-__device__ __forceinline__ void k_emf_at(long tl, const DevGeo &G, const Box &box, const R *__restrict__ W, const R *__restrict__ FA,
-                      const R *__restrict__ FB, R *__restrict__ E) {
+__device__ __forceinline__ void emf_site(const DevGeo &G, const int *c, const R *__restrict__ W, const R *__restrict__ FA,
+                                         const R *__restrict__ FB, R *__restrict__ E) {
   constexpr int A = (D + 1) % 3, B = (D + 2) % 3;
   {
-    int c[3];
-    if (!cell_at(box, tl, c)) return;
     const long p = widx(G, c[0], c[1], c[2]);
     const long wt = G.wtot;
     R e;
@@ -464,17 +664,56 @@ __device__ __forceinline__ void k_emf_at(long tl, const DevGeo &G, const Box &bo
   }
 }
 template <int D, typename R>
-__global__ void k_emf(DevGeo G, Box box, const R *__restrict__ W, const R *__restrict__ FA,
+__device__ __forceinline__ void k_emf_at(long tl, const DevGeo &G, const Box &box, const R *__restrict__ W, const R *__restrict__ FA,
                       const R *__restrict__ FB, R *__restrict__ E) {
-  k_emf_at<D, R>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, W, FA, FB, E);
+  int c[3];
+  if (cell_at(box, tl, c)) emf_site<D, R>(G, c, W, FA, FB, E);
 }
 
+// All edge directions of a site in one launch (box: [0, n] along active axes).
+template <typename R>
+__global__ void k_emf_all(DevGeo G, Box box, const R *__restrict__ W, const R *__restrict__ F0,
+                          const R *__restrict__ F1, const R *__restrict__ F2, R *__restrict__ E) {
+  int c[3];
+  if (!cell3(box, c)) return;
+  if (c[0] < G.n[0] && (G.act[1] || G.act[2])) emf_site<0, R>(G, c, W, F1, F2, E);
+  if (c[1] < G.n[1] && (G.act[2] || G.act[0])) emf_site<1, R>(G, c, W, F2, F0, E);
+  if (c[2] < G.n[2] && (G.act[0] || G.act[1])) emf_site<2, R>(G, c, W, F0, F1, E);
+}
+inline Box site_box(const DevGeo &G) {
+  return make_box(0, G.act[0] ? G.n[0] + 1 : 1, 0, G.act[1] ? G.n[1] + 1 : 1, 0, G.act[2] ? G.n[2] + 1 : 1);
+}
 
 // Launch of k_flux<D, R, NS> with NS = 0 (no mass fractions) or PHL_NSPEC_MAX.
 template <typename R>
 inline void launch_flux(int D, const DevGeo &G, const Box &b, const R *W, const double *Bf, const R *dB,
                         const uint8_t *flag, R *F, int *dflag, cudaStream_t s, Prof *prof) {
   const int kc = D == 0 ? KC_FLUX_X : (D == 1 ? KC_FLUX_Y : KC_FLUX_Z);
+  // walks in the FP64 form only: FP32 faces are not bound by the slopes'
+  // arithmetic, and strided loads cost more there (stellar box 128^3: 129-172
+  // us a direction walking, 101-111 one face per thread)
+  if (sizeof(R) == 8 && G.recon == PHL_RECON_VANLEER) {
+    // faces per thread: as many as leave several blocks per SM
+    const int step = b.n >= 600000 ? 4 : (b.n >= 150000 ? 2 : 1);
+    const int nD = b.hi[D];
+    int h[3] = {b.hi[0], b.hi[1], b.hi[2]};
+    h[D] = (nD + step - 1) / step;
+    const Box bw = make_box(b.lo[0], h[0], b.lo[1], h[1], b.lo[2], h[2]);
+    const unsigned t = bw.n < 152L * 128 ? 32u : (bw.n < 4L * 152 * 128 ? 64u : 128u);
+#define PHL_FLUX(DD, NN) \
+  PHL_LAUNCH(kc, prof, s, (k_flux_walk<DD, R, NN><<<gridt(bw, t), t, 0, s>>>(G, bw, nD, step, W, Bf, dB, flag, F, dflag)))
+    if (G.nspec == 0) {
+      if (D == 0) PHL_FLUX(0, 0);
+      if (D == 1) PHL_FLUX(1, 0);
+      if (D == 2) PHL_FLUX(2, 0);
+    } else {
+      if (D == 0) PHL_FLUX(0, PHL_NSPEC_MAX);
+      if (D == 1) PHL_FLUX(1, PHL_NSPEC_MAX);
+      if (D == 2) PHL_FLUX(2, PHL_NSPEC_MAX);
+    }
+#undef PHL_FLUX
+    return;
+  }
   const dim3 gr = grid3(b), bl = block3(b);
 #define PHL_FLUX(DD, NN) PHL_LAUNCH(kc, prof, s, (k_flux<DD, R, NN><<<gr, bl, 0, s>>>(G, b, W, Bf, dB, flag, F, dflag)))
   if (G.nspec == 0) {

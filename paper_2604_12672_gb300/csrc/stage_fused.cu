@@ -663,94 +663,6 @@ __global__ void __launch_bounds__(NT, MINB)
                                          raw_flags, sm, 0u);
 }
 
-// 5^3 dilation of the raw shock flags (Sect. 2.7) for one 8^3 tile of
-// interior cells in one pass, eight flags (one byte each) per 64-bit word: the
-// raw flags of x0-4 .. x0+11 for every row of the tile and its two neighbour
-// rows on each side are staged in shared memory as two words, then ORed along
-// x (byte shifts of the 16-byte window), y and z (word ORs) in turn -- the OR
-// over a box is the nested ORs over its axes.  Beyond a periodic boundary the
-// flags wrap; beyond any other boundary they count as unflagged.
-// The dilation of the tile at (x0, y0, z0) with the CTA's threads; r0, r1, r2:
-// shared scratch of HZ HY 2, HZ HY and HZ FY words.
-__device__ __forceinline__ void dilate_tile(const DevGeo &G, const uint8_t *__restrict__ raw, uint8_t *__restrict__ dil,
-                                            int x0, int y0, int z0, unsigned long long (*r0)[2],
-                                            unsigned long long *r1, unsigned long long *r2) {
-  const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
-  const int xs = x0 - 4;
-  const bool wide = (nx % 8) == 0 && xs >= 0 && xs + 16 <= nx;   // aligned window inside the row
-  const bool px = G.bc[0][0] == 0, py = G.bc[1][0] == 0, pz = G.bc[2][0] == 0;
-  for (int q = threadIdx.x; q < HZ * HY * 4; q += blockDim.x) {
-    const int w = q & 3, row = q >> 2;
-    int y = y0 - NGW + row % HY, z = z0 - NGW + row / HY;
-    bool in = true;
-    if (y < 0 || y >= ny) { if (py) y = (y % ny + ny) % ny; else in = false; }
-    if (z < 0 || z >= nz) { if (pz) z = (z % nz + nz) % nz; else in = false; }
-    unsigned v = 0u;
-    if (in) {
-      const uint8_t *rr = raw + (long)nx * (y + (long)ny * z);
-      if (wide) {
-        v = *reinterpret_cast<const unsigned *>(rr + xs + 4 * w);
-      } else {
-        for (int bb = 0; bb < 4; ++bb) {
-          int x = xs + 4 * w + bb;
-          bool ok = true;
-          if (x < 0 || x >= nx) { if (px) x = (x % nx + nx) % nx; else ok = false; }
-          if (ok) v |= (unsigned)rr[x] << (8 * bb);
-        }
-      }
-    }
-    reinterpret_cast<unsigned *>(&r0[row][0])[w] = v;
-  }
-  __syncthreads();
-  for (int row = threadIdx.x; row < HZ * HY; row += blockDim.x) {
-    // output byte j (x = x0 + j) ORs window bytes j+2 .. j+6
-    const unsigned long long lo = r0[row][0], hi = r0[row][1];
-    unsigned long long o = 0ull;
-#pragma unroll
-    for (int sh = 2; sh <= 6; ++sh) o |= (lo >> (8 * sh)) | (hi << (64 - 8 * sh));
-    r1[row] = o;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < HZ * FY; q += blockDim.x) {
-    const int y = q % FY, z = q / FY;
-    const unsigned long long *c = &r1[z * HY + y];
-    r2[q] = c[0] | c[1] | c[2] | c[3] | c[4];
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < FZ * FY; q += blockDim.x) {
-    const int y = q % FY, z = q / FY;
-    const int c1 = y0 + y, c2 = z0 + z;
-    if (c1 >= ny || c2 >= nz) continue;
-    const unsigned long long o = r2[z * FY + y] | r2[(z + 1) * FY + y] | r2[(z + 2) * FY + y] |
-                                 r2[(z + 3) * FY + y] | r2[(z + 4) * FY + y];
-    uint8_t *d = dil + x0 + (long)nx * (c1 + (long)ny * c2);
-    if ((nx % 8) == 0 && x0 + 8 <= nx) {
-      *reinterpret_cast<unsigned long long *>(d) = o;
-    } else {
-      for (int j = 0; j < 8 && x0 + j < nx; ++j) d[j] = (uint8_t)(o >> (8 * j));
-    }
-  }
-}
-
-// any (optional): the raw-flag kernel's vote; zero means no cell is flagged,
-// the dilation is all zero and the tile kernel, reading the same vote, loads
-// none of it -- nothing is written.
-__global__ void __launch_bounds__(256) k_flag_dilate3(DevGeo G, const uint8_t *__restrict__ raw,
-                                                     uint8_t *__restrict__ dil, int ntx, int nty,
-                                                     const unsigned int *__restrict__ any) {
-  __shared__ unsigned long long r0[HZ * HY][2];
-  __shared__ unsigned long long r1[HZ * HY], r2[HZ * FY];
-  if (any && *any == 0u) return;
-  const int nb = ntx * nty * ((G.n[2] + FZ - 1) / FZ);
-  for (int t0 = blockIdx.x; t0 < nb; t0 += gridDim.x) {   // the block's tiles; the grid fills the SMs once
-    int t = t0;
-    const int tx = t % ntx;
-    t /= ntx;
-    const int ty = t % nty, tz = t / nty;
-    dilate_tile(G, raw, dil, tx * FX, ty * FY, tz * FZ, r0, r1, r2);
-  }
-}
-
 // Contact-CT edge EMF along D at the lower corner (a-1/2, b-1/2) of cell c,
 // (D, A, B) cyclic (Sect. 2.4): the mean of the four face EMFs plus the
 // upwinded half-derivatives towards the cell-centred E = -u x B.  The face
