@@ -19,17 +19,22 @@
 // Device layout: dense cell vectors (x fastest, 32-bit indices), per-axis
 // coefficient arrays.  One BiCGSTAB iteration is five grid-stride kernels:
 //   K1  p = r + beta (p - omega v), ph = D^-1 p
-//   K2  v = A ph (= p + off-diagonal part of A applied to ph); partials of (rh, v)
-//   K3  s = r - alpha v, sh = D^-1 s;  partial sums of |w s|^2
-//   K4  t = A sh (= s + off-diagonal part on sh); partials of (t, s), (t, t)
-//   K5  x += alpha ph + omega sh, r = s - omega t;  partials of (rh, r), |w r|^2
-// Each reduction leaves one partial per block; a consumer kernel's first warp
-// sums the partials in a fixed order, so every block derives the same
-// scalars (alpha, omega, the norms) and takes the same decision without a
-// grid-wide barrier.  Convergence and breakdown are decided on the device and
-// recorded in a small status block, so the host enqueues iterations in
-// batches and reads the status once per batch; the kernels of an iteration
-// after the decision return at once.
+//   K2  v = A ph (= p + off-diagonal part of A applied to ph); (rh, v)
+//   K3  s = r - alpha v, sh = D^-1 s;  |w s|^2
+//   K4  t = A sh (= s + off-diagonal part on sh); (t, s), (t, t)
+//   K5  x += alpha ph + omega sh, r = s - omega t;  (rh, r), |w r|^2
+// Each reduction leaves one partial per block; the block that finishes last
+// sums them in a fixed order (so the result does not depend on which block that
+// is) and derives the scalars -- alpha, beta, omega, the norms -- and the
+// decisions, which the next kernel reads from a small status block.  The FP64
+// pipe (1/64 of the FP32 rate) bounds the iteration, so the sums are arranged
+// for few FP64 instructions: a block's 256 values go through shared memory to
+// one warp (13 instructions, where eight warps' shuffles took 45), and the
+// partials are summed once, not by every block of the consumer (7 us a column
+// at 608 blocks when one warp of each did).  96^3: 99 -> 70 us of kernels an iteration.
+// Convergence and breakdown are decided on the device, so the host enqueues
+// iterations in batches and reads the status once per batch; the kernels of
+// an iteration after the decision return at once.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -48,8 +53,9 @@ enum { Q_RR = 0, Q_NR, Q_RV, Q_NS, Q_TS, Q_TT, Q_COUNT };
 enum { ST_RUN = 0, ST_HALF = 2, ST_DONE = 3, ST_BREAK = -2, ST_BADRHO = -3 };
 
 struct Status {
-  double rho_old, alpha, omega, rho, resid;
+  double alpha, beta, omega, rho, resid;
   int status, iters;
+  unsigned done;   // blocks of the running kernel that have left their partials
 };
 
 struct PGeo {
@@ -63,6 +69,7 @@ struct PGeo {
   int lmax, relative, nb;
   double tol;
   unsigned gofs[3];                      // offsets of the x, y, z ghost blocks
+  FastDiv fx, fy;                        // by n[0], n[1] (cells below 2^31)
 };
 
 struct Vecs {
@@ -73,11 +80,66 @@ struct Vecs {
 };
 
 __device__ __forceinline__ void decode(const PGeo &g, unsigned q, int &i, int &j, int &k) {
-  const unsigned a = q / (unsigned)g.n[0];
-  const unsigned b = a / (unsigned)g.n[1];
+  unsigned a, b;
+  if (g.nc < 0x80000000u) {
+    a = fastdiv(q, g.fx);
+    b = fastdiv(a, g.fy);
+  } else {
+    a = q / (unsigned)g.n[0];
+    b = a / (unsigned)g.n[1];
+  }
   i = (int)(q - a * (unsigned)g.n[0]);
   j = (int)(a - b * (unsigned)g.n[1]);
   k = (int)b;
+}
+
+// Sums of N values over the block's threads (all call), N <= PT / 32: warp c
+// sums the c-th and returns it.  sh: N * PT doubles.
+template <int N>
+__device__ __forceinline__ double block_sums(const double *v, double *sh) {
+#pragma unroll
+  for (int c = 0; c < N; ++c) sh[c * PT + threadIdx.x] = v[c];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  double t = 0.0;
+  if (w < N) {
+#pragma unroll
+    for (int k = 0; k < PT / 32; ++k) t += sh[w * PT + 32 * k + l];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  __syncthreads();
+  return t;   // warp c: the sum of v[c]
+}
+
+// Leaves the block's sums of N columns as its partials; the block that does so
+// last sums every block's partials, and its thread 0 gets the totals (true).
+template <int N>
+__device__ __forceinline__ bool reduce_last(const double *v, double *const *part, int nb, Status *st, double *sh,
+                                            double *tot) {
+  __shared__ bool last;
+  const int w = threadIdx.x >> 5;
+  double t = block_sums<N>(v, sh);
+  if (w < N && (threadIdx.x & 31) == 0) part[w][blockIdx.x] = t;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(&st->done, (unsigned)nb - 1u) == (unsigned)nb - 1u;   // wraps to 0
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double a[N];
+#pragma unroll
+  for (int c = 0; c < N; ++c) a[c] = 0.0;
+  for (int b = (int)threadIdx.x; b < nb; b += PT)
+#pragma unroll
+    for (int c = 0; c < N; ++c) a[c] += __ldcg(part[c] + b);
+  t = block_sums<N>(a, sh);
+  if (w < N && (threadIdx.x & 31) == 0) sh[w] = t;
+  __syncthreads();
+  if (threadIdx.x != 0) return false;
+#pragma unroll
+  for (int c = 0; c < N; ++c) tot[c] = sh[c];
+  return true;
 }
 
 // Block sum of v (all threads), result valid in every thread after the call.
@@ -164,7 +226,23 @@ __device__ __forceinline__ double apply_pre(const PGeo &g, const double *__restr
   return s;
 }
 
-__device__ __forceinline__ bool block0_lead() { return blockIdx.x == 0 && threadIdx.x == 0; }
+// After `it` full steps, from (rh, r) and |w r|^2: convergence or breakdown,
+// else beta of the next step.
+__device__ __forceinline__ void step_decision(const PGeo &g, Status *st, double rr, double nr, int it) {
+  if (*(volatile int *)&st->status != ST_RUN) return;   // ST_BADRHO
+  const double res = sqrt(nr / (double)g.nc);
+  st->resid = res;
+  if (res < g.tol) {
+    st->status = ST_DONE;
+    st->iters = it;
+  } else if ((it > 0 && st->omega == 0.0) || rr == 0.0) {
+    st->status = ST_BREAK;
+    st->iters = it;
+  } else {
+    st->beta = it == 0 ? 0.0 : (rr / st->rho) * (st->alpha / st->omega);
+    st->rho = rr;
+  }
+}
 
 // ---------------------------------------------------------------- multipoles
 
@@ -319,8 +397,8 @@ __global__ void k_ghost(PGeo g, Vecs V, unsigned nghost) {
 
 // r = b - A x0 with b = 4 pi G rho - (ghost terms); rh = r; p = v = 0;
 // D^-1, the residual weights; partials of (rh, r) and |w r|^2.
-__global__ void k_init(PGeo g, Vecs V) {
-  __shared__ double sh[PT / 32];
+__global__ void __launch_bounds__(PT) k_init(PGeo g, Vecs V) {
+  __shared__ double sh[2 * PT];
   const double fpg = 4.0 * 3.14159265358979323846 * g.G;
   double rr = 0.0, nr = 0.0;
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
@@ -339,49 +417,32 @@ __global__ void k_init(PGeo g, Vecs V) {
     rr += r * r;
     nr += (w * r) * (w * r);
   }
-  rr = block_sum(rr, sh);
-  nr = block_sum(nr, sh);
-  if (threadIdx.x == 0) {
-    V.part[Q_RR * g.nb + blockIdx.x] = rr;
-    V.part[Q_NR * g.nb + blockIdx.x] = nr;
-  }
+  const double v[2] = {rr, nr};
+  double *const part[2] = {V.part + Q_RR * g.nb, V.part + Q_NR * g.nb};
+  double tot[2];
+  if (reduce_last<2>(v, part, g.nb, V.st, sh, tot)) step_decision(g, V.st, tot[0], tot[1], 0);
 }
 
 // ------------------------------------------------------------ one iteration
 
-// K1: residual check of the previous full step; p and ph.
-__global__ void k_bi_p(PGeo g, Vecs V, int it) {
+// K1: p and ph
+__global__ void __launch_bounds__(PT) k_bi_p(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double s2[2];
-  if (threadIdx.x < 32) {
-    const double rr = sum_parts(V.part + Q_RR * g.nb, g.nb), nr = sum_parts(V.part + Q_NR * g.nb, g.nb);
-    if (threadIdx.x == 0) { s2[0] = rr; s2[1] = nr; }
-  }
-  __syncthreads();
-  const double rr = s2[0], res = sqrt(s2[1] / (double)g.nc);
-  if (res < g.tol) {
-    if (block0_lead()) { V.st->status = ST_DONE; V.st->iters = it - 1; V.st->resid = res; }
-    return;
-  }
-  if ((it > 1 && V.st->omega == 0.0) || rr == 0.0) {
-    if (block0_lead()) { V.st->status = ST_BREAK; V.st->iters = it - 1; V.st->resid = res; }
-    return;
-  }
-  const double beta = it == 1 ? 0.0 : (rr / V.st->rho_old) * (V.st->alpha / V.st->omega);
-  const double om = V.st->omega;
+  const double beta = V.st->beta, om = V.st->omega;
+#pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
     const double p = it == 1 ? V.r[q] : V.r[q] + beta * (V.p[q] - om * V.v[q]);
     V.p[q] = p;
     V.ph[q] = V.dinv[q] * p;
   }
-  if (block0_lead()) { V.st->rho = rr; V.st->resid = res; }
 }
 
-// K2: v = A ph, partials of (rh, v)
-__global__ void k_bi_av(PGeo g, Vecs V) {
+// K2: v = A ph; (rh, v) and alpha
+__global__ void __launch_bounds__(PT) k_bi_av(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[PT / 32];
+  __shared__ double sh[PT];
   double rv = 0.0;
+#pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
     int i, j, k;
     decode(g, q, i, j, k);
@@ -389,27 +450,21 @@ __global__ void k_bi_av(PGeo g, Vecs V) {
     V.v[q] = v;
     rv += V.rh[q] * v;
   }
-  rv = block_sum(rv, sh);
-  if (threadIdx.x == 0) V.part[Q_RV * g.nb + blockIdx.x] = rv;
+  double *const part[1] = {V.part + Q_RV * g.nb};
+  double tot[1];
+  if (reduce_last<1>(&rv, part, g.nb, V.st, sh, tot)) {
+    if (tot[0] == 0.0) { V.st->status = ST_BREAK; V.st->iters = it; }
+    else V.st->alpha = V.st->rho / tot[0];
+  }
 }
 
-// K3: alpha, s, sh; partials of |w s|^2
-__global__ void k_bi_s(PGeo g, Vecs V, int it) {
+// K3: s, sh; |w s|^2 and the half-step check
+__global__ void __launch_bounds__(PT) k_bi_s(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[PT / 32];
-  __shared__ double s1;
-  if (threadIdx.x < 32) {
-    const double rv = sum_parts(V.part + Q_RV * g.nb, g.nb);
-    if (threadIdx.x == 0) s1 = rv;
-  }
-  __syncthreads();
-  const double rv = s1;
-  if (rv == 0.0) {
-    if (block0_lead()) { V.st->status = ST_BREAK; V.st->iters = it; }
-    return;
-  }
-  const double alpha = V.st->rho / rv;
+  __shared__ double sh[PT];
+  const double alpha = V.st->alpha;
   double ns = 0.0;
+#pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
     const double s = V.r[q] - alpha * V.v[q];
     V.s[q] = s;
@@ -417,27 +472,20 @@ __global__ void k_bi_s(PGeo g, Vecs V, int it) {
     const double ws = g.relative ? V.w[q] * s : s;   // the absolute criterion has unit weights
     ns += ws * ws;
   }
-  ns = block_sum(ns, sh);
-  if (threadIdx.x == 0) V.part[Q_NS * g.nb + blockIdx.x] = ns;
-  if (block0_lead()) V.st->alpha = alpha;
+  double *const part[1] = {V.part + Q_NS * g.nb};
+  double tot[1];
+  if (reduce_last<1>(&ns, part, g.nb, V.st, sh, tot)) {
+    const double res = sqrt(tot[0] / (double)g.nc);
+    if (res < g.tol) { V.st->status = ST_HALF; V.st->iters = it; V.st->resid = res; }
+  }
 }
 
-// K4: half-step check; t = A sh, partials of (t, s), (t, t)
-__global__ void k_bi_at(PGeo g, Vecs V, int it) {
+// K4: t = A sh; (t, s), (t, t) and omega
+__global__ void __launch_bounds__(PT) k_bi_at(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[PT / 32];
-  __shared__ double s1;
-  if (threadIdx.x < 32) {
-    const double ns = sum_parts(V.part + Q_NS * g.nb, g.nb);
-    if (threadIdx.x == 0) s1 = ns;
-  }
-  __syncthreads();
-  const double res = sqrt(s1 / (double)g.nc);
-  if (res < g.tol) {
-    if (block0_lead()) { V.st->status = ST_HALF; V.st->iters = it; V.st->resid = res; }
-    return;
-  }
+  __shared__ double sh[2 * PT];
   double ts = 0.0, tt = 0.0;
+#pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
     int i, j, k;
     decode(g, q, i, j, k);
@@ -446,17 +494,18 @@ __global__ void k_bi_at(PGeo g, Vecs V, int it) {
     ts += t * V.s[q];
     tt += t * t;
   }
-  ts = block_sum(ts, sh);
-  tt = block_sum(tt, sh);
-  if (threadIdx.x == 0) {
-    V.part[Q_TS * g.nb + blockIdx.x] = ts;
-    V.part[Q_TT * g.nb + blockIdx.x] = tt;
+  const double v[2] = {ts, tt};
+  double *const part[2] = {V.part + Q_TS * g.nb, V.part + Q_TT * g.nb};
+  double tot[2];
+  if (reduce_last<2>(v, part, g.nb, V.st, sh, tot)) {
+    if (tot[1] == 0.0) { V.st->status = ST_BREAK; V.st->iters = it; }
+    else V.st->omega = tot[0] / tot[1];
   }
 }
 
 // K5: the solution and residual updates (or the half-step update decided by
-// K4 of this iteration); partials of (rh, r) and |w r|^2 for the next K1.
-__global__ void k_bi_x(PGeo g, Vecs V, int it) {
+// K3 of this iteration); (rh, r), |w r|^2 and the decision on them.
+__global__ void __launch_bounds__(PT) k_bi_x(PGeo g, Vecs V, int it) {
   const int st = V.st->status;
   const double alpha = V.st->alpha;
   if (st == ST_HALF) {
@@ -468,19 +517,10 @@ __global__ void k_bi_x(PGeo g, Vecs V, int it) {
     return;
   }
   if (st != ST_RUN) return;
-  __shared__ double sh[PT / 32];
-  __shared__ double s2[2];
-  if (threadIdx.x < 32) {
-    const double ts = sum_parts(V.part + Q_TS * g.nb, g.nb), tt = sum_parts(V.part + Q_TT * g.nb, g.nb);
-    if (threadIdx.x == 0) { s2[0] = ts; s2[1] = tt; }
-  }
-  __syncthreads();
-  if (s2[1] == 0.0) {
-    if (block0_lead()) { V.st->status = ST_BREAK; V.st->iters = it; }
-    return;
-  }
-  const double omega = s2[0] / s2[1];
+  __shared__ double sh[2 * PT];
+  const double omega = V.st->omega;
   double rr = 0.0, nr = 0.0;
+#pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
     V.x[q] += alpha * V.ph[q] + omega * V.sh[q];
     const double r = V.s[q] - omega * V.t[q];
@@ -489,16 +529,10 @@ __global__ void k_bi_x(PGeo g, Vecs V, int it) {
     const double wr = g.relative ? V.w[q] * r : r;
     nr += wr * wr;
   }
-  rr = block_sum(rr, sh);
-  nr = block_sum(nr, sh);
-  if (threadIdx.x == 0) {
-    V.part[Q_RR * g.nb + blockIdx.x] = rr;
-    V.part[Q_NR * g.nb + blockIdx.x] = nr;
-  }
-  if (block0_lead()) {
-    V.st->omega = omega;
-    V.st->rho_old = V.st->rho;
-  }
+  const double v[2] = {rr, nr};
+  double *const part[2] = {V.part + Q_RR * g.nb, V.part + Q_NR * g.nb};
+  double tot[2];
+  if (reduce_last<2>(v, part, g.nb, V.st, sh, tot)) step_decision(g, V.st, tot[0], tot[1], it);
 }
 
 // g = -grad phi (non-uniform central difference), ghost potentials at the sides
@@ -588,6 +622,8 @@ phl_status phl_poisson_create(const phl_poisson_desc *d, phl_poisson **out) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const unsigned want = (unsigned)(sms > 0 ? sms : 1) * 4u, most = (g.nc + PT - 1) / PT;
   g.nb = (int)(want < most ? want : most);
+  g.fx = make_fastdiv((unsigned)g.n[0]);
+  g.fy = make_fastdiv((unsigned)g.n[1]);
 
   // per-axis coefficients on the host (FP64)
   std::vector<double> hc;
@@ -666,7 +702,7 @@ phl_status phl_poisson_solve(phl_poisson *P, const double *rho, double *phi, int
   const cudaMemcpyKind kin = where == PHL_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   cudaError_t e = cudaMemcpyAsync(V.rho, rho, bytes, kin, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(V.x, phi, bytes, kin, s);
-  Status h0{1.0, 1.0, 1.0, 0.0, 0.0, ST_RUN, 0};
+  Status h0{1.0, 0.0, 1.0, 1.0, 0.0, ST_RUN, 0, 0u};
   if (e == cudaSuccess) e = cudaMemcpyAsync(P->st, &h0, sizeof(Status), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return pcuda(e, "Poisson inputs");
   const dim3 grid((unsigned)g.nb), block(PT);
@@ -681,13 +717,11 @@ phl_status phl_poisson_solve(phl_poisson *P, const double *rho, double *phi, int
     const int last = it + P->batch - 1 < P->max_iter ? it + P->batch - 1 : P->max_iter;
     for (; it <= last; ++it) {
       k_bi_p<<<grid, block, 0, s>>>(g, V, it);
-      k_bi_av<<<grid, block, 0, s>>>(g, V);
+      k_bi_av<<<grid, block, 0, s>>>(g, V, it);
       k_bi_s<<<grid, block, 0, s>>>(g, V, it);
       k_bi_at<<<grid, block, 0, s>>>(g, V, it);
       k_bi_x<<<grid, block, 0, s>>>(g, V, it);
     }
-    // the residual check of the last full step happens in the next K1
-    if (it > P->max_iter) k_bi_p<<<grid, block, 0, s>>>(g, V, it);
     e = cudaMemcpyAsync(&h, P->st, sizeof(Status), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return pcuda(e, "Poisson iterations");
