@@ -99,9 +99,10 @@ __device__ __forceinline__ void block_dmax(double m, unsigned long long *dmax) {
 // second pass over the state.
 __global__ void __launch_bounds__(256) k_prim(DevGeo G, Box box, const double *__restrict__ U,
                                               const double *__restrict__ Bf, double *__restrict__ W, int *dflag,
-                                              unsigned long long *dmax) {
+                                              unsigned long long *dmax, unsigned int *any) {
   int c[3], s[3];
   double rate = 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *any = 0u;   // the raw-flag kernel's vote, taken after this kernel
   if (cell3(box, c)) {
     bool fl[3], in = true;
     for (int d = 0; d < 3; ++d) {
@@ -122,11 +123,11 @@ __global__ void __launch_bounds__(256) k_prim(DevGeo G, Box box, const double *_
   if (dmax) block_dmax(rate, dmax);
 }
 
-__global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
+__device__ __forceinline__ void update_cell(const DevGeo &G, const Box &box, long tl, const StageBufs &S) {
   const double dt = *S.dt;
   {
     int c[3];
-    if (!cell3(box, c)) return;
+    if (!cell_at(box, tl, c)) return;
     const long p = widx(G, c[0], c[1], c[2]);
     const long ps = sidx(G, c[0], c[1], c[2]);
     const long wt = G.wtot, pl = G.plane;
@@ -158,6 +159,21 @@ __global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
       const long q = v * pl + ps;
       S.Uout[q] = S.a * S.Ubase[q] + S.b * S.Uin[q] - S.b * dt * r[v];
     }
+  }
+}
+
+__global__ void k_update_cells(DevGeo G, Box box, StageBufs S) {
+  update_cell(G, box, blockIdx.x * (long)blockDim.x + threadIdx.x, S);
+}
+
+// Edge EMFs and the cell update in one launch (small grids): both need the
+// faces only.  The first nemf blocks take the sites.
+__global__ void __launch_bounds__(256) k_emf_cells(DevGeo G, Box bsite, Box bcell, unsigned nemf, StageBufs S) {
+  if (blockIdx.x < nemf) {
+    int c[3];
+    if (cell3(bsite, c)) emf_sites<double>(G, c, S.W, S.F[0], S.F[1], S.F[2], S.E);
+  } else {
+    update_cell(G, bcell, (blockIdx.x - nemf) * (long)blockDim.x + threadIdx.x, S);
   }
 }
 
@@ -238,7 +254,7 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
                                S.cfl_dmax, const_cast<double *>(S.dt));
     } else {
       const unsigned t = tpb_for(b.n);
-      PHL_LAUNCH(KC_PRIM, prof, s, k_prim<<<gridt(b, t), t, 0, s>>>(G, b, S.Uin, S.Bin, S.W, S.dflag, S.cfl_dmax));
+      PHL_LAUNCH(KC_PRIM, prof, s, k_prim<<<gridt(b, t), t, 0, s>>>(G, b, S.Uin, S.Bin, S.W, S.dflag, S.cfl_dmax, S.any));
       if (S.cfl_dmax) {
         PHL_LAUNCH(KC_DT, prof, s, k_dt_finalize<<<1, 1, 0, s>>>(G.cfl, S.cfl_dmax, const_cast<double *>(S.dt)));
         ++nl;
@@ -247,34 +263,67 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
     }
   }
   // (2) shock flags
-  if (G.eps_sf > 0.0) nl += launch_flags<double>(G, S.W, S.raw, S.raw + (long)G.n[0] * G.n[1] * G.n[2], S.flag, S.any, s, prof);
+  if (G.eps_sf > 0.0)
+    nl += launch_flags<double>(G, S.W, S.raw, S.raw + (long)G.n[0] * G.n[1] * G.n[2], S.flag, S.any, s, prof,
+                               G.eos != 1);
   // (3) fluxes: normal faces [0, n], one transverse ghost row each side
+  Box bf[3];
+  long most = 0;
   for (int D = 0; D < 3; ++D) {
-    if (!G.act[D]) continue;
     int l[3], h[3];
     for (int d = 0; d < 3; ++d) {
       if (d == D) { l[d] = 0; h[d] = G.n[d] + 1; }
       else rng(d, 1, 1, l[d], h[d]);
     }
-    Box b = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
-    launch_flux<double>(D, G, b, S.W, S.Bin, (const double *)nullptr, S.flag, S.F[D], S.dflag, s, prof);
+    bf[D] = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
+    if (G.act[D] && bf[D].n > most) most = bf[D].n;
+  }
+  // one launch for all directions, and one for the EMFs and the cell update,
+  // where a direction's faces are fewer than the GPU's threads in a wave (128
+  // x 128: 40 + 12 -> 28 + 8 us a stage, and two launches fewer)
+  const bool small = most < 4L * 152 * 128 && G.recon == PHL_RECON_VANLEER;
+  if (small) {
+    FaceSet<double> A{};
+    const unsigned t = most < 152L * 128 ? 32u : 64u;
+    unsigned blocks = 0;
+    for (int D = 0; D < 3; ++D) {
+      A.first[D] = ~0u;
+      if (!G.act[D]) continue;
+      A.box[D] = bf[D];
+      A.F[D] = S.F[D];
+      A.Bf[D] = S.Bin;
+      A.first[D] = blocks;
+      blocks += (unsigned)((bf[D].n + t - 1) / t);
+    }
+    if (G.nspec == 0)
+      PHL_LAUNCH(KC_FLUX_X, prof, s, (k_flux_all<double, 0><<<blocks, t, 0, s>>>(G, A, S.W, S.flag, S.dflag)));
+    else
+      PHL_LAUNCH(KC_FLUX_X, prof, s, (k_flux_all<double, PHL_NSPEC_MAX><<<blocks, t, 0, s>>>(G, A, S.W, S.flag, S.dflag)));
+    ++nl;
+  }
+  for (int D = 0; D < 3 && !small; ++D) {
+    if (!G.act[D]) continue;
+    launch_flux<double>(D, G, bf[D], S.W, S.Bin, (const double *)nullptr, S.flag, S.F[D], S.dflag, s, prof);
     ++nl;
   }
   // (4) edge EMFs
-  {
-    const Box b = site_box(G);
-    const unsigned t = tpb_for(b.n);
-    PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<double><<<gridt(b, t), t, 0, s>>>(G, b, S.W, S.F[0], S.F[1], S.F[2], S.E));
+  const Box bs = site_box(G), bc = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
+  if (small) {
+    const unsigned t = tpb_for(bs.n), nemf = gridt(bs, t).x;
+    PHL_LAUNCH(KC_EMF, prof, s, k_emf_cells<<<nemf + gridt(bc, t).x, t, 0, s>>>(G, bs, bc, nemf, S));
     ++nl;
-  }
-  // (5) updates
-  {
-    Box b = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-    const unsigned t = tpb_for(b.n);
-    PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells<<<gridt(b, t), t, 0, s>>>(G, b, S));
-    Box bf = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
-    PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<<<gridt(bf, t), t, 0, s>>>(G, bf, S));
+  } else {
+    const unsigned t = tpb_for(bs.n);
+    PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<double><<<gridt(bs, t), t, 0, s>>>(G, bs, S.W, S.F[0], S.F[1], S.F[2], S.E));
+    PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells<<<gridt(bc, t), t, 0, s>>>(G, bc, S));
     nl += 2;
+  }
+  // (5) face updates
+  {
+    const Box bu = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
+    const unsigned t = tpb_for(bu.n);
+    PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<<<gridt(bu, t), t, 0, s>>>(G, bu, S));
+    ++nl;
   }
   if (nlaunch) *nlaunch += nl;
 }

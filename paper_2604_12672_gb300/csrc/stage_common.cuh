@@ -401,12 +401,12 @@ inline dim3 gridt(const Box &b, unsigned t) { return dim3((unsigned)((b.n + t - 
 
 // Raw flags (W holds the stage input), then the flags of the cells the face
 // stencils touch; tmp: one interior byte field, any: one device word.  Returns
-// the launches.
+// the launches.  zeroed: an earlier kernel of the stage has cleared the word.
 template <typename R>
 inline int launch_flags(const DevGeo &G, const R *W, uint8_t *raw, uint8_t *tmp, uint8_t *flag, unsigned int *any, cudaStream_t s,
-                        Prof *prof) {
+                        Prof *prof, bool zeroed = false) {
   Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-  cudaMemsetAsync(any, 0, sizeof(unsigned int), s);
+  if (!zeroed) cudaMemsetAsync(any, 0, sizeof(unsigned int), s);
   const unsigned t = tpb_for(bi.n);
   PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw<R><<<gridt(bi, t), t, 0, s>>>(G, bi, W, raw, any));
   int l[3], h[3];
@@ -576,11 +576,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_flux(DevGeo G, 
 // box: the faces with the D extent divided by step (rounded up); nD: number
 // of D-faces.
 template <int D, typename R, int NS>
-__global__ void __launch_bounds__(128, NS ? 3 : 4)
-    k_flux_walk(DevGeo G, Box box, int nD, int step, const R *__restrict__ W, const double *__restrict__ Bf,
-                const R *__restrict__ dB, const uint8_t *__restrict__ flag, R *__restrict__ F, int *dflag) {
+__device__ __forceinline__ void walk_faces(const DevGeo &G, const Box &box, long tl, int nD, int step,
+                                           const R *__restrict__ W, const double *__restrict__ Bf,
+                                           const R *__restrict__ dB, const uint8_t *__restrict__ flag,
+                                           R *__restrict__ F, int *dflag) {
   int c[3];
-  if (!cell3(box, c)) return;
+  if (!cell_at(box, tl, c)) return;
   c[D] *= step;
   const long sd = wstride(G, D);
   constexpr int NWC = W_X0 + NS;
@@ -612,6 +613,35 @@ __global__ void __launch_bounds__(128, NS ? 3 : 4)
     for (int v = 0; v < NWC; ++v)
       if (used(v)) ql[v] = qn[v];
   }
+}
+
+template <int D, typename R, int NS>
+__global__ void __launch_bounds__(128, NS ? 3 : 4)
+    k_flux_walk(DevGeo G, Box box, int nD, int step, const R *__restrict__ W, const double *__restrict__ Bf,
+                const R *__restrict__ dB, const uint8_t *__restrict__ flag, R *__restrict__ F, int *dflag) {
+  walk_faces<D, R, NS>(G, box, blockIdx.x * (long)blockDim.x + threadIdx.x, nD, step, W, Bf, dB, flag, F, dflag);
+}
+
+// The faces of every direction in one launch, one face per thread (small
+// grids: one direction's faces leave most of the GPU's FP64 pipes idle while
+// each face's own chain of operations runs, 20 us a direction on 128 x 128).
+template <typename R>
+struct FaceSet {
+  Box box[3];
+  unsigned first[3];   // first block of each direction; ~0u: inactive
+  R *F[3];
+  const double *Bf[3];
+};
+template <typename R, int NS>
+__global__ void __launch_bounds__(128, NS ? 3 : 4)
+    k_flux_all(DevGeo G, FaceSet<R> A, const R *__restrict__ W, const uint8_t *__restrict__ flag, int *dflag) {
+  auto at = [&](int d) { return (blockIdx.x - A.first[d]) * (long)blockDim.x + threadIdx.x; };
+  if (A.first[2] <= blockIdx.x)
+    walk_faces<2, R, NS>(G, A.box[2], at(2), A.box[2].hi[2], 1, W, A.Bf[2], (const R *)nullptr, flag, A.F[2], dflag);
+  else if (A.first[1] <= blockIdx.x)
+    walk_faces<1, R, NS>(G, A.box[1], at(1), A.box[1].hi[1], 1, W, A.Bf[1], (const R *)nullptr, flag, A.F[1], dflag);
+  else
+    walk_faces<0, R, NS>(G, A.box[0], at(0), A.box[0].hi[0], 1, W, A.Bf[0], (const R *)nullptr, flag, A.F[0], dflag);
 }
 
 // Edge EMF along D at the lower corner (a-1/2, b-1/2), (D, A, B) cyclic.
@@ -670,15 +700,21 @@ __device__ __forceinline__ void k_emf_at(long tl, const DevGeo &G, const Box &bo
   if (cell_at(box, tl, c)) emf_site<D, R>(G, c, W, FA, FB, E);
 }
 
-// All edge directions of a site in one launch (box: [0, n] along active axes).
+// All edge directions of site c.
+template <typename R>
+__device__ __forceinline__ void emf_sites(const DevGeo &G, const int *c, const R *__restrict__ W,
+                                          const R *__restrict__ F0, const R *__restrict__ F1,
+                                          const R *__restrict__ F2, R *__restrict__ E) {
+  if (c[0] < G.n[0] && (G.act[1] || G.act[2])) emf_site<0, R>(G, c, W, F1, F2, E);
+  if (c[1] < G.n[1] && (G.act[2] || G.act[0])) emf_site<1, R>(G, c, W, F2, F0, E);
+  if (c[2] < G.n[2] && (G.act[0] || G.act[1])) emf_site<2, R>(G, c, W, F0, F1, E);
+}
+// The same for every site in one launch (box: [0, n] along active axes).
 template <typename R>
 __global__ void k_emf_all(DevGeo G, Box box, const R *__restrict__ W, const R *__restrict__ F0,
                           const R *__restrict__ F1, const R *__restrict__ F2, R *__restrict__ E) {
   int c[3];
-  if (!cell3(box, c)) return;
-  if (c[0] < G.n[0] && (G.act[1] || G.act[2])) emf_site<0, R>(G, c, W, F1, F2, E);
-  if (c[1] < G.n[1] && (G.act[2] || G.act[0])) emf_site<1, R>(G, c, W, F2, F0, E);
-  if (c[2] < G.n[2] && (G.act[0] || G.act[1])) emf_site<2, R>(G, c, W, F0, F1, E);
+  if (cell3(box, c)) emf_sites<R>(G, c, W, F0, F1, F2, E);
 }
 inline Box site_box(const DevGeo &G) {
   return make_box(0, G.act[0] ? G.n[0] + 1 : 1, 0, G.act[1] ? G.n[1] + 1 : 1, 0, G.act[2] ? G.n[2] + 1 : 1);
