@@ -264,7 +264,7 @@ cudaError_t launch_stage_phases(phl_ensemble *E, int stage, int nstages, float b
   return cudaSuccess;
 }
 
-// Mode 2: every box runs its own per-kernel step (CFL reduction + 3 stages)
+// Mode 2: every box runs its own per-kernel step (3 stages)
 // on one of nstreams streams forked from the ensemble's stream and joined back.
 cudaError_t launch_step_chains(phl_ensemble *E) {
   const int ns = E->nstreams;
@@ -299,10 +299,10 @@ cudaError_t launch_step_chains(phl_ensemble *E) {
     M.tmapW = v.tmapW; M.fused_variant = v.fused;   // the box's own stage decomposition
     M.pipeline3 = v.pipeline3;
     M.primed = false;   // each replay forms W from the state it finds
-    M.fmax = nullptr;   // the step's own CFL launch comes first: no maximum to carry
+    M.fmax = nullptr;   // no maximum to carry
+    M.cfl_fmax = v.fmax;   // the CFL step from the first stage's primitives
     *v.w_valid = false;
     int nl = 0;
-    launch_dt_mixed(*v.G, v.U, v.B, v.fmax, v.dt, v.dflag, st, &nl, nullptr);
     for (int stg = 0; stg < 3; ++stg) launch_stage_mixed(*v.G, M, stg, 3, b3[stg], st, &nl, nullptr);
     launches += nl;
     e = cudaGetLastError();

@@ -8,9 +8,15 @@ namespace phl {
 using namespace stage;
 namespace {
 
+// The raw-flag kernel's vote of this stage, taken after the primitives.
+__device__ __forceinline__ void clear_vote(unsigned int *any) {
+  if (any && blockIdx.x == 0 && threadIdx.x == 0) *any = 0u;
+}
+
 __global__ void k_prim_mx(DevGeo G, Box box, const double *__restrict__ U, const double *__restrict__ Bf,
                           const float *__restrict__ dU, const float *__restrict__ dB, float *__restrict__ W,
-                          int *dflag) {
+                          int *dflag, unsigned int *any) {
+  clear_vote(any);
   k_prim_mx_at(blockIdx.x * (long)blockDim.x + threadIdx.x, G, box, U, Bf, dU, dB, W, dflag);
 }
 
@@ -18,21 +24,38 @@ __global__ void k_prim_mx(DevGeo G, Box box, const double *__restrict__ U, const
 // the loads in flight, and this cap measured fastest (3 .. 8 tried).
 __global__ void __launch_bounds__(256, 5) k_prim_mx2(DevGeo G, Box hbox, const double *__restrict__ U,
                                                   const double *__restrict__ Bf, const float *__restrict__ dU,
-                                                  const float *__restrict__ dB, float *__restrict__ W, int *dflag) {
+                                                  const float *__restrict__ dB, float *__restrict__ W, int *dflag,
+                                                  unsigned int *any) {
+  clear_vote(any);
   k_prim_mx2_at<false>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, hbox, U, Bf, dU, dB, W, dflag);
 }
 
-// Block maximum of the CFL rates, one atomicMax per block (non-negative
-// floats order like their bit patterns).
-__device__ __forceinline__ void block_rate_max(float m, unsigned int *fmax_bits) {
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+// The CFL maximum of the launch (non-negative floats order like their bit
+// patterns): block maximum, one atomicMax per block.  With dt non-null the
+// block that finishes last turns it into the step length and clears it and its
+// counter (fmax_bits[1]) -- no launch of its own for that.
+struct DtOut {
+  double cfl, t_s;
+  double *dt;
+};
+__device__ __forceinline__ void block_rate_max(float m, unsigned int *fmax_bits, const DtOut &o) {
+  for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
   __shared__ float red[8];
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x < 32) {
     float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) atomicMax(fmax_bits, __float_as_uint(v));
+    for (int d = 16; d > 0; d >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
+    if (threadIdx.x == 0) {
+      atomicMax(fmax_bits, __float_as_uint(v));
+      if (o.dt) {
+        __threadfence();
+        if (atomicInc(fmax_bits + 1, gridDim.x - 1u) == gridDim.x - 1u) {   // the counter wraps to 0
+          __threadfence();
+          *o.dt = o.cfl * o.t_s / (double)__uint_as_float(atomicExch(fmax_bits, 0u));
+        }
+      }
+    }
   }
 }
 
@@ -40,10 +63,12 @@ __device__ __forceinline__ void block_rate_max(float m, unsigned int *fmax_bits)
 // rate of the interior cells taken from the same deviations.
 __global__ void __launch_bounds__(256, 5) k_prim_mx2_cfl(DevGeo G, Box hbox, const double *__restrict__ U,
                                                        const double *__restrict__ Bf, float *__restrict__ W,
-                                                       int *dflag, unsigned int *fmax_bits) {
+                                                       int *dflag, unsigned int *fmax_bits, DtOut o,
+                                                       unsigned int *any) {
+  clear_vote(any);
   const float m = k_prim_mx2_at<true>(blockIdx.x * (long)blockDim.x + threadIdx.x, G, hbox, U, Bf, nullptr, nullptr,
                                       W, dflag);
-  block_rate_max(m, fmax_bits);
+  block_rate_max(m, fmax_bits, o);
 }
 
 // The first stage's primitives of U^n with the CFL rate of the interior
@@ -51,12 +76,13 @@ __global__ void __launch_bounds__(256, 5) k_prim_mx2_cfl(DevGeo G, Box hbox, con
 // just formed): block maximum, one atomicMax per block.
 __global__ void __launch_bounds__(256) k_prim_mx_cfl(DevGeo G, Box box, const double *__restrict__ U,
                                                      const double *__restrict__ Bf, float *__restrict__ W, int *dflag,
-                                                     unsigned int *fmax_bits) {
+                                                     unsigned int *fmax_bits, DtOut o, unsigned int *any) {
+  clear_vote(any);
   float m = 0.0f;
   int c[3];
   if (cell_at(box, blockIdx.x * (long)blockDim.x + threadIdx.x, c))
     prim_store_cell(G, c, U, Bf, nullptr, nullptr, W, dflag, &m);
-  block_rate_max(m, fmax_bits);
+  block_rate_max(m, fmax_bits, o);
 }
 
 __global__ void k_update_cells_mx(DevGeo G, Box box, StageMx S) {
@@ -132,11 +158,12 @@ cudaError_t launch_prims_form(const DevGeo &G, const double *U, const double *Bf
   }
   const Box bx = make_box(l[0], h[0], l[1], h[1], l[2], h[2]);
   const Box hb = make_box(0, (G.n[0] + 2 * G.ge[0]) / 2, l[1], h[1], l[2], h[2]);
+  const DtOut none{0.0, 0.0, nullptr};
   switch (form) {
-    case 0: k_prim_mx<<<grid3(bx), block3(bx), 0, s>>>(G, bx, U, Bf, dU, dB, W, dflag); break;
-    case 1: k_prim_mx2<<<grid3(hb), block3(hb), 0, s>>>(G, hb, U, Bf, dU, dB, W, dflag); break;
-    case 2: k_prim_mx_cfl<<<grid3(bx), block3(bx), 0, s>>>(G, bx, U, Bf, W, dflag, fmax_bits); break;
-    default: k_prim_mx2_cfl<<<grid3(hb), block3(hb), 0, s>>>(G, hb, U, Bf, W, dflag, fmax_bits); break;
+    case 0: k_prim_mx<<<grid3(bx), block3(bx), 0, s>>>(G, bx, U, Bf, dU, dB, W, dflag, nullptr); break;
+    case 1: k_prim_mx2<<<grid3(hb), block3(hb), 0, s>>>(G, hb, U, Bf, dU, dB, W, dflag, nullptr); break;
+    case 2: k_prim_mx_cfl<<<grid3(bx), block3(bx), 0, s>>>(G, bx, U, Bf, W, dflag, fmax_bits, none, nullptr); break;
+    default: k_prim_mx2_cfl<<<grid3(hb), block3(hb), 0, s>>>(G, hb, U, Bf, W, dflag, fmax_bits, none, nullptr); break;
   }
   return cudaGetLastError();
 }
@@ -167,25 +194,24 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
                               first ? M.cfl_dmax : nullptr, const_cast<double *>(M.dt), G.use_mlp == 1 ? 0 : 2);
     } else {
       if (first && M.cfl_fmax) {   // the step's CFL step from the same pass over U^n
+        const DtOut o{G.cfl, G.sc_t, const_cast<double *>(M.dt)};
         if (prim_pairs_ok(G)) {
           Box hb = make_box(0, (G.n[0] + 2 * G.ge[0]) / 2, l[1], h[1], l[2], h[2]);
           PHL_LAUNCH(KC_PRIM, prof, s,
-                     k_prim_mx2_cfl<<<grid3(hb), block3(hb), 0, s>>>(G, hb, M.U, M.B, M.W, M.dflag, M.cfl_fmax));
+                     k_prim_mx2_cfl<<<grid3(hb), block3(hb), 0, s>>>(G, hb, M.U, M.B, M.W, M.dflag, M.cfl_fmax, o, M.anyraw));
         } else {
           PHL_LAUNCH(KC_PRIM, prof, s,
-                     k_prim_mx_cfl<<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.U, M.B, M.W, M.dflag, M.cfl_fmax));
+                     k_prim_mx_cfl<<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.U, M.B, M.W, M.dflag, M.cfl_fmax, o, M.anyraw));
         }
-        PHL_LAUNCH(KC_DT, prof, s, k_dt_mx_finalize<<<1, 1, 0, s>>>(G.cfl, G.sc_t, M.cfl_fmax, const_cast<double *>(M.dt)));
-        nl += 2;
       } else if (prim_pairs_ok(G)) {   // two cells of a row per thread
         Box hb = make_box(0, (G.n[0] + 2 * G.ge[0]) / 2, l[1], h[1], l[2], h[2]);
         PHL_LAUNCH(KC_PRIM, prof, s,
-                   k_prim_mx2<<<grid3(hb), block3(hb), 0, s>>>(G, hb, M.U, M.B, dU, dB, M.W, M.dflag));
-        ++nl;
+                   k_prim_mx2<<<grid3(hb), block3(hb), 0, s>>>(G, hb, M.U, M.B, dU, dB, M.W, M.dflag, M.anyraw));
       } else {
-        PHL_LAUNCH(KC_PRIM, prof, s, k_prim_mx<<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.U, M.B, dU, dB, M.W, M.dflag));
-        ++nl;
+        PHL_LAUNCH(KC_PRIM, prof, s,
+                   k_prim_mx<<<grid3(bx), block3(bx), 0, s>>>(G, bx, M.U, M.B, dU, dB, M.W, M.dflag, M.anyraw));
       }
+      ++nl;
     }
     if (three && G.eps_sf > 0.0) {
       Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
@@ -193,7 +219,8 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
       ++nl;
     }
   }
-  if (G.eps_sf > 0.0 && !fused) nl += launch_flags<float>(G, M.W, M.raw, M.raw + (long)G.n[0] * G.n[1] * G.n[2], M.flag, M.anyraw, s, prof);
+  if (G.eps_sf > 0.0 && !fused) nl += launch_flags<float>(G, M.W, M.raw, M.raw + (long)G.n[0] * G.n[1] * G.n[2], M.flag, M.anyraw, s, prof,
+                                                               G.eos != 1);
   if (fused) launch_fused_tail(G, M, first, last, b, s, &nl, prof);   // flags, faces, cells, EMFs, faces B
   for (int D = 0; D < 3 && !fused; ++D) {
     if (!G.act[D]) continue;

@@ -72,7 +72,8 @@ struct phl_grid {
   uint8_t *raw = nullptr, *flag = nullptr;
   // mixed precision: FP32 increments and work arrays
   float *dUf = nullptr, *dBf = nullptr, *Wf = nullptr, *Ff[3] = {nullptr, nullptr, nullptr}, *Ef = nullptr;
-  unsigned int *fmax = nullptr;         // [0]: the step's CFL maximum (three-launch path), [1]: phl_compute_dt
+  unsigned int *fmax = nullptr;         // [0]: the step's CFL maximum (three-launch path), [1]: the one taken from
+                                        // U^n, [2]: blocks that have added theirs to it
   unsigned int *anyraw = nullptr;       // fused path: some cell carries a raw shock flag (this stage)
   bool mixed = false;
   bool pipeline3 = false;               // fused mixed stage in three launches (phl_set_fused 201..209)
@@ -472,7 +473,7 @@ phl_status phl_create_grid(const phl_grid_desc *d, phl_grid **out) {
     for (int k = 0; k < 3; ++k)
       if (G.act[k]) AL(&g->Ff[k], (long)(G.nf + 1) * G.wtot);
     AL(&g->Ef, 3 * G.wtot);
-    AL(&g->fmax, 2);
+    AL(&g->fmax, 3);
     g->stage_a = (double *)g->Wf;
     g->stage_a_bytes = (size_t)(G.wstr + NAUX) * G.wtot * sizeof(float);
     g->stage_b = (double *)g->Ff[0];

@@ -312,7 +312,8 @@ struct MixedBufs {
   bool primed = false;
   unsigned int *fmax = nullptr; // CFL rate maximum the last stage folds into (pipeline3)
   // ideal gas, device CFL step: the first stage's primitives of U^n also
-  // fold the CFL rate into this maximum and set dt (no separate CFL pass)
+  // fold the CFL rate into this maximum and set dt (no separate CFL pass);
+  // the word after it counts the blocks
   unsigned int *cfl_fmax = nullptr;
   // the raw-flag kernel's "some cell is flagged" vote (zeroed before it)
   unsigned int *anyraw = nullptr;

@@ -647,7 +647,10 @@ __global__ void __launch_bounds__(NT, MINB)
                      float *__restrict__ F0, float *__restrict__ F1, float *__restrict__ F2, int ntx, int nty,
                      int *dflag, unsigned extra_tx, int raw_flags, const unsigned int *__restrict__ any) {
   extern __shared__ unsigned char smraw[];
-  if (any && *any == 0u) flag = nullptr;   // no cell flagged: the tile stages zero flags
+  if (any && *any == 0u) {   // no cell flagged: the tile stages zero flags
+    flag = nullptr;
+    raw_flags = 0;
+  }
   FusedSmem &sm = *reinterpret_cast<FusedSmem *>(smraw + ((128u - (smem_u32(smraw) & 127u)) & 127u));
   int t = blockIdx.x;
   const int tx = t % ntx;
@@ -1145,6 +1148,12 @@ cudaError_t fused_init() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flux_update_mx<256, 2, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem_bytes(true));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_flux_update_mx<576, 1, true, false, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_flux_update_mx<576, 1, true, false, true, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true));
   // the PPH instantiations
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flux_update_mx<256, 2, false, false, false, true>,
@@ -1226,6 +1235,11 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
   const int ntx = (G.n[0] + FX - 1) / FX, nty = (G.n[1] + FY - 1) / FY, ntz = (G.n[2] + FZ - 1) / FZ;
   const int nb = ntx * nty * ntz;
   const long ncell = (long)G.n[0] * G.n[1] * G.n[2];
+  // at most one tile per SM: twice the threads per tile (one face each instead
+  // of two), and the tile dilates the raw flags itself -- with one CTA per SM
+  // a tile's own latency is the launch's time (32 x 32 x 48 with flags: 15.5 +
+  // 4.9 us in two launches -> 13.4 us in one)
+  const bool few = nb <= 152 && M.fused_variant == PHL_FUSED_DEFAULT;
   const uint8_t *dil = nullptr;
   const unsigned int *any = nullptr;
   int raw_mode = 0;
@@ -1234,7 +1248,6 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
     raw_mode = 1;
   } else if (G.eps_sf > 0.0) {   // raw flags, then their 5^3 dilation, both on the interior layout
     Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
-    if (M.anyraw) cudaMemsetAsync(M.anyraw, 0, sizeof(unsigned int), s);
     if (flag_raw4_ok(G)) {   // four cells of a row per thread
       Box b4 = make_box(0, G.n[0] / 4, 0, G.n[1], 0, G.n[2]);
       PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw4<<<grid3(b4), block3(b4), 0, s>>>(G, b4, M.W, M.raw, M.anyraw));
@@ -1242,15 +1255,18 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
       PHL_LAUNCH(KC_FLAG_RAW, prof, s,
                  k_flag_raw<float><<<grid3(bi), block3(bi), 0, s>>>(G, bi, M.W, M.raw, M.anyraw));
     }
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int nbd = std::min(nb, 8 * std::max(nsm, 1));   // eight 256-thread CTAs per SM
-    PHL_LAUNCH(KC_FLAG_DILATE, prof, s,
-               k_flag_dilate3<<<nbd, 256, 0, s>>>(G, M.raw, M.raw + ncell, ntx, nty, M.anyraw));
-    dil = M.raw + ncell;
     any = M.anyraw;
-    *nl += 2;
+    ++*nl;
+    if (few) {
+      dil = M.raw;
+      raw_mode = 1;
+    } else {
+      const int nbd = std::min(nb, 8 * 152);   // eight 256-thread CTAs per SM
+      PHL_LAUNCH(KC_FLAG_DILATE, prof, s,
+                 k_flag_dilate3<<<nbd, 256, 0, s>>>(G, M.raw, M.raw + ncell, ntx, nty, M.anyraw));
+      dil = M.raw + ncell;
+      ++*nl;
+    }
   }
   const CUtensorMap *tm = (const CUtensorMap *)M.tmapW;
   // launch shapes: (threads, min CTAs per SM, phased)
@@ -1272,7 +1288,10 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
     case 5: PHL_FUSED(288, 1, true, true, false); break;
     case 6: PHL_FUSED(256, 2, true, true, false); break;
     case 7: PHL_FUSED(288, 2, true, true, false); break;
-    case 8: PHL_FUSED(288, 3, true, false, true); break;
+    case 8:
+      if (few) PHL_FUSED(576, 1, true, false, true);
+      else PHL_FUSED(288, 3, true, false, true);
+      break;
     case 9: PHL_FUSED(256, 2, false, false, true); break;
     default: PHL_FUSED(256, 2, false, false, false); break;
   }
