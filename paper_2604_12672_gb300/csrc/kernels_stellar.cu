@@ -145,7 +145,7 @@ __device__ __forceinline__ double eos_cell_step(const DevGeo &G, const int *c, c
     const unsigned tot = __reduce_add_sync(m, it > 0 ? (unsigned)it : 0u);
     if ((int)(threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(G.niter, (unsigned long long)tot);
   }
-  if (it < 0 || !(o.P > 0.0) || !(rho > 0.0)) atomicOr(dflag, it < 0 ? FLAG_NEWTON : FLAG_NEG);
+  if (it < 0 || !positive(o.P) || !positive(rho)) atomicOr(dflag, it < 0 ? FLAG_NEWTON : FLAG_NEG);
   Tout[p] = T;
   const Bg b = bg_cell(G, c[2]);
   const long q = widx(G, c[0], c[1], c[2]);

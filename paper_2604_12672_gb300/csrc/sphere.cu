@@ -703,8 +703,11 @@ __global__ void __launch_bounds__(SPT) k_sph_mlp_guess(SphDev D, const double *_
 // three float4 records per cell, and with dmax the CFL rate folded in.
 // pm (mixed form): 1 records each cell's inversion in D.pred, 2 also starts
 // from the previous record (eos_invert_rec; the second and third stages).
+// Bound by the FP64 pipe and its latency: two blocks on an SM (128 registers
+// instead of 172) and integer compares take 954 us instead of 1204 per launch
+// on N = 64, N_r = 96 (mixed).
 template <typename R>
-__global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, const double *__restrict__ U,
+__global__ void __launch_bounds__(SPT, 2) k_sph_prims_st(SphDev D, SphWork<R> Wk, const double *__restrict__ U,
                                                       const float *__restrict__ dU, const double *__restrict__ phi,
                                                       const float *__restrict__ phif, unsigned long long *dmax,
                                                       int pm) {
@@ -760,8 +763,10 @@ __global__ void __launch_bounds__(SPT) k_sph_prims_st(SphDev D, SphWork<R> Wk, c
     if (it < 0) atomicOr(D.dflag, FLAG_NEWTON);
     D.T[c] = T;
     const double P = o.P * D.ip_u;
-    if (!(rho > 0.0) || !(P > 0.0)) atomicOr(D.dflag, FLAG_NEG);
-    if (!isfinite(rho) || !isfinite(P)) atomicOr(D.dflag, FLAG_NAN);
+    if (!positive(rho) || !positive(P)) {   // false for infinities and NaN too
+      if (!(rho > 0.0) || !(P > 0.0)) atomicOr(D.dflag, FLAG_NEG);
+      if (!isfinite(rho) || !isfinite(P)) atomicOr(D.dflag, FLAG_NAN);
+    }
     double geh, gch;
     bg_gammas<double>(D, k, false, geh, gch);
     const double dP = P - bg_p(D, k), dge = o.ge - geh, dgc = o.gc - gch;

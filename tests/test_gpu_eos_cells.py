@@ -47,3 +47,25 @@ def test_cells_and_edges(P, lr, nr, lT, nT, precision):
     for key, tol in (("P", 1e-11), ("gamma_e", 1e-11), ("gamma_c", 1e-9)):
         assert np.abs(out[key] / np.array([r[key] for r in inv]) - 1).max() <= tol, key
     dt.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nr", [4, 81])
+def test_outside_is_refused(P, nr, precision):
+    """Densities beside either end of the table, far outside and NaN are
+    refused one by one; those just inside converge."""
+    lr, lT = (5.0, 7.0), (8.0, 9.5)
+    dt, ot = P.EosTable(lr, nr, lT, 61), O.EosTable(lr, nr, lT, 61)
+    cfg = O.stellar_cfg(W.STELLAR_A, W.STELLAR_Z, ot)
+    ye, T = 0.5, 10 ** 8.7
+    last = nr - 1
+    place = np.array([1e-9, 0.5, last - 1e-9, -1e-9, -1.0, last + 1e-9, last + 0.5])
+    rho = np.append(10 ** (lr[0] + place * (lr[1] - lr[0]) / last) / ye, [1e-200, 1e200, np.nan])
+    e = np.full(10, O.eos_rt(cfg, 10 ** 6 / ye, T, [0.5, 0.5])["e"])
+    for k in (0, 1, 2):
+        e[k] = O.eos_rt(cfg, rho[k], T, [0.5, 0.5])["e"]
+    one = np.ones(10)
+    out = P.eos(dt, rho, e, one / (0.5 / 16.0 + 0.5 / 28.0), ye * one, T * one * (1 + 1e-5), precision=precision)
+    assert (out["iters"][:3] > 0).all() and np.abs(out["T"][:3] / T - 1).max() <= 1e-9
+    assert (out["iters"][3:] == -1).all() and np.isnan(out["P"][3:]).all()
+    dt.close()
