@@ -63,6 +63,9 @@ __device__ __forceinline__ V fma(V a, V b, V c) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
   return r;
 }
+// a + b rounded lane by lane on its own: a packed add that follows a packed
+// multiplication may be contracted with it
+__device__ __forceinline__ V add_rn(V a, V b) { return V{__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)}; }
 __device__ __forceinline__ V neg(V a) { return V{-a.x, -a.y}; }
 __device__ __forceinline__ V rcp(V a) { return V{1.0f / a.x, 1.0f / a.y}; }
 __device__ __forceinline__ V sqrt2(V a) { return V{sqrtf(a.x), sqrtf(a.y)}; }
@@ -77,13 +80,11 @@ __device__ __forceinline__ B2 operator||(B2 a, B2 b) { return B2{a.x || b.x, a.y
 __device__ __forceinline__ B2 operator!(B2 a) { return B2{!a.x, !a.y}; }
 __device__ __forceinline__ V sel(B2 c, V a, V b) { return V{c.x ? a.x : b.x, c.y ? a.y : b.y}; }
 
-// One side of the face: full rho and P, deviations of the total pressure and
-// energy, fast speed, Mach number squared, u.B and the physical flux minus
-// the background flux (as Side in riemann.cuh).
+// One side of the face: full rho and P, velocity and transverse field, deviations of the total pressure and
+// energy, fast speed, Mach number squared and u.B (as Side in riemann.cuh).
 struct SideV {
-  V rho, un, ut1, ut2, bt1, bt2;
+  V rho, p, un, ut1, ut2, bt1, bt2;
   V dpt, enth, de, cf, m2, vb;
-  V F[7];
 };
 
 __device__ __forceinline__ void side_init_v(SideV &s, const V *w, V bn, V rh, V ph, const GasK<float> &K) {
@@ -92,7 +93,7 @@ __device__ __forceinline__ void side_init_v(SideV &s, const V *w, V bn, V rh, V 
   s.un = w[RD_UN]; s.ut1 = w[RD_UT1]; s.ut2 = w[RD_UT2];
   s.bt1 = w[RD_BT1]; s.bt2 = w[RD_BT2];
   const V dp = w[RD_P];
-  const V p = ph + dp;
+  const V p = s.p = ph + dp;
   const V irho = rcp(s.rho);
   const V bn2 = bn * bn;
   const V b2 = fma(s.bt2, s.bt2, fma(s.bt1, s.bt1, bn2));
@@ -104,18 +105,23 @@ __device__ __forceinline__ void side_init_v(SideV &s, const V *w, V bn, V rh, V 
   const V a2 = (vv(K.g) * p) * irho;
   const V bb = b2 * irho, bnn = bn2 * irho;
   const V ab = a2 + bb;
-  V disc = fma(ab, ab, neg(vv(4.0f) * a2 * bnn));
+  V disc = fma(ab, ab, vv(-4.0f) * a2 * bnn);
   disc = vmax(disc, vv(0.0f));
   s.cf = sqrt2(half * (ab + sqrt2(disc)));
   s.m2 = u2 * rcp(a2);
   s.vb = fma(s.ut2, s.bt2, fma(s.ut1, s.bt1, s.un * bn));
-  s.F[RF_RHO] = s.rho * s.un;
-  s.F[RF_MN] = fma(s.F[RF_RHO], s.un, s.dpt - bn2);
-  s.F[RF_MT1] = fma(s.F[RF_RHO], s.ut1, neg(bn * s.bt1));
-  s.F[RF_MT2] = fma(s.F[RF_RHO], s.ut2, neg(bn * s.bt2));
-  s.F[RF_E] = fma(s.enth, s.un, neg(bn * s.vb));
-  s.F[RF_BT1] = fma(s.un, s.bt1, neg(s.ut1 * bn));
-  s.F[RF_BT2] = fma(s.un, s.bt2, neg(s.ut2 * bn));
+}
+
+// The physical flux of the side minus the background flux.
+__device__ __forceinline__ void side_flux_v(const SideV &s, V bn, V *F) {
+  const V nbn = neg(bn);
+  F[RF_RHO] = s.rho * s.un;
+  F[RF_MN] = fma(F[RF_RHO], s.un, s.dpt - bn * bn);
+  F[RF_MT1] = fma(F[RF_RHO], s.ut1, nbn * s.bt1);
+  F[RF_MT2] = fma(F[RF_RHO], s.ut2, nbn * s.bt2);
+  F[RF_E] = fma(s.enth, s.un, nbn * s.vb);
+  F[RF_BT1] = fma(s.un, s.bt1, s.ut1 * nbn);
+  F[RF_BT2] = fma(s.un, s.bt2, s.ut2 * nbn);
 }
 
 // U* - U of one side and its intermediate transverse velocity and field (as
@@ -165,6 +171,9 @@ __device__ __forceinline__ void riemann_ideal_x2(const V *wl, const V *wr, V bn,
   SideV L, R;
   side_init_v(L, wl, bn, rh, ph, K);
   side_init_v(R, wr, bn, rh, ph, K);
+  V FL[7], FR[7];
+  side_flux_v(L, bn, FL);
+  side_flux_v(R, bn, FR);
   const V SL = vmin(L.un - L.cf, R.un - R.cf);
   const V SR = vmax(L.un + L.cf, R.un + R.cf);
   const V zero = vv(0.0f), one = vv(1.0f);
@@ -214,7 +223,7 @@ __device__ __forceinline__ void riemann_ideal_x2(const V *wl, const V *wr, V bn,
   const V Ssd = sel(dbl, Ss, zero);
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
-    const V fx = sel(left, L.F[q], R.F[q]);
+    const V fx = sel(left, FL[q], FR[q]);
     const V dux = sel(left, dUL[q], dUR[q]);
     f[q] = sel(fan, fma(Ssd, d2[q], fma(S, dux, fx)), fx);
   }
@@ -242,8 +251,8 @@ __device__ __forceinline__ void riemann_ideal_x2(const V *wl, const V *wr, V bn,
     const V sLR = SL * SR;
 #pragma unroll
     for (int q = 0; q < 7; ++q) {
-      const V mid = fma(sLR, dU[q], fma(SR, L.F[q], neg(SL * R.F[q]))) * idn;
-      h[q] = sel(oL, L.F[q], sel(rOut, R.F[q], mid));
+      const V mid = fma(sLR, dU[q], fma(SR, FL[q], neg(SL * FR[q]))) * idn;
+      h[q] = sel(oL, FL[q], sel(rOut, FR[q], mid));
     }
 #pragma unroll
     for (int q = 0; q < 7; ++q) f[q] = sel(hll, h[q], f[q]);
@@ -263,7 +272,9 @@ namespace x2 {
 // HLLD intermediate states are the same arithmetic on each side, so they run
 // as packed pairs without doubling the live state; everything that mixes the
 // sides (wave speeds, S_M, p_T*, the double-star states, the region choice)
-// stays scalar.  Same method and formulas as riemann_dev with IDEAL = true.
+// stays scalar, and once the side that holds the face is known, its flux and
+// U* - U are formed for it alone.  Same method and formulas as riemann_dev
+// with IDEAL = true.  pos: both states have positive density and pressure.
 
 __device__ __forceinline__ void sides_init_lr(SideV &s, const float *wl, const float *wr, float bn, float rh, float ph,
                                               const GasK<float> &K) {
@@ -277,18 +288,22 @@ __device__ __forceinline__ void sides_init_lr(SideV &s, const float *wl, const f
 }
 
 __device__ __forceinline__ void riemann_ideal_lr(const float *wl, const float *wr, float bn, float rh, float ph,
-                                                 int solver, float mthr, float *f, int &up, const GasK<float> &K) {
+                                                 int solver, float mthr, float *f, int &up, bool &pos,
+                                                 const GasK<float> &K) {
   SideV s;   // lane x: left side, lane y: right side
   sides_init_lr(s, wl, wr, bn, rh, ph, K);
+  pos = s.rho.x > 0.0f && s.rho.y > 0.0f && s.p.x > 0.0f && s.p.y > 0.0f;
   const V lo = s.un - s.cf, hi = s.un + s.cf;
   const float SL = fminf(lo.x, lo.y), SR = fmaxf(hi.x, hi.y);
   if (solver == SOLVER_HLL) {
+    V F[7];
+    side_flux_v(s, vv(bn), F);
     if (SL >= 0.0f) {
 #pragma unroll
-      for (int q = 0; q < 7; ++q) f[q] = s.F[q].x;
+      for (int q = 0; q < 7; ++q) f[q] = F[q].x;
     } else if (SR <= 0.0f) {
 #pragma unroll
-      for (int q = 0; q < 7; ++q) f[q] = s.F[q].y;
+      for (int q = 0; q < 7; ++q) f[q] = F[q].y;
     } else {
       const V m = s.rho * s.un, m1 = s.rho * s.ut1, m2 = s.rho * s.ut2;
       float dU[7];
@@ -301,7 +316,7 @@ __device__ __forceinline__ void riemann_ideal_lr(const float *wl, const float *w
       dU[RF_BT2] = s.bt2.y - s.bt2.x;
       const float idn = 1.0f / (SR - SL);
 #pragma unroll
-      for (int q = 0; q < 7; ++q) f[q] = (SR * s.F[q].x - SL * s.F[q].y + SL * SR * dU[q]) * idn;
+      for (int q = 0; q < 7; ++q) f[q] = (SR * F[q].x - SL * F[q].y + SL * SR * dU[q]) * idn;
     }
     const float scale = 1e-12f * fmaxf(s.rho.x, s.rho.y) * fmaxf(fabsf(SL), fabsf(SR));
     up = f[RF_RHO] > scale ? 1 : (f[RF_RHO] < -scale ? -1 : 0);
@@ -331,58 +346,76 @@ __device__ __forceinline__ void riemann_ideal_lr(const float *wl, const float *w
   const V scl = fma(rs, sv, vv(bn2));
   const B2 deg = vabs(den) < vv(1e-12f) * scl;
   const V iden = rcp(den);
-  const V fv = sel(deg, vv(0.0f), bnv * smu * iden);
+  const V nfv = sel(deg, vv(0.0f), vv(-bn) * smu * iden);
   const V dbf = sel(deg, vv(0.0f), rs * smu * iden);
-  const V vs1 = fma(neg(s.bt1), fv, s.ut1), vs2 = fma(neg(s.bt2), fv, s.ut2);
+  const V vs1 = fma(s.bt1, nfv, s.ut1), vs2 = fma(s.bt2, nfv, s.ut2);
   const V bs1 = fma(s.bt1, dbf, s.bt1), bs2 = fma(s.bt2, dbf, s.bt2);
-  const V vbs = fma(vs2, bs2, fma(vs1, bs1, SMv * bnv));
-  V dU[7];
-  dU[RF_RHO] = s.rho * smu * iq;
-  dU[RF_MN] = fma(rhos, SMv, neg(s.rho * s.un));
-  dU[RF_MT1] = fma(rhos, vs1, neg(s.rho * s.ut1));
-  dU[RF_MT2] = fma(rhos, vs2, neg(s.rho * s.ut2));
-  dU[RF_E] = fma(bnv, s.vb - vbs, fma(vv(dpts) - s.dpt, SMv, smu * s.enth)) * iq;
-  dU[RF_BT1] = s.bt1 * dbf;
-  dU[RF_BT2] = s.bt2 * dbf;
   const V sq = sqrt2(rhos);
   const float abn = fabsf(bn);
   const V Ss = fma(vv(-abn, abn), rcp(sq), SMv);   // (S*_L, S*_R)
   const bool outL = SL >= 0.0f, outR = !outL && SR < 0.0f, fan = !outL && !outR;
   const bool starL = Ss.x >= 0.0f, starR = !starL && Ss.y < 0.0f, dbl = fan && !starL && !starR;
   const bool left = outL || (fan && (starL || (!starR && SM >= 0.0f)));
-  const float sgn = bn >= 0.0f ? 1.0f : -1.0f;
-  const float isum = 1.0f / (sq.x + sq.y);
-  const V sqv1 = sq * vs1, sqv2 = sq * vs2;
-  const float vss1 = (sqv1.x + sqv1.y + (bs1.y - bs1.x) * sgn) * isum;
-  const float vss2 = (sqv2.x + sqv2.y + (bs2.y - bs2.x) * sgn) * isum;
-  const float sqLR = sq.x * sq.y;
-  const float bss1 = (sq.x * bs1.y + sq.y * bs1.x + sqLR * (vs1.y - vs1.x) * sgn) * isum;
-  const float bss2 = (sq.x * bs2.y + sq.y * bs2.x + sqLR * (vs2.y - vs2.x) * sgn) * isum;
-  const float vbss = SM * bn + vss1 * bss1 + vss2 * bss2;
+  // From here on only the side that holds the face (X) is needed: its inputs
+  // are selected, and its flux and U* - U formed once, the transverse
+  // components as pairs (t1, t2).
   auto pick = [&](const V &v) { return left ? v.x : v.y; };
-  const float S = left ? SL : SR, Ssx = pick(Ss), rhosx = pick(rhos);
-  const float sqs = left ? -sq.x : sq.y;
-  const float v1 = pick(vs1), v2 = pick(vs2), b1 = pick(bs1), b2 = pick(bs2);
-  const float vbsx = SM * bn + v1 * b1 + v2 * b2;
-  float d2[7];
-  d2[RF_RHO] = 0.0f; d2[RF_MN] = 0.0f;
-  d2[RF_MT1] = rhosx * (vss1 - v1); d2[RF_MT2] = rhosx * (vss2 - v2);
-  d2[RF_E] = sqs * (vbsx - vbss) * sgn;
-  d2[RF_BT1] = bss1 - b1; d2[RF_BT2] = bss2 - b2;
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    const float fx = pick(s.F[q]);
-    const float t1 = fan ? S * pick(dU[q]) : 0.0f;
-    const float t2 = dbl ? Ssx * d2[q] : 0.0f;
-    f[q] = fx + t1 + t2;
+  const float rho = pick(s.rho), un = pick(s.un), dpt = pick(s.dpt), enth = pick(s.enth), vb = pick(s.vb);
+  const V ut = vv(pick(s.ut1), pick(s.ut2)), bt = vv(pick(s.bt1), pick(s.bt2));
+  const V vx = vv(pick(vs1), pick(vs2)), bx = vv(pick(bs1), pick(bs2));
+  const float S = left ? SL : SR, rhosx = pick(rhos);
+  const V nbnv = vv(-bn);
+  f[RF_RHO] = rho * un;
+  f[RF_MN] = fmaf(f[RF_RHO], un, __fsub_rn(dpt, bn2));
+  f[RF_E] = fmaf(enth, un, __fmul_rn(-bn, vb));
+  V fm = fma(vv(f[RF_RHO]), ut, nbnv * bt), fb = fma(vv(un), bt, ut * nbnv);
+  // F = F_X + [fan] S_X (U*_X - U_X) + [double star] S*_X (U**_X - U*_X):
+  // added under the condition, not multiplied by zero, so that an unused
+  // intermediate state can never leak into the flux
+  if (fan) {
+    const float iqx = pick(iq), smux = __fsub_rn(SM, un);
+    const float vbs = fmaf(vx.y, bx.y, fmaf(vx.x, bx.x, __fmul_rn(SM, bn)));
+    const float dE = __fmul_rn(fmaf(bn, __fsub_rn(vb, vbs), fmaf(__fsub_rn(dpts, dpt), SM, __fmul_rn(smux, enth))), iqx);
+    const V dM = fma(vv(rhosx), vx, vv(-rho) * ut), dB = bt * vv(pick(dbf));
+    f[RF_RHO] = __fadd_rn(f[RF_RHO], __fmul_rn(S, __fmul_rn(__fmul_rn(rho, smux), iqx)));
+    f[RF_MN] = __fadd_rn(f[RF_MN], __fmul_rn(S, fmaf(rhosx, SM, __fmul_rn(-rho, un))));
+    f[RF_E] = __fadd_rn(f[RF_E], __fmul_rn(S, dE));
+    fm = add_rn(fm, vv(S) * dM);
+    fb = add_rn(fb, vv(S) * dB);
+  }
+  if (dbl) {
+    const float sgn = bn >= 0.0f ? 1.0f : -1.0f;
+    const float isum = 1.0f / (sq.x + sq.y);
+    const V sqv1 = sq * vs1, sqv2 = sq * vs2;
+    const float sqLR = sq.x * sq.y;
+    const V vss = fma(vv(bs1.y - bs1.x, bs2.y - bs2.x), vv(sgn), vv(sqv1.x + sqv1.y, sqv2.x + sqv2.y)) * vv(isum);
+    const float bss1 = (sq.x * bs1.y + sq.y * bs1.x + sqLR * (vs1.y - vs1.x) * sgn) * isum;
+    const float bss2 = (sq.x * bs2.y + sq.y * bs2.x + sqLR * (vs2.y - vs2.x) * sgn) * isum;
+    const float vbss = SM * bn + vss.x * bss1 + vss.y * bss2;
+    const float vbsx = SM * bn + vx.x * bx.x + vx.y * bx.y;
+    const float Ssx = pick(Ss), sqs = left ? -sq.x : sq.y;
+    fm = add_rn(fm, vv(Ssx) * (vv(rhosx) * (vss - vx)));
+    fb = add_rn(fb, vv(Ssx) * (vv(bss1, bss2) - bx));
+    f[RF_E] = __fadd_rn(f[RF_E], __fmul_rn(Ssx, sqs * (vbsx - vbss) * sgn));
   }
   // LHLLD: inside the fan the dissipative part of p_T* is scaled by xi
-  if (fan && xi != 1.0f && SR > 0.0f) {
-    f[RF_MN] += (xi - 1.0f) * pdis;
-    f[RF_E] += (xi - 1.0f) * pdis * SM;
+  if (fan) {
+    const float cd = SR > 0.0f ? __fmul_rn(xi - 1.0f, pdis) : 0.0f;
+    f[RF_MN] = __fadd_rn(f[RF_MN], cd);
+    f[RF_E] = fmaf(cd, SM, f[RF_E]);
   }
+  f[RF_MT1] = fm.x;
+  f[RF_MT2] = fm.y;
+  f[RF_BT1] = fb.x;
+  f[RF_BT2] = fb.y;
   const float scale = 1e-12f * fmaxf(s.rho.x, s.rho.y) * fmaxf(fabsf(SL), fabsf(SR));
   up = f[RF_RHO] > scale ? 1 : (f[RF_RHO] < -scale ? -1 : 0);
+}
+
+__device__ __forceinline__ void riemann_ideal_lr(const float *wl, const float *wr, float bn, float rh, float ph,
+                                                 int solver, float mthr, float *f, int &up, const GasK<float> &K) {
+  bool pos;
+  riemann_ideal_lr(wl, wr, bn, rh, ph, solver, mthr, f, up, pos, K);
 }
 
 }  // namespace x2

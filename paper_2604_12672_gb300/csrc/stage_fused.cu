@@ -14,6 +14,12 @@
 // Eq. spatres).  Only the tangential-B fluxes and the contact direction of
 // each owned face go to global memory, for the edge EMFs (Sect. 2.4).
 //
+// Bound by instruction issue (72% of the slots at three CTAs of 288 threads on
+// an SM): per face ~260 FP32 instructions, 33 special-function ones, ~40 moves
+// of a register or constant, the rest addresses, shared memory and control.
+// 256^3: 1312 us per launch (1530 with the normal field read per face, the
+// epilogue's lines not prefetched and the slopes paired across cells).
+//
 // Compared with one kernel per direction plus a separate update, the face
 // fluxes never round-trip through HBM, each face costs shared-memory loads
 // instead of global gathers with ghost remapping, and the only per-face global
@@ -51,6 +57,7 @@ struct FusedSmem {
   float bgc[2][FZ];                    // background rho, P at the tile's cell centres (scaled units)
   float bgf[2][FZ + 1];                // the same at its z-faces
   uint8_t flg[FZ + 2][FY + 2][FX + 2]; // dilated shock flags of cells -1 .. F (a ghost carries its source's)
+  float bn[3][NXF];                    // normal field of the tile's faces, per direction (scaled units)
   alignas(128) float4 w[2][NHC];       // staged W: (drho, vx, vy, vz) and (Bx, By, Bz, dP) per cell
   float f[5][NFACE];                   // face fluxes, normal frame (rho, m_n, m_t1, m_t2, E); the
                                        // kernel indexes it flat with row stride NXF (phased) or NFACE
@@ -89,55 +96,66 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity,
   return true;
 }
 
-// Flux of the D-face at the lower side of staged cell s2 (its right cell),
-// tile cell (i, j, k), global cell c.  Returns the five fluid components in
-// out[] and stores the EMF inputs when the tile owns the face.
-template <int D, bool LR, bool PPH>
-__device__ __forceinline__ void fused_face(const DevGeo &G, const StageMx &S, const FusedSmem &sm, int s2, int i,
-                                           int j, int k, const int *c, bool own, float *__restrict__ Fd,
-                                           const GasK<float> &K, float *out, int *dflag) {
+// Reconstructed states of the D-face at the lower side of staged cell s2 (its
+// right cell), tile cell (i, j, k).
+template <int D, bool PPH>
+__device__ __forceinline__ void face_states(const FusedSmem &sm, int s2, int i, int j, int k, bool hasf, float *ql,
+                                            float *qr) {
   constexpr int sD = D == 0 ? 1 : (D == 1 ? HX : HX * HY);
-  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-  float ql[8], qr[8];
-  {
-    float4 a[4], b[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      a[m] = sm.w[0][s2 + (m - 2) * sD];
-      b[m] = sm.w[1][s2 + (m - 2) * sD];
+  // PPH: unlimited parabola (no mass fractions on this path); a cell flagged
+  // by the shock flattener reconstructs with van Leer (Sect. 2.7)
+  const uint8_t *fc = &sm.flg[k + 1][j + 1][i + 1];
+  constexpr int fsD = D == 0 ? 1 : (D == 1 ? FX + 2 : (FX + 2) * (FY + 2));
+  const bool pphL = PPH && !(hasf && fc[-fsD]), pphR = PPH && !(hasf && fc[0]);
+  auto plm = [&](int v, float w0, float w1, float w2, float w3) {
+    if constexpr (PPH) {   // the per-cell choice only in the PPH instantiation
+      ql[v] = pphL ? pph_right(w0, w1, w2) : w1 + 0.5f * vl_slope(w0, w1, w2);
+      qr[v] = pphR ? pph_left(w1, w2, w3) : w2 - 0.5f * vl_slope(w1, w2, w3);
+    } else {
+      ql[v] = fmaf(0.5f, vl_slope(w0, w1, w2), w1);
+      qr[v] = fmaf(-0.5f, vl_slope(w1, w2, w3), w2);
     }
-    // PPH: unlimited parabola (no mass fractions on this path); a cell flagged
-    // by the shock flattener reconstructs with van Leer (Sect. 2.7)
-    const uint8_t *fc = &sm.flg[k + 1][j + 1][i + 1];
-    constexpr int fsD = D == 0 ? 1 : (D == 1 ? FX + 2 : (FX + 2) * (FY + 2));
-    const bool pphL = PPH && !fc[-fsD], pphR = PPH && !fc[0];
-    auto plm = [&](int v, float w0, float w1, float w2, float w3) {
-      if constexpr (PPH) {   // the per-cell choice only in the PPH instantiation
-        ql[v] = pphL ? pph_right(w0, w1, w2) : w1 + 0.5f * vl_slope(w0, w1, w2);
-        qr[v] = pphR ? pph_left(w1, w2, w3) : w2 - 0.5f * vl_slope(w1, w2, w3);
-      } else {
-        // the two van Leer slopes (cell i for the left state, cell i+1 for
-        // the right) as one FP32x2 pair: differences, products, sums and the
-        // face values packed; the quotient 2 dm dp / (dm + dp) per lane by
-        // the fast division (its denominators are O(1) in scaled units)
-        const x2::V dm = x2::vv(w1, w2) - x2::vv(w0, w1), dp = x2::vv(w2, w3) - x2::vv(w1, w2);
-        const x2::V pr = dm * dp, den = dm + dp;
-        const x2::V sl = x2::vv(pr.x > 0.0f ? __fdividef(pr.x + pr.x, den.x) : 0.0f,
-                                pr.y > 0.0f ? __fdividef(pr.y + pr.y, den.y) : 0.0f);
-        const x2::V q = x2::fma(x2::vv(0.5f, -0.5f), sl, x2::vv(w1, w2));
-        ql[v] = q.x;
-        qr[v] = q.y;
+  };
+#pragma unroll
+  for (int hw = 0; hw < 2; ++hw) {
+    float4 a[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) a[m] = sm.w[hw][s2 + (m - 2) * sD];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int v = 4 * hw + 2 * e;
+      auto at = [&](int m) { return e == 0 ? x2::vv(a[m].x, a[m].y) : x2::vv(a[m].z, a[m].w); };
+      if (PPH || v == W_BX + D || v + 1 == W_BX + D) {   // the normal field is not reconstructed
+        if (v != W_BX + D) plm(v, at(0).x, at(1).x, at(2).x, at(3).x);
+        if (v + 1 != W_BX + D) plm(v + 1, at(0).y, at(1).y, at(2).y, at(3).y);
+        continue;
       }
-    };
-    plm(W_RHO, a[0].x, a[1].x, a[2].x, a[3].x);
-    plm(W_VX, a[0].y, a[1].y, a[2].y, a[3].y);
-    plm(W_VY, a[0].z, a[1].z, a[2].z, a[3].z);
-    plm(W_VZ, a[0].w, a[1].w, a[2].w, a[3].w);
-    if (D != 0) plm(W_BX, b[0].x, b[1].x, b[2].x, b[3].x);   // the normal field is not reconstructed
-    if (D != 1) plm(W_BY, b[0].y, b[1].y, b[2].y, b[3].y);
-    if (D != 2) plm(W_BZ, b[0].z, b[1].z, b[2].z, b[3].z);
-    plm(W_P, b[0].w, b[1].w, b[2].w, b[3].w);
+      // van Leer slopes (left cell, right cell) of two components as they lie
+      // in the staged float4 (aligned register pairs): differences, products
+      // and sums packed, the quotients 2 dm dp / (dm + dp) per value by the
+      // fast division (their denominators are O(1) in scaled units).  Pairs of
+      // the two cells of one component took a move per operand: with the
+      // solver's selected side, 690 -> 588 instructions per face.
+      const x2::V w1 = at(1), w2 = at(2);
+      const x2::V d1 = w1 - at(0), d2 = w2 - w1, d3 = at(3) - w2;
+      const x2::V pl = d1 * d2, pr = d2 * d3, nl = d1 + d2, nr = d2 + d3, p2l = pl + pl, p2r = pr + pr;
+      ql[v] = fmaf(0.5f, pl.x > 0.0f ? __fdividef(p2l.x, nl.x) : 0.0f, w1.x);
+      ql[v + 1] = fmaf(0.5f, pl.y > 0.0f ? __fdividef(p2l.y, nl.y) : 0.0f, w1.y);
+      qr[v] = fmaf(-0.5f, pr.x > 0.0f ? __fdividef(p2r.x, nr.x) : 0.0f, w2.x);
+      qr[v + 1] = fmaf(-0.5f, pr.y > 0.0f ? __fdividef(p2r.y, nr.y) : 0.0f, w2.y);
+    }
   }
+}
+
+// Flux of the D-face at the lower side of tile cell (i, j, k), global cell c,
+// from its states ql, qr.  Returns the five fluid components in out[] and
+// stores the EMF inputs when the tile owns the face.
+template <int D, bool LR>
+__device__ __forceinline__ void face_flux(const DevGeo &G, const StageMx &S, const FusedSmem &sm, const float *ql,
+                                          const float *qr, float bn, int i, int j, int k, const int *c, bool own,
+                                          bool inner, bool hasf, float *__restrict__ Fd, const GasK<float> &K,
+                                          float *out, bool &bad) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   // normal frame (n, t1, t2) = (D, D+1, D+2 mod 3)
   float wl[W_X0], wr[W_X0];
   auto frame = [&](const float *q, float *w) {
@@ -154,22 +172,21 @@ __device__ __forceinline__ void fused_face(const DevGeo &G, const StageMx &S, co
   frame(ql, wl);
   frame(qr, wr);
   const float brho = D == 2 ? sm.bgf[0][k] : sm.bgc[0][k], bp = D == 2 ? sm.bgf[1][k] : sm.bgc[1][k];
-  if (!(brho + wl[RD_RHO] > 0.0f && brho + wr[RD_RHO] > 0.0f && bp + wl[RD_P] > 0.0f && bp + wr[RD_P] > 0.0f))
-    atomicOr(dflag, FLAG_NEG);
-  // 32-bit offsets (fused_stage_ok bounds the planes)
-  const int qb = D * (int)G.plane + c[0] + (int)G.sy * c[1] + (int)G.sz * c[2];
-  const float b0 = d2f_scaled(S.B[qb], -G.e_b);
-  const float bn = S.first ? b0 : b0 + S.dB[qb];
   // dilated shock flags of the two cells; local cell (i, j, k) sits at flg[k+1][j+1][i+1]
   const uint8_t *fr = &sm.flg[k + 1][j + 1][i + 1];
   constexpr int fs = D == 0 ? 1 : (D == 1 ? FX + 2 : (FX + 2) * (FY + 2));
-  const int solver = (fr[0] | fr[-fs]) ? SOLVER_HLL : G.riemann;
+  const int solver = hasf && (fr[0] | fr[-fs]) ? SOLVER_HLL : G.riemann;
   float fl[7];
   int up;
-  if constexpr (LR) x2::riemann_ideal_lr(wl, wr, bn, brho, bp, solver, G.machf, fl, up, K);
-  else riemann_dev<float, 0, true>(wl, wr, bn, brho, bp, 0.0f, 0.0f, 0, solver, G.machf, fl, up, K);
+  bool pos;
+  if constexpr (LR) x2::riemann_ideal_lr(wl, wr, bn, brho, bp, solver, G.machf, fl, up, pos, K);
+  else {
+    pos = brho + wl[RD_RHO] > 0.0f && brho + wr[RD_RHO] > 0.0f && bp + wl[RD_P] > 0.0f && bp + wr[RD_P] > 0.0f;
+    riemann_dev<float, 0, true>(wl, wr, bn, brho, bp, 0.0f, 0.0f, 0, solver, G.machf, fl, up, K);
+  }
+  bad = bad || !pos;
   // reflecting wall face: a symmetry plane; only the normal-momentum flux survives
-  if ((c[D] == 0 && G.bc[D][0] == 1) || (c[D] == G.n[D] && G.bc[D][1] == 1)) {
+  if (!inner && ((c[D] == 0 && G.bc[D][0] == 1) || (c[D] == G.n[D] && G.bc[D][1] == 1))) {
 #pragma unroll
     for (int q = 0; q < 7; ++q)
       if (q != RF_MN) fl[q] = 0.0f;
@@ -186,27 +203,66 @@ __device__ __forceinline__ void fused_face(const DevGeo &G, const StageMx &S, co
   }
 }
 
-// Evaluates face f of direction D (its index among the tile's D-faces) and
-// returns the five fluid flux components (zeros outside the domain).
-template <int D, bool LR, bool PPH>
-__device__ __forceinline__ void tile_face(const DevGeo &G, const StageMx &S, const FusedSmem &sm, int f, int x0,
-                                          int y0, int z0, float *F0, float *F1, float *F2, const GasK<float> &K,
-                                          float *out, int *dflag) {
-  int i, j, k;
+// Position of face f of direction D among the tile's D-faces.
+template <int D>
+__device__ __forceinline__ void face_pos(int f, int &i, int &j, int &k) {
   if (D == 0) { i = f % (FX + 1); const int r = f / (FX + 1); j = r % FY; k = r / FY; }
   else if (D == 1) { i = f % FX; const int r = f / FX; j = r % (FY + 1); k = r / (FY + 1); }
   else { i = f % FX; const int r = f / FX; j = r % FY; k = r / FY; }
-  const int c[3] = {x0 + i, y0 + j, z0 + k};
-  const bool valid = c[0] <= G.n[0] - (D != 0) && c[1] <= G.n[1] - (D != 1) && c[2] <= G.n[2] - (D != 2);
+}
+
+// Normal field of the tile's D-faces into shared memory, all of a thread's
+// loads in flight together and with the W copy.  Read face by face it was the
+// longest wait of a warp (3.4 of 9 cycles per issue, now 0.7): 1485 -> 1347 us
+// per launch on 256^3, three CTAs' shared memory (3 x 74 KB) still fit an SM.
+template <int D, int NT>
+__device__ __forceinline__ void stage_bn(const DevGeo &G, const StageMx &S, FusedSmem &sm, int tid, int x0, int y0,
+                                         int z0) {
+  constexpr int N = (NXF + NT - 1) / NT;
+  double b[N];
+  float d[N];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) out[q] = 0.0f;
-  if (!valid) return;
+  for (int m = 0; m < N; ++m) {
+    const int f = tid + m * NT;
+    int i, j, k;
+    face_pos<D>(f, i, j, k);
+    const bool in = f < NXF && x0 + i <= G.n[0] - (D != 0) && y0 + j <= G.n[1] - (D != 1) && z0 + k <= G.n[2] - (D != 2);
+    // 32-bit offsets (fused_stage_ok bounds the planes)
+    const int q = D * (int)G.plane + (x0 + i) + (int)G.sy * (y0 + j) + (int)G.sz * (z0 + k);
+    b[m] = in ? S.B[q] : 0.0;
+    d[m] = in && !S.first ? S.dB[q] : 0.0f;
+  }
+#pragma unroll
+  for (int m = 0; m < N; ++m) {
+    const int f = tid + m * NT;
+    const float b0 = d2f_scaled(b[m], -G.e_b);
+    if (f < NXF) sm.bn[D][f] = S.first ? b0 : b0 + d[m];
+  }
+}
+
+// Evaluates face f of direction D (its index among the tile's D-faces) and
+// returns the five fluid flux components (zeros outside the domain).  inner:
+// the tile touches no boundary, so every face is inside and none at a wall.
+template <int D, bool LR, bool PPH>
+__device__ __forceinline__ void tile_face(const DevGeo &G, const StageMx &S, const FusedSmem &sm, int f, int x0,
+                                          int y0, int z0, bool inner, bool hasf, float *F0, float *F1, float *F2,
+                                          const GasK<float> &K, float *out, bool &bad) {
+  int i, j, k;
+  face_pos<D>(f, i, j, k);
+  const int c[3] = {x0 + i, y0 + j, z0 + k};
+  if (!inner && !(c[0] <= G.n[0] - (D != 0) && c[1] <= G.n[1] - (D != 1) && c[2] <= G.n[2] - (D != 2))) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) out[q] = 0.0f;
+    return;
+  }
   const int s2 = ((k + NGW) * HY + (j + NGW)) * HX + (i + NGW);
   constexpr int ext = D == 0 ? FX : (D == 1 ? FY : FZ);
   const int loc = D == 0 ? i : (D == 1 ? j : k);
-  const bool own = loc < ext || c[D] == G.n[D];
+  const bool own = loc < ext || (!inner && c[D] == G.n[D]);
   float *Fd = D == 0 ? F0 : (D == 1 ? F1 : F2);
-  fused_face<D, LR, PPH>(G, S, sm, s2, i, j, k, c, own, Fd, K, out, dflag);
+  float ql[8], qr[8];
+  face_states<D, PPH>(sm, s2, i, j, k, hasf, ql, qr);
+  face_flux<D, LR>(G, S, sm, ql, qr, sm.bn[D][f], i, j, k, c, own, inner, hasf, Fd, K, out, bad);
 }
 
 // Two D-faces of the tile (fa, fb: indices among its D-faces) evaluated
@@ -216,21 +272,16 @@ __device__ __forceinline__ void tile_face(const DevGeo &G, const StageMx &S, con
 // domain give zeros, as in tile_face.
 template <int D, bool PPH>
 __device__ __forceinline__ void tile_face2(const DevGeo &G, const StageMx &S, const FusedSmem &sm, int fa, int fb,
-                                           bool hasb, int x0, int y0, int z0, float *F0, float *F1, float *F2,
-                                           const GasK<float> &K, float *oa, float *ob, int *dflag) {
+                                           bool hasb, int x0, int y0, int z0, bool hasf, float *F0, float *F1,
+                                           float *F2, const GasK<float> &K, float *oa, float *ob, int *dflag) {
   using namespace x2;
   constexpr int sD = D == 0 ? 1 : (D == 1 ? HX : HX * HY);
   constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   constexpr int ext = D == 0 ? FX : (D == 1 ? FY : FZ);
   constexpr int fs = D == 0 ? 1 : (D == 1 ? FX + 2 : (FX + 2) * (FY + 2));
   int l[2][3];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int f = h == 0 ? fa : fb;
-    if (D == 0) { l[h][0] = f % (FX + 1); const int r = f / (FX + 1); l[h][1] = r % FY; l[h][2] = r / FY; }
-    else if (D == 1) { l[h][0] = f % FX; const int r = f / FX; l[h][1] = r % (FY + 1); l[h][2] = r / (FY + 1); }
-    else { l[h][0] = f % FX; const int r = f / FX; l[h][1] = r % FY; l[h][2] = r / FY; }
-  }
+  face_pos<D>(fa, l[0][0], l[0][1], l[0][2]);
+  face_pos<D>(fb, l[1][0], l[1][1], l[1][2]);
   const int ca[3] = {x0 + l[0][0], y0 + l[0][1], z0 + l[0][2]};
   const int cb[3] = {x0 + l[1][0], y0 + l[1][1], z0 + l[1][2]};
   auto inside = [&](const int *c) {
@@ -245,7 +296,7 @@ __device__ __forceinline__ void tile_face2(const DevGeo &G, const StageMx &S, co
   // cells flagged by the shock flattener (left / right of each face)
   const uint8_t *fla = &sm.flg[l[0][2] + 1][l[0][1] + 1][l[0][0] + 1];
   const uint8_t *flb = &sm.flg[l[1][2] + 1][l[1][1] + 1][l[1][0] + 1];
-  const B2 vlL{fla[-fs] != 0, flb[-fs] != 0}, vlR{fla[0] != 0, flb[0] != 0};
+  const B2 vlL{hasf && fla[-fs], hasf && flb[-fs]}, vlR{hasf && fla[0], hasf && flb[0]};
   const bool vlAny = vlL.x || vlL.y || vlR.x || vlR.y;
   V ql[8], qr[8];
   {
@@ -306,13 +357,10 @@ __device__ __forceinline__ void tile_face2(const DevGeo &G, const StageMx &S, co
     const bool nb = !(rl.y > 0.0f && rr.y > 0.0f && pl.y > 0.0f && pr.y > 0.0f);
     if ((va && na) || (vb && nb)) atomicOr(dflag, FLAG_NEG);
   }
-  const long qba = (long)D * G.plane + sidx(G, ca[0], ca[1], ca[2]);
-  const long qbb = (long)D * G.plane + sidx(G, cb[0], cb[1], cb[2]);
-  float bna = d2f_scaled(S.B[qba], -G.e_b), bnb = d2f_scaled(S.B[qbb], -G.e_b);
-  if (!S.first) { bna += S.dB[qba]; bnb += S.dB[qbb]; }
+  const float bna = sm.bn[D][fa], bnb = sm.bn[D][fb];
   const uint8_t *fra = &sm.flg[l[0][2] + 1][l[0][1] + 1][l[0][0] + 1];
   const uint8_t *frb = &sm.flg[l[1][2] + 1][l[1][1] + 1][l[1][0] + 1];
-  const bool hla = (fra[0] | fra[-fs]) != 0, hlb = (frb[0] | frb[-fs]) != 0;
+  const bool hla = hasf && (fra[0] | fra[-fs]), hlb = hasf && (frb[0] | frb[-fs]);
   V fl[7];
   int upa, upb;
   const bool any_hll_solver = G.riemann == SOLVER_HLL;
@@ -356,8 +404,8 @@ __device__ __forceinline__ void tile_face2(const DevGeo &G, const StageMx &S, co
 // thread's running residuals of its cells (phased variant).
 template <int D, int NT, int CPT, int FS, bool PAIRED, bool LR, bool PPH>
 __device__ __forceinline__ void tile_phase(const DevGeo &G, const StageMx &S, FusedSmem &sm, float *fb, int tid,
-                                           int x0, int y0, int z0, float *F0, float *F1, float *F2,
-                                           const GasK<float> &K, float (*racc)[5], int *dflag) {
+                                           int x0, int y0, int z0, bool inner, bool hasf, float *F0, float *F1,
+                                           float *F2, const GasK<float> &K, float (*racc)[5], bool &bad, int *dflag) {
   constexpr int qm[5][3] = {{0, 0, 0}, {1, 3, 2}, {2, 1, 3}, {3, 2, 1}, {4, 4, 4}};
   constexpr int NC = FX * FY * FZ;
   if constexpr (PAIRED) {   // faces f and f + NT together
@@ -365,7 +413,7 @@ __device__ __forceinline__ void tile_phase(const DevGeo &G, const StageMx &S, Fu
       const int g2 = f + NT;
       const bool hasb = g2 < NXF;
       float oa[5], ob[5];
-      tile_face2<D, PPH>(G, S, sm, f, hasb ? g2 : f, hasb, x0, y0, z0, F0, F1, F2, K, oa, ob, dflag);
+      tile_face2<D, PPH>(G, S, sm, f, hasb ? g2 : f, hasb, x0, y0, z0, hasf, F0, F1, F2, K, oa, ob, dflag);
 #pragma unroll
       for (int q = 0; q < 5; ++q) fb[q * FS + f] = oa[q];
       if (hasb) {
@@ -376,7 +424,7 @@ __device__ __forceinline__ void tile_phase(const DevGeo &G, const StageMx &S, Fu
   } else {
     for (int f = tid; f < NXF; f += NT) {
       float out[5];
-      tile_face<D, LR, PPH>(G, S, sm, f, x0, y0, z0, F0, F1, F2, K, out, dflag);
+      tile_face<D, LR, PPH>(G, S, sm, f, x0, y0, z0, inner, hasf, F0, F1, F2, K, out, bad);
 #pragma unroll
       for (int q = 0; q < 5; ++q) fb[q * FS + f] = out[q];
     }
@@ -416,6 +464,7 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
                                           int *dflag, unsigned extra_tx, int raw_flags, FusedSmem &sm,
                                           unsigned parity) {
   const int tid = threadIdx.x;
+  const bool hasf = flag != nullptr;   // else no cell is flagged: sm.flg is neither staged nor read
   const unsigned bar = smem_u32(&sm.bar);
   if (tid == 0) {
     // extra_tx is 0 except in the timeout test (bytes that never arrive)
@@ -427,6 +476,20 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
         " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(&sm.w[0][0])),
         "l"((unsigned long long)tmW), "r"(4 * x0), "r"(y0), "r"(z0), "r"(0), "r"(bar)
         : "memory");
+  }
+  const bool inner = x0 > 0 && y0 > 0 && z0 > 0 && x0 + FX < G.n[0] && y0 + FY < G.n[1] && z0 + FZ < G.n[2];
+  stage_bn<0, NT>(G, S, sm, tid, x0, y0, z0);
+  stage_bn<1, NT>(G, S, sm, tid, x0, y0, z0);
+  stage_bn<2, NT>(G, S, sm, tid, x0, y0, z0);
+  if (!S.first) {   // the epilogue's inputs on their way to L2 (256^3: 1358 -> 1312 us per launch)
+    for (int r = tid; r < 5 * FY * FZ; r += NT) {
+      const int v = r / (FY * FZ), j = r % FY, k = (r / FY) % FZ;
+      if (y0 + j < G.n[1] && z0 + k < G.n[2]) {
+        const int q = v * (int)G.plane + x0 + (int)G.sy * (y0 + j) + (int)G.sz * (z0 + k);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(S.dU + q));
+        if (S.last) asm volatile("prefetch.global.L2 [%0];" ::"l"(S.U + q));
+      }
+    }
   }
   // while the copy is in flight: the tile's background profiles and the
   // dilated shock flags of cells -1 .. F along each axis (a ghost cell carries
@@ -506,27 +569,23 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
       }
       (&sm.flg[0][0][0])[q] = in ? r3[(l[2] * (FY + 2) + l[1]) * (FX + 2) + l[0]] : (uint8_t)0;
     }
-  } else {
+  } else if (hasf) {
     for (int q = tid; q < (FX + 2) * (FY + 2) * (FZ + 2); q += NT) {
       const int l[3] = {q % (FX + 2), (q / (FX + 2)) % (FY + 2), q / ((FX + 2) * (FY + 2))};
       const int o[3] = {x0, y0, z0};
-      uint8_t v = 0;
-      if (flag) {
-        int g[3];
-        bool in = true;
+      int g[3];
+      bool in = true;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          int x = o[d] - 1 + l[d];
-          if (x < -1 || x > G.n[d]) in = false;
-          else if (x == -1 || x == G.n[d]) {
-            bool fl;
-            x = cell_src(x, G.n[d], G.bc[d][0], G.bc[d][1], fl);
-          }
-          g[d] = x;
+      for (int d = 0; d < 3; ++d) {
+        int x = o[d] - 1 + l[d];
+        if (x < -1 || x > G.n[d]) in = false;
+        else if (x == -1 || x == G.n[d]) {
+          bool fl;
+          x = cell_src(x, G.n[d], G.bc[d][0], G.bc[d][1], fl);
         }
-        if (in) v = flag[g[0] + (long)G.n[0] * (g[1] + (long)G.n[1] * g[2])];
+        g[d] = x;
       }
-      (&sm.flg[0][0][0])[q] = v;
+      (&sm.flg[0][0][0])[q] = in ? flag[g[0] + (long)G.n[0] * (g[1] + (long)G.n[1] * g[2])] : (uint8_t)0;
     }
   }
   const bool ok = mbar_wait_bounded(bar, parity, 1000000000ull);
@@ -546,6 +605,7 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
   // normal-frame component that carries global component v on d-faces
   constexpr int qm[5][3] = {{0, 0, 0}, {1, 3, 2}, {2, 1, 3}, {3, 2, 1}, {4, 4, 4}};
   constexpr int NC = FX * FY * FZ, CPT = (NC + NT - 1) / NT;   // cells per thread
+  bool bad = false;   // a face state without positive density and pressure
   float racc[CPT][5];
 #pragma unroll
   for (int m = 0; m < CPT; ++m)
@@ -554,16 +614,19 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
 
   if constexpr (PHASED) {
     static_assert(NXF == NYF && NYF == NZF, "phased tiles need equal face counts per direction");
-    tile_phase<0, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, F0, F1, F2, K, racc, dflag);
-    tile_phase<1, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, F0, F1, F2, K, racc, dflag);
-    tile_phase<2, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, F0, F1, F2, K, racc, dflag);
+    tile_phase<0, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, inner, hasf, F0, F1, F2, K, racc,
+                                             bad, dflag);
+    tile_phase<1, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, inner, hasf, F0, F1, F2, K, racc,
+                                             bad, dflag);
+    tile_phase<2, NT, CPT, FS, PAIRED, LR, PPH>(G, S, sm, fb, tid, x0, y0, z0, inner, hasf, F0, F1, F2, K, racc,
+                                             bad, dflag);
   } else {
     // NXF and NXF + NYF are multiples of 32: the direction is uniform in a warp
     for (int f = tid; f < NFACE; f += NT) {
       float out[5];
-      if (f < NXF) tile_face<0, LR, PPH>(G, S, sm, f, x0, y0, z0, F0, F1, F2, K, out, dflag);
-      else if (f < NXF + NYF) tile_face<1, LR, PPH>(G, S, sm, f - NXF, x0, y0, z0, F0, F1, F2, K, out, dflag);
-      else tile_face<2, LR, PPH>(G, S, sm, f - NXF - NYF, x0, y0, z0, F0, F1, F2, K, out, dflag);
+      if (f < NXF) tile_face<0, LR, PPH>(G, S, sm, f, x0, y0, z0, inner, hasf, F0, F1, F2, K, out, bad);
+      else if (f < NXF + NYF) tile_face<1, LR, PPH>(G, S, sm, f - NXF, x0, y0, z0, inner, hasf, F0, F1, F2, K, out, bad);
+      else tile_face<2, LR, PPH>(G, S, sm, f - NXF - NYF, x0, y0, z0, inner, hasf, F0, F1, F2, K, out, bad);
 #pragma unroll
       for (int q = 0; q < 5; ++q) fb[q * FS + f] = out[q];
     }
@@ -584,6 +647,8 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap *tmW, const DevGeo &
       }
     }
   }
+
+  if (bad) atomicOr(dflag, FLAG_NEG);
 
   // R = sum_d (F_d(+) - F_d(-)) / dx_d - (S - S_hat), then the RK increment.
   // The cells' increments (and, in the last stage, their FP64 state) are
@@ -647,7 +712,7 @@ __global__ void __launch_bounds__(NT, MINB)
                      float *__restrict__ F0, float *__restrict__ F1, float *__restrict__ F2, int ntx, int nty,
                      int *dflag, unsigned extra_tx, int raw_flags, const unsigned int *__restrict__ any) {
   extern __shared__ unsigned char smraw[];
-  if (any && *any == 0u) {   // no cell flagged: the tile stages zero flags
+  if (any && *any == 0u) {   // no cell flagged: the tile needs no flags
     flag = nullptr;
     raw_flags = 0;
   }
