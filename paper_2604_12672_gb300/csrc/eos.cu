@@ -142,6 +142,7 @@ phl_status phl_eos_table_create(double lrhoye_lo, double lrhoye_hi, int nrho, do
   gauss_legendre(GLN, gxw, gxw + GLN);
   cudaError_t e = cudaSuccess;
   phl_eos_table *t = new phl_eos_table();
+  scratch_owner(1);
   t->t.nx = nrho;
   t->t.ny = nT;
   t->t.x0 = log(pow(10.0, lrhoye_lo) * NAV);
@@ -195,6 +196,7 @@ void phl_eos_table_destroy(phl_eos_table *t) {
   cudaFree(t->dc);
   cudaFree(t->dcf);
   delete t;
+  scratch_owner(-1);
 }
 
 phl_status phl_eos_table_export(const phl_eos_table *t, double *out, long nout) {
@@ -217,11 +219,11 @@ phl_status phl_eos(const phl_eos_table *t, long n, const double *rho, const doub
   const double *drho = rho, *dein = eint, *dab = abar, *dye = ye;
   double *dT = T_inout, *dP = P, *dge = gamma_e, *dgc = gamma_c, *dcs = cs;
   int *dit = iters;
-  void *buf = nullptr;
+  CallScratch buf;
   if (where == PHL_HOST) {   // stage through one device buffer
     const size_t nb = (size_t)n * (9 * sizeof(double) + sizeof(int));
-    if (cudaMalloc(&buf, nb) != cudaSuccess) { cudaGetLastError(); return (phl_status)set_error(PHL_ENOMEM, "phl_eos: alloc"); }
-    double *b = (double *)buf;
+    if (buf.get(nb, s) != cudaSuccess) { cudaGetLastError(); return (phl_status)set_error(PHL_ENOMEM, "phl_eos: alloc"); }
+    double *b = (double *)buf.p;
     double *a[9];
     for (int k = 0; k < 9; ++k) a[k] = b + (size_t)k * n;
     cudaMemcpyAsync(a[0], rho, n * 8, cudaMemcpyHostToDevice, s);
@@ -249,7 +251,6 @@ phl_status phl_eos(const phl_eos_table *t, long n, const double *rho, const doub
       if (iters) cudaMemcpyAsync(iters, dit, n * sizeof(int), cudaMemcpyDeviceToHost, s);
       e = cudaStreamSynchronize(s);
     }
-    cudaFree(buf);
   }
   if (e != cudaSuccess) return (phl_status)set_error(PHL_ECUDA, "phl_eos: %s", cudaGetErrorString(e));
   return PHL_OK;

@@ -298,20 +298,22 @@ cudaError_t build_fragments(phl_mlp *M) {
   return e;
 }
 
-// Scratch of one training batch (feature-major activations and errors).
+// Scratch of one training batch (the loss sum, feature-major activations and
+// errors) and `extra` floats for the caller, in one piece.
 struct Scratch {
-  float *H1 = nullptr, *H2 = nullptr, *D1 = nullptr, *D2 = nullptr, *dy = nullptr;
+  float *H1 = nullptr, *H2 = nullptr, *D1 = nullptr, *D2 = nullptr, *dy = nullptr, *extra = nullptr;
   double *loss = nullptr;
-  long cap = 0;
-  cudaError_t alloc(long nb) {
-    cap = nb;
-    float *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, (4 * NH + 1) * nb * sizeof(float));
+  CallScratch room;
+  cudaError_t alloc(long nb, long nextra) {
+    constexpr size_t HEAD = 256;   // the loss sum; keeps the arrays aligned
+    cudaError_t e = room.get(HEAD + ((4 * NH + 1) * nb + nextra) * sizeof(float), 0);
     if (e != cudaSuccess) return e;
-    H1 = p; H2 = p + NH * nb; D1 = p + 2 * NH * nb; D2 = p + 3 * NH * nb; dy = p + 4 * NH * nb;
-    return cudaMalloc(&loss, sizeof(double));
+    loss = (double *)room.p;
+    extra = (float *)((char *)room.p + HEAD);
+    H1 = extra + nextra;
+    H2 = H1 + NH * nb; D1 = H1 + 2 * NH * nb; D2 = H1 + 3 * NH * nb; dy = H1 + 4 * NH * nb;
+    return e;
   }
-  ~Scratch() { cudaFree(H1); cudaFree(loss); }
 };
 
 // grad <- d loss / d w over nb samples (normalised x, t on the device); loss
@@ -348,11 +350,12 @@ phl_status phl_mlp_create(unsigned long long seed, phl_mlp **out) {
   if (!out) return (phl_status)set_error(PHL_EINVAL, "phl_mlp_create: null out");
   *out = nullptr;
   phl_mlp *M = new phl_mlp();
+  scratch_owner(1);
   cudaError_t e = cudaMalloc(&M->w, 4 * NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&M->frag, F_TOTAL * sizeof(uint2));
   if (e == cudaSuccess) e = cudaMalloc(&M->bias, 2 * NH * sizeof(float));
   if (e != cudaSuccess) {
-    cudaFree(M->w); cudaFree(M->frag); cudaFree(M->bias); delete M;
+    phl_mlp_destroy(M);
     return (phl_status)set_error(PHL_ENOMEM, "phl_mlp_create: %s", cudaGetErrorString(e));
   }
   M->m = M->w + NPARAM;
@@ -382,6 +385,7 @@ void phl_mlp_destroy(phl_mlp *M) {
   cudaFree(M->frag);
   cudaFree(M->bias);
   delete M;
+  scratch_owner(-1);
 }
 
 phl_status phl_mlp_set_weights(phl_mlp *M, const float *w) {
@@ -421,17 +425,14 @@ phl_status phl_mlp_loss_grad(phl_mlp *M, long n, const float *x, const float *t,
   if (!M || n <= 0 || !x || !t || !loss || !grad)
     return (phl_status)set_error(PHL_EINVAL, "phl_mlp_loss_grad: bad arguments");
   const float *dx = x, *dt = t;
-  float *tmp = nullptr;
-  cudaError_t e = cudaSuccess;
-  if (where == PHL_HOST) {
-    e = cudaMalloc(&tmp, 4 * n * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemcpy(tmp, x, 3 * n * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(tmp + 3 * n, t, n * sizeof(float), cudaMemcpyHostToDevice);
-    dx = tmp;
-    dt = tmp + 3 * n;
-  }
   Scratch S;
-  if (e == cudaSuccess) e = S.alloc(n);
+  cudaError_t e = S.alloc(n, where == PHL_HOST ? 4 * n : 0);
+  if (e == cudaSuccess && where == PHL_HOST) {
+    e = cudaMemcpy(S.extra, x, 3 * n * sizeof(float), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(S.extra + 3 * n, t, n * sizeof(float), cudaMemcpyHostToDevice);
+    dx = S.extra;
+    dt = S.extra + 3 * n;
+  }
   if (e == cudaSuccess) {
     launch_loss_grad(M, n, dx, dt, S, 0);
     e = cudaGetLastError();
@@ -441,7 +442,7 @@ phl_status phl_mlp_loss_grad(phl_mlp *M, long n, const float *x, const float *t,
   if (e == cudaSuccess)
     e = cudaMemcpy(grad, M->grad, NPARAM * sizeof(float),
                    where == PHL_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice);
-  cudaFree(tmp);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();   // a copy within the device does not wait
   if (e != cudaSuccess) return cuda_status(e, "phl_mlp_loss_grad");
   *loss = l / (double)n;
   return PHL_OK;
@@ -450,10 +451,12 @@ phl_status phl_mlp_loss_grad(phl_mlp *M, long n, const float *x, const float *t,
 phl_status phl_mlp_forward(const phl_mlp *M, long n, const float *x, float *y, int where) {
   if (!M || n <= 0 || !x || !y) return (phl_status)set_error(PHL_EINVAL, "phl_mlp_forward: bad arguments");
   const float *dx = x;
-  float *dy = y, *tmp = nullptr;
+  float *dy = y;
+  CallScratch room;
   cudaError_t e = cudaSuccess;
   if (where == PHL_HOST) {
-    e = cudaMalloc(&tmp, 4 * n * sizeof(float));
+    e = room.get(4 * n * sizeof(float), 0);
+    float *tmp = (float *)room.p;
     if (e == cudaSuccess) e = cudaMemcpy(tmp, x, 3 * n * sizeof(float), cudaMemcpyHostToDevice);
     dx = tmp;
     dy = tmp + 3 * n;
@@ -464,7 +467,6 @@ phl_status phl_mlp_forward(const phl_mlp *M, long n, const float *x, float *y, i
   }
   if (e == cudaSuccess && where == PHL_HOST) e = cudaMemcpy(y, dy, n * sizeof(float), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  cudaFree(tmp);
   return e == cudaSuccess ? PHL_OK : cuda_status(e, "phl_mlp_forward");
 }
 
@@ -475,10 +477,12 @@ phl_status phl_mlp_guess_temperature(const phl_mlp *M, const phl_eos_table *tab,
   const eos::Table &t = *eos_table_view(tab);
   const double Tlo = exp(t.y0), Thi = exp(t.y0 + (t.ny - 1) * t.dy);
   const double *dr = rho, *de = eint, *dx = X0;
-  double *dT = T, *tmp = nullptr;
+  double *dT = T;
+  CallScratch room;
   cudaError_t e = cudaSuccess;
   if (where == PHL_HOST) {
-    e = cudaMalloc(&tmp, 4 * n * sizeof(double));
+    e = room.get(4 * n * sizeof(double), 0);
+    double *tmp = (double *)room.p;
     if (e == cudaSuccess) e = cudaMemcpy(tmp, rho, n * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(tmp + n, eint, n * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(tmp + 2 * n, X0, n * 8, cudaMemcpyHostToDevice);
@@ -490,7 +494,6 @@ phl_status phl_mlp_guess_temperature(const phl_mlp *M, const phl_eos_table *tab,
   }
   if (e == cudaSuccess && where == PHL_HOST) e = cudaMemcpy(T, dT, n * 8, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  cudaFree(tmp);
   return e == cudaSuccess ? PHL_OK : cuda_status(e, "phl_mlp_guess_temperature");
 }
 
@@ -511,7 +514,7 @@ phl_status phl_mlp_train(phl_mlp *M, const phl_eos_table *tab, const phl_mlp_tra
   if (e == cudaSuccess) e = cudaMalloc(&fail, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&mm, 2 * sizeof(unsigned int));
   Scratch S;
-  if (e == cudaSuccess) e = S.alloc(cfg->batch);
+  if (e == cudaSuccess) e = S.alloc(cfg->batch, 0);
   phl_status ret = PHL_OK;
   auto done = [&](phl_status r) {
     cudaFree(x); cudaFree(tt); cudaFree(pred); cudaFree(fail); cudaFree(mm);

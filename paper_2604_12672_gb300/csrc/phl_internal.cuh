@@ -461,6 +461,21 @@ __host__ __device__ __forceinline__ double iusc(const DevGeo &G, int v) {
 // returns st (phl_api.cu).
 int set_error(int st, const char *fmt, ...);
 
+// Device scratch of one call on host arrays, from the device's pool
+// (scratch.cu): given back to it in stream order when the call returns.
+struct CallScratch {
+  void *p = nullptr;
+  cudaStream_t s = nullptr;
+  CallScratch() = default;
+  CallScratch(const CallScratch &) = delete;
+  CallScratch &operator=(const CallScratch &) = delete;
+  cudaError_t get(size_t bytes, cudaStream_t stream);
+  ~CallScratch();
+};
+// +1 for an EOS table or network made, -1 for one destroyed: the pools keep
+// nothing once the last is gone.
+void scratch_owner(int change);
+
 // FP64 multi-kernel stage (kernels_fp64.cu)
 void launch_stage_fp64(const DevGeo &G, const StageBufs &B, cudaStream_t s, int *nlaunch, Prof *prof);
 void launch_dt_fp64(const DevGeo &G, const double *U, const double *Bf, double *T, unsigned long long *dmax,
