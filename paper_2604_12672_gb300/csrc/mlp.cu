@@ -9,6 +9,7 @@
 // of the mapped target.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -95,127 +96,203 @@ __global__ void k_minmax_e(long n, const float *x, unsigned int *mn, unsigned in
   atomicMax(mx, hi);
 }
 
-// Forward + backward of one sample per thread in FP32 (weights in shared
-// memory, rounded to BF16 as in inference: straight-through gradient).  Writes per-sample activations and back-propagated errors in
-// feature-major layout [NH][nb] for the weight-gradient reduction.
-constexpr int FB_THREADS = 128;
-__global__ void __launch_bounds__(FB_THREADS) k_fwd_bwd(const float *__restrict__ w, long nb,
-                                                        const float *__restrict__ x, const float *__restrict__ t,
-                                                        float inv_n, float *H1, float *H2, float *D1, float *D2,
-                                                        float *dy_out, double *loss) {
-  // the weight matrices as the inference sees them (rounded to BF16), the
-  // biases in FP32; the gradient updates the FP32 master weights
-  __shared__ float sw[NPARAM];
-  for (int k = threadIdx.x; k < NPARAM; k += blockDim.x) {
-    const bool is_w = k < O_B1 || (k >= O_W2 && k < O_B2) || (k >= O_W3 && k < O_B3);
-    sw[k] = is_w ? __bfloat162float(__float2bfloat16_rn(w[k])) : w[k];
-  }
-  __syncthreads();
-  const long s = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  float r2 = 0.0f;
-  if (s < nb) {
-    const float x0 = x[3 * s], x1 = x[3 * s + 1], x2 = x[3 * s + 2];
-    float h1[NH];
-#pragma unroll
-    for (int a = 0; a < NH; ++a) {
-      const float z = sw[O_B1 + a] + sw[O_W1 + 3 * a] * x0 + sw[O_W1 + 3 * a + 1] * x1 + sw[O_W1 + 3 * a + 2] * x2;
-      h1[a] = tanhf(z);
-      H1[(long)a * nb + s] = h1[a];
-    }
-    float y = sw[O_B3];
-    for (int a = 0; a < NH; ++a) {
-      float z = sw[O_B2 + a];
-#pragma unroll
-      for (int b = 0; b < NH; ++b) z += sw[O_W2 + a * NH + b] * h1[b];
-      const float h2 = tanhf(z);
-      H2[(long)a * nb + s] = h2;
-      y += sw[O_W3 + a] * h2;
-    }
-    const float r = y - t[s];
-    r2 = r * r;
-    const float dy = 2.0f * r * inv_n;
-    dy_out[s] = dy;
-    float d1[NH];
-#pragma unroll
-    for (int b = 0; b < NH; ++b) d1[b] = 0.0f;
-    for (int a = 0; a < NH; ++a) {
-      const float h2 = H2[(long)a * nb + s];
-      const float d2 = dy * sw[O_W3 + a] * (1.0f - h2 * h2);
-      D2[(long)a * nb + s] = d2;
-#pragma unroll
-      for (int b = 0; b < NH; ++b) d1[b] += sw[O_W2 + a * NH + b] * d2;
-    }
-#pragma unroll
-    for (int b = 0; b < NH; ++b) D1[(long)b * nb + s] = d1[b] * (1.0f - h1[b] * h1[b]);
-  }
-  for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, (double)r2);
-}
+// Loss and weight gradient in FP32 (weights in shared memory, rounded to BF16
+// as in inference: straight-through gradient).  A block takes tiles of LG_S
+// samples: first layer, second layer (64 x 64 times the tile), output and
+// residual, the back-propagated errors (the transposed product) and the
+// tile's weight gradient D2 H1^T, which stays in registers over the block's
+// tiles and is added to grad at the end.
+// Bound by FP32 issue: 12288 multiply-adds per sample in the three products.
+// Each thread forms 8 x 4 (4 x 8 in the last) of a product from 16-byte
+// shared-memory reads, 10.7 multiply-adds per read; one sample per thread had
+// one read per four, and the activations and errors made a round trip of
+// 1 KB per sample through memory to a second kernel.  65536 samples:
+// 68 us instead of 84 + 53.  The rows a thread takes are spread so that the
+// eight lanes of a read phase fall into different banks (row stride 68).
+constexpr int LG_T = 128, LG_S = 64, LG_LD = 68;
+struct LossGradSmem {
+  float w2[NH][LG_LD];   // W2[a][b]
+  float h1[NH][LG_LD];   // h1[b][s]
+  float d2[NH][LG_LD];   // d2[a][s]
+  float w1[NH * NIN], b1[NH], b2[NH], w3[NH], b3;
+  alignas(16) float x[NIN][LG_S];
+  float t[LG_S];
+  float row[LG_T / 32][6][NH];   // per warp: sums over the samples of d2, dy h2, d1, d1 x
+};
+static_assert(offsetof(LossGradSmem, w2) % 16 == 0 && offsetof(LossGradSmem, h1) % 16 == 0 &&
+                  offsetof(LossGradSmem, d2) % 16 == 0 && offsetof(LossGradSmem, x) % 16 == 0 && LG_LD % 4 == 0 &&
+                  LG_S % 4 == 0,
+              "rows read by float4");
+constexpr size_t LG_SMEM = sizeof(LossGradSmem);
 
-// Weight gradients: sums over the samples of a chunk, one 4x4 block of dW2 per
-// thread (256 threads = 64 x 64), plus the bias, W1 and W3 sums; partial sums
-// are added to grad with atomics.
-constexpr int RED_CHUNK = 32;
-__global__ void __launch_bounds__(256) k_grad_reduce(long nb, const float *__restrict__ x, const float *H1,
-                                                     const float *H2, const float *D1, const float *D2,
-                                                     const float *dy, float *grad) {
-  __shared__ float sH1[RED_CHUNK][NH + 4], sD2[RED_CHUNK][NH + 4];
-  __shared__ float sH2[RED_CHUNK][NH + 1], sD1[RED_CHUNK][NH + 1];
-  __shared__ float sx[RED_CHUNK][3], sdy[RED_CHUNK];
-  const int tid = threadIdx.x;
-  const int tj = tid >> 4, tk = tid & 15;   // dW2 rows 4 tj.., cols 4 tk..
-  float acc[4][4] = {};
-  float accb1 = 0.f, accb2 = 0.f, accw3 = 0.f, accw1[3] = {0.f, 0.f, 0.f}, accb3 = 0.f;
-  for (long s0 = (long)blockIdx.x * RED_CHUNK; s0 < nb; s0 += (long)gridDim.x * RED_CHUNK) {
-    const int cnt = (int)min((long)RED_CHUNK, nb - s0);
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float elem(const float4 &v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
+
+__global__ void __launch_bounds__(LG_T, 3) k_loss_grad(const float *__restrict__ w, long nb,
+                                                       const float *__restrict__ x, const float *__restrict__ t,
+                                                       float inv_n, float *__restrict__ grad, double *loss) {
+  extern __shared__ __align__(16) unsigned char lg_raw[];
+  LossGradSmem &sm = *reinterpret_cast<LossGradSmem *>(lg_raw);
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the weight matrices as the inference sees them, the biases in FP32; the
+  // gradient updates the FP32 master weights
+  auto bf = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
+  for (int k = tid; k < NH * NH; k += LG_T) sm.w2[k / NH][k % NH] = bf(w[O_W2 + k]);
+  for (int k = tid; k < NH * NIN; k += LG_T) sm.w1[k] = bf(w[O_W1 + k]);
+  if (tid < NH) {
+    sm.b1[tid] = w[O_B1 + tid];
+    sm.b2[tid] = w[O_B2 + tid];
+    sm.w3[tid] = bf(w[O_W3 + tid]);
+  }
+  if (tid == 0) sm.b3 = w[O_B3];
+  const int rg = tid & 7, s4 = 4 * (tid >> 3);       // products 1, 2: row group, first of four samples
+  const int gb = tid & 7, ga = tid >> 3;             // product 3: columns gb + 8 j, rows ga + 16 i
+  float gw[4][8] = {}, gb3 = 0.0f, r2 = 0.0f;
+  // per-row sums: over the warp's four sample groups, then into the warp's own
+  // row of shared memory (48 registers less than keeping them per thread)
+  float (*row)[NH] = sm.row[tid >> 5];
+  for (int k = lane; k < 6 * NH; k += 32) (&row[0][0])[k] = 0.0f;
+  __syncwarp();
+  auto rows = [&](float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    return v + __shfl_xor_sync(0xffffffffu, v, 16);
+  };
+  auto add_row = [&](float *dst, float v) {
+    v = rows(v);
+    if (lane < 8) *dst += v;
+  };
+  for (long s0 = (long)blockIdx.x * LG_S; s0 < nb; s0 += (long)gridDim.x * LG_S) {
+    const int cnt = (int)min((long)LG_S, nb - s0);
+    __syncthreads();   // the previous tile's readers are done
+    for (int e = tid; e < NIN * LG_S; e += LG_T) sm.x[e % NIN][e / NIN] = e < NIN * cnt ? x[NIN * s0 + e] : 0.0f;
+    if (tid < LG_S) sm.t[tid] = tid < cnt ? t[s0 + tid] : 0.0f;
     __syncthreads();
-    for (int e = tid; e < RED_CHUNK * NH; e += blockDim.x) {
-      const int a = e / RED_CHUNK, ss = e % RED_CHUNK;
-      const bool in = ss < cnt;
-      const long gi = (long)a * nb + s0 + ss;
-      sH1[ss][a] = in ? H1[gi] : 0.f;
-      sD2[ss][a] = in ? D2[gi] : 0.f;
-      sH2[ss][a] = in ? H2[gi] : 0.f;
-      sD1[ss][a] = in ? D1[gi] : 0.f;
-    }
-    for (int e = tid; e < RED_CHUNK; e += blockDim.x) {
-      const bool in = e < cnt;
-      sdy[e] = in ? dy[s0 + e] : 0.f;
-      for (int c = 0; c < 3; ++c) sx[e][c] = in ? x[3 * (s0 + e) + c] : 0.f;
+    {
+      const int ss = tid & (LG_S - 1), b0 = (tid / LG_S) * (NH / 2);
+      const float x0 = sm.x[0][ss], x1 = sm.x[1][ss], x2 = sm.x[2][ss];
+      for (int b = b0; b < b0 + NH / 2; ++b)
+        sm.h1[b][ss] = tanhf(sm.b1[b] + sm.w1[3 * b] * x0 + sm.w1[3 * b + 1] * x1 + sm.w1[3 * b + 2] * x2);
     }
     __syncthreads();
-    for (int ss = 0; ss < RED_CHUNK; ++ss) {
-      float dv[4], hv[4];
+    {   // z[a][s] = b2 + sum_b W2[a][b] h1[b][s], rows a = rg + 8 i
+      float z[8][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { dv[i] = sD2[ss][4 * tj + i]; hv[i] = sH1[ss][4 * tk + i]; }
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int q = 0; q < 4; ++q) z[i][q] = sm.b2[rg + 8 * i];
+#pragma unroll 4
+      for (int k = 0; k < NH; k += 4) {
+        float4 h[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += dv[i] * hv[j];
-    }
-    if (tid < NH) {
-      for (int ss = 0; ss < RED_CHUNK; ++ss) {
-        const float d1 = sD1[ss][tid];
-        accb1 += d1;
-        for (int c = 0; c < 3; ++c) accw1[c] += d1 * sx[ss][c];
-        accb2 += sD2[ss][tid];
-        accw3 += sdy[ss] * sH2[ss][tid];
+        for (int q = 0; q < 4; ++q) h[q] = ld4(&sm.h1[k + q][s4]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 a = ld4(&sm.w2[rg + 8 * i][k]);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z[i][q] += elem(a, kk) * elem(h[kk], q);
+        }
       }
-    } else if (tid == NH) {
-      for (int ss = 0; ss < RED_CHUNK; ++ss) accb3 += sdy[ss];
+      float y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          z[i][q] = tanhf(z[i][q]);
+          y[q] += sm.w3[rg + 8 * i] * z[i][q];
+        }
+      float dy[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        for (int o = 1; o < 8; o <<= 1) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
+        const float r = s4 + q < cnt ? sm.b3 + y[q] - sm.t[s4 + q] : 0.0f;   // no contribution beyond the batch
+        dy[q] = 2.0f * r * inv_n;
+        if (rg == 0) {
+          r2 += r * r;
+          gb3 += dy[q];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float w3 = sm.w3[rg + 8 * i];
+        float d[4], gb2 = 0.0f, gw3 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          d[q] = dy[q] * w3 * (1.0f - z[i][q] * z[i][q]);
+          gb2 += d[q];
+          gw3 += dy[q] * z[i][q];
+        }
+        add_row(&row[0][rg + 8 * i], gb2);
+        add_row(&row[1][rg + 8 * i], gw3);
+        *reinterpret_cast<float4 *>(&sm.d2[rg + 8 * i][s4]) = make_float4(d[0], d[1], d[2], d[3]);
+      }
+    }
+    __syncthreads();
+    {   // d1[b][s] = (1 - h1^2) sum_a W2[a][b] d2[a][s], rows b = 4 rg + i and 32 + 4 rg + i
+      float d1[8][4] = {};
+#pragma unroll 16
+      for (int k = 0; k < NH; ++k) {
+        const float4 a0 = ld4(&sm.w2[k][4 * rg]), a1 = ld4(&sm.w2[k][32 + 4 * rg]), d = ld4(&sm.d2[k][s4]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            d1[i][q] += elem(a0, i) * elem(d, q);
+            d1[4 + i][q] += elem(a1, i) * elem(d, q);
+          }
+      }
+      float4 xs[NIN];
+#pragma unroll
+      for (int c = 0; c < NIN; ++c) xs[c] = ld4(&sm.x[c][s4]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int b = (i < 4 ? 0 : 28) + 4 * rg + i;
+        const float4 h = ld4(&sm.h1[b][s4]);
+        float gb1 = 0.0f, gw1[NIN] = {};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float v = d1[i][q] * (1.0f - elem(h, q) * elem(h, q));
+          gb1 += v;
+#pragma unroll
+          for (int c = 0; c < NIN; ++c) gw1[c] += v * elem(xs[c], q);
+        }
+        add_row(&row[2][b], gb1);
+#pragma unroll
+        for (int c = 0; c < NIN; ++c) add_row(&row[3 + c][b], gw1[c]);
+      }
+    }
+    // dW2[a][b] += sum_s d2[a][s] h1[b][s]
+#pragma unroll 4
+    for (int k = 0; k < LG_S; k += 4) {
+      float4 d[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[i] = ld4(&sm.d2[ga + 16 * i][k]);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 h = ld4(&sm.h1[gb + 8 * j][k]);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) gw[i][j] += elem(d[i], kk) * elem(h, kk);
+      }
     }
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) atomicAdd(&grad[O_W2 + (4 * tj + i) * NH + 4 * tk + j], acc[i][j]);
-  if (tid < NH) {
-    atomicAdd(&grad[O_B1 + tid], accb1);
-    for (int c = 0; c < 3; ++c) atomicAdd(&grad[O_W1 + 3 * tid + c], accw1[c]);
-    atomicAdd(&grad[O_B2 + tid], accb2);
-    atomicAdd(&grad[O_W3 + tid], accw3);
-  } else if (tid == NH) {
-    atomicAdd(&grad[O_B3], accb3);
+    for (int j = 0; j < 8; ++j) atomicAdd(&grad[O_W2 + (ga + 16 * i) * NH + gb + 8 * j], gw[i][j]);
+  __syncwarp();
+  for (int k = lane; k < 6 * NH; k += 32) {
+    const int m = k / NH, a = k % NH;
+    const int o = m == 0 ? O_B2 + a : (m == 1 ? O_W3 + a : (m == 2 ? O_B1 + a : O_W1 + 3 * a + m - 3));
+    atomicAdd(&grad[o], row[m][a]);
+  }
+  gb3 = rows(gb3);
+  r2 = rows(r2);
+  if (lane == 0) {
+    atomicAdd(&grad[O_B3], gb3);
+    atomicAdd(loss, (double)r2);
   }
 }
 
@@ -298,34 +375,17 @@ cudaError_t build_fragments(phl_mlp *M) {
   return e;
 }
 
-// Scratch of one training batch (the loss sum, feature-major activations and
-// errors) and `extra` floats for the caller, in one piece.
-struct Scratch {
-  float *H1 = nullptr, *H2 = nullptr, *D1 = nullptr, *D2 = nullptr, *dy = nullptr, *extra = nullptr;
-  double *loss = nullptr;
-  CallScratch room;
-  cudaError_t alloc(long nb, long nextra) {
-    constexpr size_t HEAD = 256;   // the loss sum; keeps the arrays aligned
-    cudaError_t e = room.get(HEAD + ((4 * NH + 1) * nb + nextra) * sizeof(float), 0);
-    if (e != cudaSuccess) return e;
-    loss = (double *)room.p;
-    extra = (float *)((char *)room.p + HEAD);
-    H1 = extra + nextra;
-    H2 = H1 + NH * nb; D1 = H1 + 2 * NH * nb; D2 = H1 + 3 * NH * nb; dy = H1 + 4 * NH * nb;
-    return e;
-  }
-};
-
 // grad <- d loss / d w over nb samples (normalised x, t on the device); loss
 // (device double) receives the sum of squared residuals.
-void launch_loss_grad(phl_mlp *M, long nb, const float *x, const float *t, Scratch &S, cudaStream_t s) {
+cudaError_t launch_loss_grad(phl_mlp *M, long nb, const float *x, const float *t, double *loss, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(k_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LG_SMEM);
+  if (e != cudaSuccess) return e;
   cudaMemsetAsync(M->grad, 0, NPARAM * sizeof(float), s);
-  cudaMemsetAsync(S.loss, 0, sizeof(double), s);
-  k_fwd_bwd<<<(unsigned)((nb + FB_THREADS - 1) / FB_THREADS), FB_THREADS, 0, s>>>(
-      M->w, nb, x, t, 1.0f / (float)nb, S.H1, S.H2, S.D1, S.D2, S.dy, S.loss);
-  const long chunks = (nb + RED_CHUNK - 1) / RED_CHUNK;
-  const unsigned grid = (unsigned)std::min<long>(chunks, 4 * 152);
-  k_grad_reduce<<<grid, 256, 0, s>>>(nb, x, S.H1, S.H2, S.D1, S.D2, S.dy, M->grad);
+  cudaMemsetAsync(loss, 0, sizeof(double), s);
+  // three blocks fit an SM; a block's tiles share its weights and its sums
+  const unsigned grid = (unsigned)std::min<long>((nb + LG_S - 1) / LG_S, 3 * 152);
+  k_loss_grad<<<grid, LG_T, LG_SMEM, s>>>(M->w, nb, x, t, 1.0f / (float)nb, M->grad, loss);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -425,20 +485,20 @@ phl_status phl_mlp_loss_grad(phl_mlp *M, long n, const float *x, const float *t,
   if (!M || n <= 0 || !x || !t || !loss || !grad)
     return (phl_status)set_error(PHL_EINVAL, "phl_mlp_loss_grad: bad arguments");
   const float *dx = x, *dt = t;
-  Scratch S;
-  cudaError_t e = S.alloc(n, where == PHL_HOST ? 4 * n : 0);
+  CallScratch room;   // the loss sum, then the samples
+  constexpr size_t HEAD = 256;
+  cudaError_t e = room.get(HEAD + (where == PHL_HOST ? 4 * n * sizeof(float) : 0), 0);
+  double *dloss = (double *)room.p;
   if (e == cudaSuccess && where == PHL_HOST) {
-    e = cudaMemcpy(S.extra, x, 3 * n * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(S.extra + 3 * n, t, n * sizeof(float), cudaMemcpyHostToDevice);
-    dx = S.extra;
-    dt = S.extra + 3 * n;
+    float *tmp = (float *)((char *)room.p + HEAD);
+    e = cudaMemcpy(tmp, x, 3 * n * sizeof(float), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(tmp + 3 * n, t, n * sizeof(float), cudaMemcpyHostToDevice);
+    dx = tmp;
+    dt = tmp + 3 * n;
   }
-  if (e == cudaSuccess) {
-    launch_loss_grad(M, n, dx, dt, S, 0);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = launch_loss_grad(M, n, dx, dt, dloss, 0);
   double l = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpy(&l, S.loss, sizeof(double), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&l, dloss, sizeof(double), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess)
     e = cudaMemcpy(grad, M->grad, NPARAM * sizeof(float),
                    where == PHL_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice);
@@ -513,8 +573,9 @@ phl_status phl_mlp_train(phl_mlp *M, const phl_eos_table *tab, const phl_mlp_tra
   if (e == cudaSuccess) e = cudaMalloc(&pred, nval * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fail, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&mm, 2 * sizeof(unsigned int));
-  Scratch S;
-  if (e == cudaSuccess) e = S.alloc(cfg->batch, 0);
+  CallScratch room;
+  if (e == cudaSuccess) e = room.get(sizeof(double), 0);
+  double *dloss = (double *)room.p;
   phl_status ret = PHL_OK;
   auto done = [&](phl_status r) {
     cudaFree(x); cudaFree(tt); cudaFree(pred); cudaFree(fail); cudaFree(mm);
@@ -558,7 +619,8 @@ phl_status phl_mlp_train(phl_mlp *M, const phl_eos_table *tab, const phl_mlp_tra
     std::vector<double> losses;
     for (long b = 0; b < nbat; ++b, ++step) {
       const long off = b * cfg->batch;
-      launch_loss_grad(M, cfg->batch, x + 3 * off, tt + off, S, 0);
+      e = launch_loss_grad(M, cfg->batch, x + 3 * off, tt + off, dloss, 0);
+      if (e != cudaSuccess) return done(cuda_status(e, "phl_mlp_train"));
       ++M->adam_t;
       const float lr = (float)(cfg->lr * 0.5 * (1.0 + cos(3.141592653589793 * (double)step / (double)total)));
       const float b1 = 0.9f, b2 = 0.999f;
@@ -566,7 +628,7 @@ phl_status phl_mlp_train(phl_mlp *M, const phl_eos_table *tab, const phl_mlp_tra
       k_adam<<<(NPARAM + 255) / 256, 256>>>(NPARAM, M->w, M->m, M->v, M->grad, lr, b1, b2, 1e-8f, c1, c2);
       if (b + 1 == nbat) {
         double l = 0.0;
-        cudaMemcpy(&l, S.loss, sizeof(double), cudaMemcpyDeviceToHost);
+        cudaMemcpy(&l, dloss, sizeof(double), cudaMemcpyDeviceToHost);
         ep_loss = l / (double)cfg->batch;
       }
     }
