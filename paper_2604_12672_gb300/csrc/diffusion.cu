@@ -29,11 +29,12 @@
 // per z layer (the background temperature of the delta_T option), and 4
 // doubles per cell for the FP64 form's K and face fluxes.  FP64:
 // 1/rho, k0/rho^nR, e_int^(0), the operator at e_int^(0), three stage
-// buffers.  Mixed: e_int^(0) in double (set-up only), then as floats
-// y0 = e_int^(0)/2^eY, the scaled conductivity factor, 1/(rho c_v), the
-// operator at d = 0, the three upper-face differences of y0 and three stage
-// buffers.
+// buffers.  Mixed: e_int^(0) in double (set-up only), then as floats the
+// three upper-face differences of y0 = e_int^(0)/2^eY with 1/(rho c_v) (one
+// 16-byte word per cell), y0 with the scaled conductivity factor (8 bytes),
+// the operator at d = 0 and three stage buffers.
 #include <math.h>
+#include <stdint.h>
 #include <string.h>
 
 #include <cmath>
@@ -56,7 +57,9 @@ struct DiffArrays {       // FP64 form
 
 struct DiffMx {           // mixed form
   double *Y0d;            // e_int^(0) (set-up only)
-  float *y0, *kp, *a, *l0, *g[3], *d[3];
+  float2 *q;              // per cell: y0, kp (until the scales are known: k0/rho^nR, 1/(rho c_v) as they are)
+  float4 *p;              // g_x, g_y, g_z, a
+  float *l0, *d[3];
   const double *That;
 };
 
@@ -159,8 +162,7 @@ __global__ void k_diff_init(DevGeo G, Box box, const double *__restrict__ U, con
     kr = p.k0 * powi_dev(ir, p.nR);
     if (MX) {   // kp and a as raw floats, rescaled once the maxima are known
       M.Y0d[q] = e;
-      M.kp[q] = d2f_scaled(kr, 0);
-      M.a[q] = d2f_scaled(ir * icv, 0);
+      M.q[q] = make_float2(d2f_scaled(kr, 0), d2f_scaled(ir * icv, 0));
     } else {
       A.irho[q] = ir;
       A.krho[q] = kr;
@@ -298,11 +300,9 @@ __global__ void k_dmx_prep(DevGeo G, Box box, Stencil S, DiffMx M, double kt, in
     if (d == 2 && M.That) dY -= cv * (M.That[up] - M.That[c[2]]);
     gd[d] = d2f_scaled(dY, -eY);
   }
-  M.y0[q] = d2f_scaled(Y, -eY);
-  M.kp[q] = d2f_scaled((double)M.kp[q] * kt, -eK);
-  M.a[q] *= asc;
-  for (int d = 0; d < 3; ++d)
-    if (S.act[d]) M.g[d][q] = gd[d];
+  const float2 ra = M.q[q];
+  M.q[q] = make_float2(d2f_scaled(Y, -eY), d2f_scaled((double)ra.x * kt, -eK));
+  M.p[q] = make_float4(gd[0], gd[1], gd[2], ra.y * asc);
 }
 
 // Half the harmonic mean of the two cells' conductivity factors.
@@ -323,20 +323,27 @@ constexpr int DTX = 32, DTY = 8;                  // xy tile of the stage kernel
 constexpr int DHALO = 2 * DTX + 2 * DTY;          // its x and y halo cells
 constexpr int DTZ_DEFAULT = 16;                   // planes per CTA
 
-// Raw slot data of one cell as loaded: d^(m-1), y0, kp (src = NOSRC: a
-// cell outside the domain on a non-periodic side, all zero).
+// Raw slot data of one cell as loaded: d^(m-1), y0, kp (all zero for a cell
+// outside the domain on a non-periodic side).
 struct Raw {
   float d, y, k;
 };
-constexpr unsigned NOSRC = 0xffffffffu;
+
+// p[cell] of a plane: the plane's start (block-uniform, 64-bit) plus a 32-bit
+// offset within it in units of 4 bytes.  (A plane's byte offsets fit: the state
+// of 2^28 cells alone exceeds the device.)
+template <class T>
+__device__ __forceinline__ T pld(const T *p, long plane, unsigned off) {
+  return __ldg(p + plane + off);
+}
 
 template <bool FIRST>
-__device__ __forceinline__ Raw raw_load(const DiffMx &M, const float *__restrict__ dm1, unsigned i) {
+__device__ __forceinline__ Raw raw_load(const DiffMx &M, const float *__restrict__ dm1, long plane, unsigned off) {
   Raw r{0.0f, 0.0f, 0.0f};
-  if (i == NOSRC) return r;
-  if (!FIRST) r.d = __ldg(dm1 + i);
-  r.y = __ldg(M.y0 + i);
-  r.k = __ldg(M.kp + i);
+  if (!FIRST) r.d = pld(dm1, plane, off);
+  const float2 v = pld(M.q, plane, off);
+  r.y = v.x;
+  r.k = v.y;
   return r;
 }
 
@@ -348,7 +355,8 @@ __device__ __forceinline__ float kval(const Raw &r) { return r.k * pw<NT>(r.y + 
 // 1/(rho c_v), the operator at d = 0 and d^(m-2) of the own cell.
 struct Aux {
   Raw h;
-  float gx, gy, gz, glx, gly, a, l0, d2;
+  float4 g;   // g_x, g_y, g_z, a
+  float glx, gly, l0, d2;
 };
 
 __device__ __forceinline__ int wrap_or_out(int x, int n, int per) {
@@ -368,86 +376,89 @@ __device__ __forceinline__ int wrap_or_out(int x, int n, int per) {
 //   lambda = a sum_d w_d (G_upper - G_lower).
 // A face on a non-periodic side is zero.  The loads are software-pipelined:
 // the own slot two planes ahead, everything else one plane ahead, so the
-// plane's barrier does not wait on memory.  Indices are 32-bit (the
-// caller checks the cell count).  FIRST: d^(m-1) = 0, lambda is the operator
-// at e_int^(0) (stored in l0) and d^(1) = mt lambda; else
+// plane's barrier does not wait on memory.  FIRST: d^(m-1) = 0, lambda is the
+// operator at e_int^(0) (stored in l0) and d^(1) = mt lambda; else
 // d^(m) = mu d^(m-1) + nu d^(m-2) + mt lambda + gt l0.
-template <int NT, bool FIRST>
+// Bound by instruction issue (four slots of five in use, DRAM half): five
+// harmonic means with a reciprocal each per cell.  The seven constants of a
+// cell in one 8-byte and one 16-byte load, (d, k) as one shared-memory pair, k
+// carried between planes and the boundary tests kept as predicates: 70.4 ->
+// 65.4 us per stage on 192^3 (40 B per cell, 4.3 TB/s).  D3: all three axes
+// active.
+template <int NT, bool FIRST, bool D3>
 __global__ void __launch_bounds__(DTX * DTY) k_dmx_stage(Stencil S, DiffMx M, float mu, float nu, float mt, float gt,
                                                         const float *__restrict__ dm1, const float *__restrict__ dm2,
                                                         float *__restrict__ dj, int tz) {
-  __shared__ float sdb[2][DTY + 2][DTX + 2], skb[2][DTY + 2][DTX + 2];   // double-buffered by plane parity
+  __shared__ float2 sb[2][DTY + 2][DTX + 2];   // (d, k), double-buffered by plane parity
   const int tx = threadIdx.x % DTX, ty = threadIdx.x / DTX;
   const int nx = S.n[0], ny = S.n[1], nz = S.n[2];
   const int x0 = blockIdx.x * DTX, y0 = blockIdx.y * DTY, z0 = blockIdx.z * tz;
   const int z1 = min(z0 + tz, nz);
-  const unsigned pl = (unsigned)S.st[2];
+  const long pl = S.st[2];
   const int gx = x0 + tx, gy = y0 + ty;
   const bool own = gx < nx && gy < ny;
-  // own slot's source cell within a plane (wrapped), or NOSRC
-  unsigned osrc = NOSRC;
-  {
-    const int sx = wrap_or_out(gx, nx, S.per[0]), sy = wrap_or_out(gy, ny, S.per[1]);
-    if (sx >= 0 && sy >= 0) osrc = (unsigned)(sx + nx * sy);
-  }
+  const bool a0 = D3 || S.act[0], a1 = D3 || S.act[1], a2 = D3 || S.act[2];
+  // own slot's source cell within a plane (wrapped)
+  auto source = [&](int x, int y, bool &has) {
+    const int sx = wrap_or_out(x, nx, S.per[0]), sy = wrap_or_out(y, ny, S.per[1]);
+    has = sx >= 0 && sy >= 0;
+    return has ? (unsigned)(sx + nx * sy) : 0u;
+  };
+  bool has;
+  const unsigned oo = source(gx, gy, has);
   // this thread's halo slot (threadIdx.x < DHALO): position and source
   int hr = 0, hc = 0;
-  unsigned hsrc = NOSRC;
-  if (threadIdx.x < DHALO) {
+  bool hhas = false;
+  unsigned ho = 0;
+  const bool halo = threadIdx.x < DHALO;
+  if (halo) {
     const int h = threadIdx.x;
     if (h < DTY) { hc = 0; hr = h + 1; }
     else if (h < 2 * DTY) { hc = DTX + 1; hr = h - DTY + 1; }
     else if (h < 2 * DTY + DTX) { hr = 0; hc = h - 2 * DTY + 1; }
     else { hr = DTY + 1; hc = h - 2 * DTY - DTX + 1; }
-    const int sx = wrap_or_out(x0 + hc - 1, nx, S.per[0]), sy = wrap_or_out(y0 + hr - 1, ny, S.per[1]);
-    if (sx >= 0 && sy >= 0 && S.act[(hr == 0 || hr == DTY + 1) ? 1 : 0]) hsrc = (unsigned)(sx + nx * sy);
+    ho = source(x0 + hc - 1, y0 + hr - 1, hhas);
+    hhas = hhas && ((hr == 0 || hr == DTY + 1) ? a1 : a0);
   }
-  // in-plane cells below the tile's lower boundary faces (their g), or NOSRC
-  unsigned lxsrc = NOSRC, lysrc = NOSRC;
-  if (own && S.act[0]) {
-    const int lx = wrap_or_out(gx - 1, nx, S.per[0]);
-    if (lx >= 0) lxsrc = (unsigned)(lx + nx * gy);
-  }
-  if (own && S.act[1]) {
-    const int ly = wrap_or_out(gy - 1, ny, S.per[1]);
-    if (ly >= 0) lysrc = (unsigned)(gx + nx * ly);
-  }
-  const bool hasz = S.act[2] != 0;
+  // the cells below the own lower faces in the plane (their g)
+  bool lx = false, ly = false;
+  unsigned lxo = 0, lyo = 0;
+  if (own && a0) lxo = source(gx - 1, gy, lx);
+  if (own && a1) lyo = source(gx, gy - 1, ly);
+  const bool ux = a0 && (gx + 1 < nx || S.per[0]), uy = a1 && (gy + 1 < ny || S.per[1]);
 
   auto aux_load = [&](int z) {
     Aux X{};
-    const unsigned base = (unsigned)z * pl;
-    if (threadIdx.x < DHALO && hsrc != NOSRC) X.h = raw_load<FIRST>(M, dm1, base + hsrc);
+    const long p = (long)z * pl;
+    if (hhas) X.h = raw_load<FIRST>(M, dm1, p, ho);
     if (own) {
-      const unsigned q = base + osrc;
-      if (S.act[0]) X.gx = __ldg(M.g[0] + q);
-      if (S.act[1]) X.gy = __ldg(M.g[1] + q);
-      if (hasz) X.gz = __ldg(M.g[2] + q);
-      X.a = __ldg(M.a + q);
+      X.g = pld(M.p, p, oo);
       if (!FIRST) {
-        X.l0 = __ldg(M.l0 + q);
-        X.d2 = __ldg(dm2 + q);
+        X.l0 = pld(M.l0, p, oo);
+        X.d2 = pld(dm2, p, oo);
       }
     }
-    if (lxsrc != NOSRC) X.glx = __ldg(M.g[0] + base + lxsrc);
-    if (lysrc != NOSRC) X.gly = __ldg(M.g[1] + base + lysrc);
+    if (lx) X.glx = pld(&M.p->x, 4 * p, 4u * lxo);
+    if (ly) X.gly = pld(&M.p->y, 4 * p, 4u * lyo);
     return X;
   };
-  auto own_load = [&](int z) {   // own slot of plane z (wrapped), zeros outside
-    const int zz = hasz ? wrap_or_out(z, nz, S.per[2]) : (z == 0 ? 0 : -1);
-    return (zz >= 0 && osrc != NOSRC) ? raw_load<FIRST>(M, dm1, (unsigned)zz * pl + osrc) : Raw{0.0f, 0.0f, 0.0f};
+  auto own_load = [&](int z) {   // own slot of plane z (wrapped once), zeros outside
+    if (z < 0 || z >= nz) {
+      if (!a2 || !S.per[2]) return Raw{0.0f, 0.0f, 0.0f};
+      z = wrap_or_out(z, nz, 1);
+    }
+    return has ? raw_load<FIRST>(M, dm1, (long)z * pl, oo) : Raw{0.0f, 0.0f, 0.0f};
   };
 
   Raw oc = own_load(z0), on = own_load(z0 + 1);
   Aux ac = aux_load(z0);
+  float ck = kval<NT>(oc);
   float gzl = 0.0f;   // G of the z face below the current plane
-  if (hasz && own) {
-    const int pz = wrap_or_out(z0 - 1, nz, S.per[2]);
-    if (pz >= 0) {
-      const Raw pr = raw_load<FIRST>(M, dm1, (unsigned)pz * pl + osrc);
-      gzl = hmean_f(kval<NT>(pr), kval<NT>(oc)) * (__ldg(M.g[2] + (unsigned)pz * pl + osrc) + (oc.d - pr.d));
-    }
+  if (a2 && own && (z0 > 0 || S.per[2])) {
+    const Raw pr = own_load(z0 - 1);
+    gzl = hmean_f(kval<NT>(pr), ck) * (pld(M.p, (long)(z0 > 0 ? z0 - 1 : nz - 1) * pl, oo).z + (oc.d - pr.d));
   }
+#pragma unroll 2   // the pipeline registers change names instead of moving
   for (int z = z0; z < z1; ++z) {
     Raw onn = on;
     Aux an = ac;
@@ -455,40 +466,32 @@ __global__ void __launch_bounds__(DTX * DTY) k_dmx_stage(Stencil S, DiffMx M, fl
       onn = own_load(z + 2);
       an = aux_load(z + 1);
     }
-    const float cd = oc.d, ck = kval<NT>(oc);
-    float(*sd)[DTX + 2] = sdb[z & 1];
-    float(*sk)[DTX + 2] = skb[z & 1];
-    sd[ty + 1][tx + 1] = cd;
-    sk[ty + 1][tx + 1] = ck;
-    if (threadIdx.x < DHALO) {
-      sd[hr][hc] = ac.h.d;
-      sk[hr][hc] = kval<NT>(ac.h);
-    }
+    const float cd = oc.d, nk = kval<NT>(on);
+    float2(*sp)[DTX + 2] = sb[z & 1];
+    sp[ty + 1][tx + 1] = make_float2(cd, ck);
+    if (halo) sp[hr][hc] = make_float2(ac.h.d, kval<NT>(ac.h));
     // one barrier per plane: the slots alternate between two buffers, and a
     // thread two planes ahead has passed the barrier every reader reached
     __syncthreads();
     if (own) {
       float s = 0.0f;
-      if (S.act[0]) {   // each cell forms both its faces (the lower one as its neighbour does)
-        const float up = (gx + 1 < nx || S.per[0])
-                             ? hmean_f(ck, sk[ty + 1][tx + 2]) * (ac.gx + (sd[ty + 1][tx + 2] - cd)) : 0.0f;
-        const float lo = lxsrc != NOSRC ? hmean_f(sk[ty + 1][tx], ck) * (ac.glx + (cd - sd[ty + 1][tx])) : 0.0f;
-        s += S.w[0] * (up - lo);
+      if (a0) {   // each cell forms both its faces (the lower one as its neighbour does)
+        const float2 r = sp[ty + 1][tx + 2], l = sp[ty + 1][tx];
+        const float up = hmean_f(ck, r.y) * (ac.g.x + (r.x - cd)), lo = hmean_f(l.y, ck) * (ac.glx + (cd - l.x));
+        s += S.w[0] * ((ux ? up : 0.0f) - (lx ? lo : 0.0f));
       }
-      if (S.act[1]) {
-        const float up = (gy + 1 < ny || S.per[1])
-                             ? hmean_f(ck, sk[ty + 2][tx + 1]) * (ac.gy + (sd[ty + 2][tx + 1] - cd)) : 0.0f;
-        const float lo = lysrc != NOSRC ? hmean_f(sk[ty][tx + 1], ck) * (ac.gly + (cd - sd[ty][tx + 1])) : 0.0f;
-        s += S.w[1] * (up - lo);
+      if (a1) {
+        const float2 r = sp[ty + 2][tx + 1], l = sp[ty][tx + 1];
+        const float up = hmean_f(ck, r.y) * (ac.g.y + (r.x - cd)), lo = hmean_f(l.y, ck) * (ac.gly + (cd - l.x));
+        s += S.w[1] * ((uy ? up : 0.0f) - (ly ? lo : 0.0f));
       }
-      if (hasz) {
-        const bool up = z + 1 < nz || S.per[2];
-        const float gzu = up ? hmean_f(ck, kval<NT>(on)) * (ac.gz + (on.d - cd)) : 0.0f;
+      if (a2) {
+        const float gzu = z + 1 < nz || S.per[2] ? hmean_f(ck, nk) * (ac.g.z + (on.d - cd)) : 0.0f;
         s += S.w[2] * (gzu - gzl);
         gzl = gzu;
       }
-      const float lam = ac.a * s;
-      const unsigned q = (unsigned)z * pl + osrc;
+      const float lam = ac.g.w * s;
+      const long q = (long)z * pl + oo;
       if (FIRST) {
         M.l0[q] = lam;
         dj[q] = mt * lam;
@@ -498,21 +501,28 @@ __global__ void __launch_bounds__(DTX * DTY) k_dmx_stage(Stencil S, DiffMx M, fl
     }
     oc = on;
     on = onn;
+    ck = nk;
     ac = an;
   }
 }
 
+template <bool FIRST, bool D3>
+void launch_dmx_stage_d(int nT, dim3 grd, int tz, cudaStream_t s, const Stencil &S, const DiffMx &M, float mu,
+                        float nu, float mt, float gt, const float *dm1, const float *dm2, float *dj) {
+  const dim3 blk(DTX * DTY);
+  switch (nT) {
+    case 0: k_dmx_stage<0, FIRST, D3><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
+    case 1: k_dmx_stage<1, FIRST, D3><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
+    case 2: k_dmx_stage<2, FIRST, D3><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
+    case 3: k_dmx_stage<3, FIRST, D3><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
+    default: k_dmx_stage<4, FIRST, D3><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
+  }
+}
 template <bool FIRST>
 void launch_dmx_stage(int nT, dim3 grd, int tz, cudaStream_t s, const Stencil &S, const DiffMx &M, float mu,
                       float nu, float mt, float gt, const float *dm1, const float *dm2, float *dj) {
-  const dim3 blk(DTX * DTY);
-  switch (nT) {
-    case 0: k_dmx_stage<0, FIRST><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
-    case 1: k_dmx_stage<1, FIRST><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
-    case 2: k_dmx_stage<2, FIRST><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
-    case 3: k_dmx_stage<3, FIRST><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
-    default: k_dmx_stage<4, FIRST><<<grd, blk, 0, s>>>(S, M, mu, nu, mt, gt, dm1, dm2, dj, tz); break;
-  }
+  if (S.act[0] && S.act[1] && S.act[2]) launch_dmx_stage_d<FIRST, true>(nT, grd, tz, s, S, M, mu, nu, mt, gt, dm1, dm2, dj);
+  else launch_dmx_stage_d<FIRST, false>(nT, grd, tz, s, S, M, mu, nu, mt, gt, dm1, dm2, dj);
 }
 
 // E += rho 2^eY d^(N)
@@ -566,13 +576,10 @@ cudaError_t launch_diffuse(const DevGeo &G, double *U, const double *Bf, const p
   M.That = nullptr;
   if (mixed) {   // e_int^(0) in double, then ten float arrays: 6 doubles per cell
     M.Y0d = scratch;
-    float *f = (float *)(scratch + nc);
-    M.y0 = f;
-    M.kp = f + nc;
-    M.a = f + 2 * nc;
-    M.l0 = f + 3 * nc;
-    for (int k = 0; k < 3; ++k) M.g[k] = f + (4 + k) * nc;
-    for (int k = 0; k < 3; ++k) M.d[k] = f + (7 + k) * nc;
+    M.p = (float4 *)(((uintptr_t)(scratch + nc) + 15) & ~(uintptr_t)15);   // the seventh double per cell has room
+    M.q = (float2 *)(M.p + nc);
+    M.l0 = (float *)(M.q + nc);
+    for (int k = 0; k < 3; ++k) M.d[k] = M.l0 + (1 + k) * nc;
   } else {
     A.irho = scratch;
     A.krho = scratch + nc;
