@@ -49,9 +49,9 @@ FP64_NOMINAL_TFLOPS = 1.25     # GB300 FP64 (profiling recipe's nominal table)
 # input (5 cell + 3 face doubles), read U^n for stages 2-3, write the output.
 BYTES_PER_CELL_STAGE = {1: 128.0, 2: 192.0, 3: 192.0}
 # FP64 flux kernel: FP64 operations per face (DADD + DMUL + 2 DFMA counted from
-# the ncu SASS counters of k_flux on the stratified box at 64^3, mean of the
-# three directions).
-FP64_FLOP_PER_FACE = 637.7
+# the ncu counters of k_flux_walk on the stratified box at 128 x 96 x 112, mean
+# of the three directions).
+FP64_FLOP_PER_FACE = 475.6
 # Mixed flux kernel: FP32 operations per face (FADD + FMUL + 2 FFMA from the ncu
 # SASS counters of k_flux<0/1/2, float> on the stratified box at 160^3, per sweep
 # direction), and its DRAM bytes per face (dram__bytes_read + write, same capture;
@@ -61,17 +61,15 @@ FP64_FLOP_PER_FACE = 637.7
 FP32_FLOP_PER_FACE = {"flux_x": 381.1, "flux_y": 381.1, "flux_z": 380.1}
 FP32_DRAM_BYTES_PER_FACE = {"flux_x": 74.4, "flux_y": 75.8, "flux_z": 76.1}
 FP32_NOMINAL_TFLOPS = 80.5
-# Fused tile kernel (k_flux_update_mx): from the ncu counters of the
-# stratified box at 160^3 (W larger than L2), one launch of stage 1 and one of
-# stage 2 of the scalar launch shape (2): FP32 operations (FADD + FMUL + 2 FFMA)
-# 1398 per cell as executed, i.e. 414 per face over the 3.375 faces per cell
-# an 8^3 tile evaluates; the algorithmic count is 3 faces per cell x 414 =
-# 1243.  The default shape evaluates the same operations, partly as packed
-# FP32x2 instructions that those per-opcode counters do not include.  DRAM
-# bytes per cell of the current default shape: 111.8 (stage 1, no increment
+# Fused tile kernel (k_flux_update_mx): FP32 operations of the default launch
+# shape from ncu's per-opcode counters on the stratified box at 128^3 (FADD +
+# FMUL + 2 FFMA, the packed FP32x2 forms counted twice): 405 per face over the
+# 3.375 faces per cell an 8^3 tile evaluates; the algorithmic count is 3 faces
+# per cell x 405 = 1215.  DRAM
+# bytes per cell (160^3, W larger than L2): 111.8 (stage 1, no increment
 # to read), 144.6 (stage 2) and 205.3 (stage 3, which also reads and writes
 # the FP64 state), 153.9 on average over an RK3 step.
-FUSED_FLOP_PER_CELL = 3.0 * 414.3
+FUSED_FLOP_PER_CELL = 3.0 * 405.1
 FUSED_DRAM_BYTES_PER_CELL = (111.8 + 144.6 + 205.3) / 3.0
 
 
@@ -464,7 +462,7 @@ def l1_mixed_vs_fp64(P, pr, steps=3):
 
 # the stellar box's mixed inversion (k_eos_cells<float> from each cell's record): FP64 operations
 # per cell-stage, ncu on the 128^3 box (DADD + DMUL + 2 DFMA)
-EOS_FP64_FLOP_PER_CELL = 721.0
+EOS_FP64_FLOP_PER_CELL = 375.4
 
 
 def stellar_c3(P, n, steps, warmup, stream, ws, alu=None):
@@ -730,9 +728,9 @@ def ensemble_c4(P, steps, warmup, stream, ws):
 
 # Cubed-sphere shell (FP64): the flux kernel's FP64 operations per face
 # (DADD + DMUL + 2 DFMA from the ncu SASS counters of k_sph_flux on the
-# 6 x 64 x 64 x 64 shell: 4690.3 M over 4.743 M faces) and its DRAM bytes
-# per face in the same capture (517.4 MB; the work arrays exceed L2 there).
-SPH_FP64_FLOP_PER_FACE = 988.9
+# 6 x 64 x 64 x 96 shell: 5307.0 M over 7.102 M faces) and its DRAM bytes
+# per face on 6 x 64^3 (517.4 MB; the work arrays exceed L2 there).
+SPH_FP64_FLOP_PER_FACE = 747.3
 SPH_FLUX_DRAM_BYTES_PER_FACE = 109.1
 # the mixed form's flux kernel: FP32 operations per face, FADD + FMUL + 2 FFMA
 # of the scalar solver on the same shell (2533.6 M over 4.743 M faces; the
@@ -741,9 +739,9 @@ SPH_FLUX_DRAM_BYTES_PER_FACE = 109.1
 # (241.0 MB in the capture of the packed-lane kernel)
 SPH_FP32_FLOP_PER_FACE = 534.2
 # the stellar shell's mixed inversion (k_sph_prims_st<float>, recorded path): FP64 operations and
-# FP64-pipe instructions per cell-stage, ncu on the 6 x 64^3 stellar shell
-SPH_ST_FP64_FLOP_PER_CELL = 722.0
-SPH_ST_FP64_INST_PER_CELL = 507.1
+# FP64-pipe instructions per cell-stage, ncu on the 6 x 64 x 64 x 96 stellar shell
+SPH_ST_FP64_FLOP_PER_CELL = 346.0
+SPH_ST_FP64_INST_PER_CELL = 210.0
 SPH_MX_FLUX_DRAM_BYTES_PER_FACE = 50.8
 
 

@@ -23,10 +23,11 @@
 // 5 + 4 + 3 multiply-adds, so f, f_x, f_xx of the six rows take 72 and the six
 // needed mixed derivatives 26 more.  The Hermite form it replaces (two bases
 // of 62 operations, 108 + 36 multiply-adds) took 268.  With the shared
-// subexpressions below, the recorded inversion of the stellar box went from
-// 2.12 to ~1.03 ms per launch on 128^3 cells, the shell's kernel from 2.40 to
-// 1.20 ms on 2.36 million cells and the batch inversion from 4.63 to 2.10 ms
-// for 10^6 far guesses; FP64 pipe bound as before.  The coefficients above
+// subexpressions below and integer tests for compares and conversions, the
+// recorded inversion of the stellar box went from 2.12 to 0.95 ms per launch on
+// 128^3 cells, the shell's kernel from 2.40 to 0.95 ms on 2.36 million cells
+// and the batch inversion from 4.63 to 1.99 ms for 10^6 far guesses; FP64 pipe
+// bound as before.  The coefficients above
 // the constant are the size of the cell's own differences, so no derivative
 // cancels node values at evaluation; their set-up works on differences too.
 #pragma once
