@@ -112,7 +112,8 @@ __global__ void k_eos_batch(Table t, long n, const double *rho, const double *ei
   EosOut<double> o;
   double Td = T[i];
   int it;
-  const double r = rho[i], ir = rcp_nr(r), iab = rcp_nr(abar[i]);
+  // an infinite Abar (no ions) is a state like any other; rcp_nr gives NaN for it
+  const double r = rho[i], ir = rcp_nr(r), iab = isinf(abar[i]) ? 0.0 : rcp_nr(abar[i]);
   if (sizeof(R) == 8) it = eos_invert<double>(t, r, ir, eint[i], iab, ye[i], Td, tol, maxit, o);
   else it = eos_invert_mixed(t, r, ir, eint[i], iab, ye[i], Td, tol, maxit, o);
   const bool ok = it > 0;

@@ -246,7 +246,7 @@ __device__ __forceinline__ bool eos_rt_xy(const Table &t, const XB<R> &X, R rho,
 
 template <typename R>
 __device__ __forceinline__ bool eos_rt(const Table &t, R rho, R T, R abar, R ye, EosOut<R> &o) {
-  return eos_rt_xy<R>(t, xbasis<R>(t, log(rho * ye * R(NAV))), rho, rcp_nr(rho), T, log(T), rcp_nr(T), rcp_nr(abar), o);
+  return eos_rt_xy<R>(t, xbasis<R>(t, log(rho * ye * R(NAV))), rho, rcp_nr(rho), T, log(T), rcp_nr(T), R(1) / abar, o);
 }
 
 // Specific internal energy and c_v at (rho, T): what a Newton iteration needs.
