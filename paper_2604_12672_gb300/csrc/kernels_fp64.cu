@@ -281,7 +281,8 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
   // one launch for all directions, and one for the EMFs and the cell update,
   // where a direction's faces are fewer than the GPU's threads in a wave (128
   // x 128: 40 + 12 -> 28 + 8 us a stage, and two launches fewer)
-  const bool small = most < 4L * 152 * 128 && G.recon == PHL_RECON_VANLEER;
+  // (a grid without an active axis has no faces: nothing to launch for them)
+  const bool small = most > 0 && most < 4L * 152 * 128 && G.recon == PHL_RECON_VANLEER;
   if (small) {
     FaceSet<double> A{};
     const unsigned t = most < 152L * 128 ? 32u : 64u;

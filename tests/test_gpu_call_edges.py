@@ -1,4 +1,6 @@
 """Calls at the edge of what the entry points accept."""
+import types
+
 import numpy as np
 import pytest
 
@@ -27,3 +29,26 @@ def test_eos_without_ions(P, precision):
     assert (b["iters"][:2] > 0).all()
     for k in a:
         assert np.array_equal(a[k], b[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_one_cell_without_active_axes(P, precision):
+    """A grid of one cell has no faces, only the gravity source: the momentum
+    grows linearly and the energy with its square, which the RK3 step
+    integrates exactly (a few roundings in FP64, the FP32 increments' 1e-7 of
+    the change in the mixed form)."""
+    pr = types.SimpleNamespace(n=(1, 1, 1), lo=(0.0,) * 3, hi=(1.0,) * 3, bc=((0, 0),) * 3, gamma=5 / 3,
+                               g=(0.0, 0.0, -1.0), bg=None, heat=None, cfl=0.4, riemann="lhlld", eps_sf=0.2,
+                               mach_thr=0.6, nspec=0, eos="ideal")
+    cons = np.array([1.0, 0.1, 0.0, 0.0, 2.0]).reshape(5, 1, 1, 1)
+    faces = [np.full((1, 1, 2), 0.1), np.full((1, 2, 1), 0.2), np.full((2, 1, 1), 0.3)]
+    g = P.Grid(pr, precision=precision)
+    g.set_state(cons, *faces)
+    g.step(2, 1e-2)
+    out = [np.zeros_like(cons)] + [np.zeros_like(f) for f in faces]
+    g.get_state_into(*out)
+    g.close()
+    t = 2e-2
+    assert np.abs(out[0].ravel() - [1.0, 0.1, 0.0, -t, 2.0 + 0.5 * t * t]).max() <= (1e-15 if precision == "fp64" else 2e-9)
+    for a, b in zip(out[1:], faces):
+        assert np.array_equal(a, b)
