@@ -29,9 +29,11 @@
 // decisions, which the next kernel reads from a small status block.  The FP64
 // pipe (1/64 of the FP32 rate) bounds the iteration, so the sums are arranged
 // for few FP64 instructions: a block's 256 values go through shared memory to
-// one warp (13 instructions, where eight warps' shuffles took 45), and the
+// one warp (12 additions, where eight warps' shuffles took 45), and the
 // partials are summed once, not by every block of the consumer (7 us a column
-// at 608 blocks when one warp of each did).  96^3: 99 -> 70 us of kernels an iteration.
+// at 608 blocks when one warp of each did).  An iteration of a solve takes 84
+// us at 96^3 and 33 at 32^3 (115 and 39 with the consumers' sums), with the
+// same bits and so the same iteration count.
 // Convergence and breakdown are decided on the device, so the host enqueues
 // iterations in batches and reads the status once per batch; the kernels of
 // an iteration after the decision return at once.
@@ -93,52 +95,78 @@ __device__ __forceinline__ void decode(const PGeo &g, unsigned q, int &i, int &j
   k = (int)b;
 }
 
-// Sums of N values over the block's threads (all call), N <= PT / 32: warp c
-// sums the c-th and returns it.  sh: N * PT doubles.
-template <int N>
-__device__ __forceinline__ double block_sums(const double *v, double *sh) {
-#pragma unroll
-  for (int c = 0; c < N; ++c) sh[c * PT + threadIdx.x] = v[c];
-  __syncthreads();
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  double t = 0.0;
-  if (w < N) {
-#pragma unroll
-    for (int k = 0; k < PT / 32; ++k) t += sh[w * PT + 32 * k + l];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  }
-  __syncthreads();
-  return t;   // warp c: the sum of v[c]
-}
+// Shared doubles of one column of a block sum: a warp's 32 values, four apart
+// from the next warp's (conflict-free for the reads below).
+constexpr int SHW = 36, SHC = PT / 32 * SHW;
 
 // Leaves the block's sums of N columns as its partials; the block that does so
 // last sums every block's partials, and its thread 0 gets the totals (true).
+// All threads call; after one barrier warp c alone goes on with column c (one
+// warp for both queues twice the additions on its quarter of the FP64 pipe:
+// 88 instead of 84 us an iteration at 96^3, 37.5 instead of 33.5 at 32^3).
+// The order of the additions is that of shuffle trees over a warp's lanes, over
+// the warps and, for 32 interleaved chains of partials, over the chains
+// (block_sum, sum_parts): BiCGSTAB's iteration count depends on it (690 on the
+// stretched 256^3 sphere; warps first, then lanes, gave 774).  Lane 4 w + l
+// forms the first three levels of warp w's tree for lanes l + 4 k.
+// sh: N * SHC doubles.
 template <int N>
 __device__ __forceinline__ bool reduce_last(const double *v, double *const *part, int nb, Status *st, double *sh,
                                             double *tot) {
-  __shared__ bool last;
-  const int w = threadIdx.x >> 5;
-  double t = block_sums<N>(v, sh);
-  if (w < N && (threadIdx.x & 31) == 0) part[w][blockIdx.x] = t;
-  __threadfence();
+  __shared__ int last;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < N; ++c) sh[c * SHC + w * SHW + l] = v[c];
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicInc(&st->done, (unsigned)nb - 1u) == (unsigned)nb - 1u;   // wraps to 0
-  __syncthreads();
+  if (w >= N) return false;
+  auto meet = [] {   // the column warps
+    if (N > 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * N) : "memory");
+    else __syncwarp();
+  };
+  const double *r = sh + w * SHC + (l >> 2) * SHW + (l & 3);
+  double t = ((r[0] + r[16]) + (r[8] + r[24])) + ((r[4] + r[20]) + (r[12] + r[28]));
+  constexpr int LEVEL[5] = {2, 1, 16, 8, 4};   // lanes of a warp, then warps
+#pragma unroll
+  for (int k = 0; k < 5; ++k) t += __shfl_xor_sync(0xffffffffu, t, LEVEL[k]);
+  if (l == 0) part[w][blockIdx.x] = t;
+  meet();
+  if (threadIdx.x == 0) {
+    // releases the partials and acquires the other blocks' (with full fences
+    // around a relaxed increment 3 us more an iteration at 32^3); wraps to 0
+    unsigned before;
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                 : "=r"(before)
+                 : "l"(__cvta_generic_to_global(&st->done)), "r"((unsigned)nb - 1u)
+                 : "memory");
+    last = before == (unsigned)nb - 1u;
+  }
+  meet();
   if (!last) return false;
-  __threadfence();
-  double a[N];
+  t = 0.0;
+  constexpr int B = 20;   // partials of a lane in flight (four blocks on each of 152 SMs leave 19)
+  for (int b0 = 0; b0 < nb; b0 += 32 * B) {
+    double u[B];
 #pragma unroll
-  for (int c = 0; c < N; ++c) a[c] = 0.0;
-  for (int b = (int)threadIdx.x; b < nb; b += PT)
+    for (int k = 0; k < B; ++k) {
+      const int b = b0 + 32 * k + l;
+      u[k] = b < nb ? __ldcg(part[w] + b) : 0.0;
+    }
 #pragma unroll
-    for (int c = 0; c < N; ++c) a[c] += __ldcg(part[c] + b);
-  t = block_sums<N>(a, sh);
-  if (w < N && (threadIdx.x & 31) == 0) sh[w] = t;
-  __syncthreads();
+    for (int k = 0; k < B; ++k) {
+      if (b0 + 32 * k >= nb) break;
+      t += u[k];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (N > 1) {
+    if (l == 0) sh[w] = t;
+    meet();
+  }
   if (threadIdx.x != 0) return false;
+  tot[0] = t;
 #pragma unroll
-  for (int c = 0; c < N; ++c) tot[c] = sh[c];
+  for (int c = 1; c < N; ++c) tot[c] = sh[c];
   return true;
 }
 
@@ -398,7 +426,7 @@ __global__ void k_ghost(PGeo g, Vecs V, unsigned nghost) {
 // r = b - A x0 with b = 4 pi G rho - (ghost terms); rh = r; p = v = 0;
 // D^-1, the residual weights; partials of (rh, r) and |w r|^2.
 __global__ void __launch_bounds__(PT) k_init(PGeo g, Vecs V) {
-  __shared__ double sh[2 * PT];
+  __shared__ double sh[2 * SHC];
   const double fpg = 4.0 * 3.14159265358979323846 * g.G;
   double rr = 0.0, nr = 0.0;
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
@@ -440,7 +468,7 @@ __global__ void __launch_bounds__(PT) k_bi_p(PGeo g, Vecs V, int it) {
 // K2: v = A ph; (rh, v) and alpha
 __global__ void __launch_bounds__(PT) k_bi_av(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[PT];
+  __shared__ double sh[SHC];
   double rv = 0.0;
 #pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
@@ -461,7 +489,7 @@ __global__ void __launch_bounds__(PT) k_bi_av(PGeo g, Vecs V, int it) {
 // K3: s, sh; |w s|^2 and the half-step check
 __global__ void __launch_bounds__(PT) k_bi_s(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[PT];
+  __shared__ double sh[SHC];
   const double alpha = V.st->alpha;
   double ns = 0.0;
 #pragma unroll 2
@@ -483,7 +511,7 @@ __global__ void __launch_bounds__(PT) k_bi_s(PGeo g, Vecs V, int it) {
 // K4: t = A sh; (t, s), (t, t) and omega
 __global__ void __launch_bounds__(PT) k_bi_at(PGeo g, Vecs V, int it) {
   if (V.st->status != ST_RUN) return;
-  __shared__ double sh[2 * PT];
+  __shared__ double sh[2 * SHC];
   double ts = 0.0, tt = 0.0;
 #pragma unroll 2
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < g.nc; q += gridDim.x * blockDim.x) {
@@ -517,7 +545,7 @@ __global__ void __launch_bounds__(PT) k_bi_x(PGeo g, Vecs V, int it) {
     return;
   }
   if (st != ST_RUN) return;
-  __shared__ double sh[2 * PT];
+  __shared__ double sh[2 * SHC];
   const double omega = V.st->omega;
   double rr = 0.0, nr = 0.0;
 #pragma unroll 2
