@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(LG_T, 3) k_loss_grad(const float *__restrict__
   if (tid == 0) sm.b3 = w[O_B3];
   const int rg = tid & 7, s4 = 4 * (tid >> 3);       // products 1, 2: row group, first of four samples
   const int gb = tid & 7, ga = tid >> 3;             // product 3: columns gb + 8 j, rows ga + 16 i
-  float gw[4][8] = {}, gb3 = 0.0f, r2 = 0.0f;
+  float gw[4][8] = {}, gb3 = 0.0f;
+  double r2 = 0.0;   // squared residuals: a tile's 16 of a warp in FP32, the tiles in FP64
   // per-row sums: over the warp's four sample groups, then into the warp's own
   // row of shared memory (48 registers less than keeping them per thread)
   float (*row)[NH] = sm.row[tid >> 5];
@@ -202,17 +203,17 @@ __global__ void __launch_bounds__(LG_T, 3) k_loss_grad(const float *__restrict__
           z[i][q] = tanhf(z[i][q]);
           y[q] += sm.w3[rg + 8 * i] * z[i][q];
         }
-      float dy[4];
+      float dy[4], t2 = 0.0f;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         for (int o = 1; o < 8; o <<= 1) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
         const float r = s4 + q < cnt ? sm.b3 + y[q] - sm.t[s4 + q] : 0.0f;   // no contribution beyond the batch
         dy[q] = 2.0f * r * inv_n;
-        if (rg == 0) {
-          r2 += r * r;
-          gb3 += dy[q];
-        }
+        t2 += r * r;
+        gb3 += dy[q];
       }
+      t2 = rows(t2);
+      if (lane == 0) r2 += (double)t2;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const float w3 = sm.w3[rg + 8 * i];
@@ -289,10 +290,9 @@ __global__ void __launch_bounds__(LG_T, 3) k_loss_grad(const float *__restrict__
     atomicAdd(&grad[o], row[m][a]);
   }
   gb3 = rows(gb3);
-  r2 = rows(r2);
   if (lane == 0) {
     atomicAdd(&grad[O_B3], gb3);
-    atomicAdd(loss, (double)r2);
+    atomicAdd(loss, r2);
   }
 }
 
