@@ -118,6 +118,7 @@ struct LossGradSmem {
   alignas(16) float x[NIN][LG_S];
   float t[LG_S];
   float row[LG_T / 32][6][NH];   // per warp: sums over the samples of d2, dy h2, d1, d1 x
+  float gb3[LG_T / 32];          // and of dy
 };
 static_assert(offsetof(LossGradSmem, w2) % 16 == 0 && offsetof(LossGradSmem, h1) % 16 == 0 &&
                   offsetof(LossGradSmem, d2) % 16 == 0 && offsetof(LossGradSmem, x) % 16 == 0 && LG_LD % 4 == 0 &&
@@ -283,17 +284,21 @@ __global__ void __launch_bounds__(LG_T, 3) k_loss_grad(const float *__restrict__
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) atomicAdd(&grad[O_W2 + (ga + 16 * i) * NH + gb + 8 * j], gw[i][j]);
-  __syncwarp();
-  for (int k = lane; k < 6 * NH; k += 32) {
-    const int m = k / NH, a = k % NH;
-    const int o = m == 0 ? O_B2 + a : (m == 1 ? O_W3 + a : (m == 2 ? O_B1 + a : O_W1 + 3 * a + m - 3));
-    atomicAdd(&grad[o], row[m][a]);
-  }
+  // one addition per block and entry: more partial sums mean more roundings
+  // against the full one (a warp each: 1.5 times the error against 64 bits)
   gb3 = rows(gb3);
   if (lane == 0) {
-    atomicAdd(&grad[O_B3], gb3);
+    sm.gb3[tid >> 5] = gb3;
     atomicAdd(loss, r2);
   }
+  __syncthreads();
+  static_assert(LG_T == 128, "four warps' sums");
+  for (int k = tid; k < 6 * NH; k += LG_T) {
+    const int m = k / NH, a = k % NH;
+    const int o = m == 0 ? O_B2 + a : (m == 1 ? O_W3 + a : (m == 2 ? O_B1 + a : O_W1 + 3 * a + m - 3));
+    atomicAdd(&grad[o], (sm.row[0][m][a] + sm.row[1][m][a]) + (sm.row[2][m][a] + sm.row[3][m][a]));
+  }
+  if (tid == 0) atomicAdd(&grad[O_B3], (sm.gb3[0] + sm.gb3[1]) + (sm.gb3[2] + sm.gb3[3]));
 }
 
 __global__ void k_adam(int n, float *w, float *m, float *v, const float *g, float lr, float b1, float b2, float eps,
