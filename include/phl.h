@@ -338,6 +338,18 @@ phl_status phl_dt_device_ptr(phl_grid *g, const double **ptr);
  * pipe.  Host arrays of n values; |k| < 800 (PHL_EINVAL otherwise). */
 phl_status phl_convert_batch(long n, const double *x, int k, float *f, double *back);
 
+/* The FP64 helpers of the kernels (short reciprocals and roots, bit tests), for
+ * unit tests: out[2 i], out[2 i + 1] for each a[i], b[i], c[i]:
+ *   op 0  1 / a and b / a
+ *      1  sqrt(a) and 1 / sqrt(a)
+ *      2  b < a < c (b, c positive) and |a| below the normal range
+ *      3  |a| < 2^-10 and |a| < 2^-18
+ *      4  a with negative values (not NaN) replaced by 0; 0
+ *      5  a as a table position in [0, b], b an integer: index of its interval
+ *         in [0, b - 1] (-1 outside) and its fraction there
+ * Tests give 1 or 0.  Host arrays; PHL_EINVAL for a bad n or op. */
+phl_status phl_fp64_math_batch(long n, int op, const double *a, const double *b, const double *c, double *out);
+
 /* Evaluate the library's face flux (the device Riemann solver of the stage)
  * for n independent faces -- for unit tests of the solver itself.
  *   wl, wr  [n][9 + nspec] normal-frame primitive deviations, in order

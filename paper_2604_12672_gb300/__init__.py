@@ -138,6 +138,7 @@ _SIGS = {
     "phl_eos_table_export": (C.c_int, [C.c_void_p, C.c_void_p, C.c_long]),
     "phl_eos": (C.c_int, [C.c_void_p, C.c_long] + [C.c_void_p] * 10 + [C.c_int, C.c_double, C.c_int, C.c_int,
                                                                           C.c_void_p]),
+    "phl_fp64_math_batch": (C.c_int, [C.c_long, C.c_int] + [C.c_void_p] * 4),
     "phl_riemann_batch": (C.c_int, [C.c_long, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int,
                                     C.c_int, C.c_double, C.c_int, C.c_void_p]),
     "phl_poisson_create": (C.c_int, [C.c_void_p, C.POINTER(C.c_void_p)]),
@@ -207,6 +208,19 @@ def convert_batch(x, k):
     back = np.empty(x.shape, np.float64)
     _check(lib().phl_convert_batch(x.size, x.ctypes.data, int(k), f.ctypes.data, back.ctypes.data))
     return f, back
+
+
+FP64_MATH = {"rcp": 0, "sqrt": 1, "between": 2, "below_pow2": 3, "not_below_zero": 4, "interval": 5}
+
+
+def fp64_math_batch(op, a, b=None, c=None):
+    """The kernels' FP64 helpers on n values (see phl_fp64_math_batch in include/phl.h): (n, 2) results."""
+    a = np.ascontiguousarray(a, dtype=np.float64)
+    b, c = (np.ascontiguousarray(np.broadcast_to(0.0 if v is None else v, a.shape), dtype=np.float64) for v in (b, c))
+    out = np.zeros((a.size, 2))
+    _check(lib().phl_fp64_math_batch(a.size, FP64_MATH[op], a.ctypes.data, b.ctypes.data, c.ctypes.data,
+                                     out.ctypes.data))
+    return out
 
 
 def riemann_batch(wl, wr, bn, bg=None, nspec=0, solver="lhlld", mach_thr=0.6, precision="fp64"):

@@ -5,16 +5,18 @@
 // dozen and more.  These start from the hardware's gross approximations
 // (PTX rcp.approx.ftz.f64, rsqrt.approx.ftz.f64: relative error below 2^-19)
 // and take one third-order step of the Newton-Halley iteration, which leaves
-// a relative error below 2^-56 plus the rounding of the last operation: about
-// one unit in the last place for normal arguments.  The FP32 overloads are
-// the plain operations.
+// a relative error below 2^-56 plus the roundings: below 0.6 units in the last
+// place for the reciprocal, 1.7 for the quotient, 1.1 for the root and 1.2 for
+// its reciprocal, for arguments and results in the normal range.  The FP32
+// overloads are the plain operations.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace phl {
 
-// 1/x: y (1 + e + e^2), e = 1 - x y.  Three FP64 multiply-adds.  0 and
-// infinity give NaN.
+// 1/x: y (1 + e + e^2), e = 1 - x y.  Three FP64 multiply-adds.  Zero, an
+// argument below the normal range and infinity give NaN; above 2^1022, where
+// the result is below the normal range, it is 0.
 __device__ __forceinline__ double rcp_nr(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -84,7 +86,7 @@ __device__ __forceinline__ bool interval(float g, int n, int &i, float &u) {
   return true;
 }
 
-// x < 0 ? 0 : x by the sign bit; NaN stays NaN
+// x < 0 ? 0 : x by the sign bit (-0 gives +0); NaN stays NaN
 __device__ __forceinline__ double not_below_zero(double x) {
   const int hi = __double2hiint(x);
   return (hi < 0 && (unsigned)hi <= 0xfff00000u) ? 0.0 : x;
@@ -93,8 +95,9 @@ __device__ __forceinline__ float not_below_zero(float x) { return x < 0.0f ? 0.0
 
 // sqrt(x) and, in the second form, 1/sqrt(x): with y ~ 1/sqrt(x) and r = 1 -
 // x y^2, both are the approximation times 1 + r/2 + 3 r^2/8 (remaining error
-// 5 r^3 / 16 < 2^-57).  Five (six) FP64 instructions.  An argument below the
-// normal range gives 0 (infinity for the reciprocal), a negative one NaN.
+// 5 r^3 / 16 < 2^-55).  Five (six) FP64 instructions.  An argument below the
+// normal range, of either sign, gives 0 (infinity for the reciprocal), other
+// negative ones and +infinity NaN.
 __device__ __forceinline__ double sqrt_nr(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

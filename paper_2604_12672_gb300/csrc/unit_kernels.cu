@@ -3,6 +3,7 @@
 #include <string.h>
 
 #include "phl.h"
+#include "fp64_math.cuh"
 #include "phl_internal.cuh"
 #include "riemann_x2.cuh"
 
@@ -77,7 +78,41 @@ __global__ void k_convert_batch(long n, const double *x, int k, float *f, double
   }
 }
 
+__global__ void k_fp64_math(long n, int op, const double *a, const double *b, const double *c, double *out) {
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
+    const double x = a[t];
+    double r0 = 0.0, r1 = 0.0;
+    switch (op) {
+      case 0: r0 = rcp_nr(x); r1 = div_nr(b[t], x); break;
+      case 1: { double s; sqrt_rsqrt_nr(x, s, r1); r0 = sqrt_nr(x); break; }
+      case 2: r0 = between_pos(x, b[t], c[t]); r1 = below_normal(x); break;
+      case 3: r0 = below_pow2<10>(x); r1 = below_pow2<18>(x); break;
+      case 4: r0 = not_below_zero(x); break;
+      default: { int i; r0 = interval(x, (int)b[t], i, r1) ? (double)i : -1.0; break; }
+    }
+    out[2 * t] = r0;
+    out[2 * t + 1] = r1;
+  }
+}
+
 }  // namespace
+
+extern "C" phl_status phl_fp64_math_batch(long n, int op, const double *a, const double *b, const double *c,
+                                          double *out) {
+  if (n < 0 || op < 0 || op > 5) return (phl_status)set_error(PHL_EINVAL, "phl_fp64_math_batch: bad n or op");
+  if (n == 0) return PHL_OK;
+  if (!a || !b || !c || !out) return (phl_status)set_error(PHL_EINVAL, "phl_fp64_math_batch: null argument");
+  double *d = nullptr;
+  if (cudaMalloc(&d, 5 * n * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return PHL_ENOMEM; }
+  const double *src[3] = {a, b, c};
+  for (int k = 0; k < 3; ++k) cudaMemcpy(d + k * n, src[k], n * sizeof(double), cudaMemcpyHostToDevice);
+  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+  k_fp64_math<<<blocks, 256>>>(n, op, d, d + n, d + 2 * n, d + 3 * n);
+  cudaError_t e = cudaMemcpy(out, d + 3 * n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  if (e != cudaSuccess) { cudaGetLastError(); return PHL_ECUDA; }
+  return PHL_OK;
+}
 
 extern "C" phl_status phl_convert_batch(long n, const double *x, int k, float *f, double *back) {
   if (n < 0 || k <= -800 || k >= 800)
