@@ -345,7 +345,8 @@ phl_status phl_convert_batch(long n, const double *x, int k, float *f, double *b
  *      2  b < a < c (b, c positive) and |a| below the normal range
  *      3  |a| < 2^-10 and |a| < 2^-18
  *      4  a with negative values (not NaN) replaced by 0; 0
- *      5  a as a table position in [0, b], b an integer: index of its interval
+ *      5  a > 0, and finite too
+ *      6  a as a table position in [0, b], b an integer: index of its interval
  *         in [0, b - 1] (-1 outside) and its fraction there
  * Tests give 1 or 0.  Host arrays; PHL_EINVAL for a bad n or op. */
 phl_status phl_fp64_math_batch(long n, int op, const double *a, const double *b, const double *c, double *out);

@@ -210,7 +210,8 @@ def convert_batch(x, k):
     return f, back
 
 
-FP64_MATH = {"rcp": 0, "sqrt": 1, "between": 2, "below_pow2": 3, "not_below_zero": 4, "interval": 5}
+FP64_MATH = {"rcp": 0, "sqrt": 1, "between": 2, "below_pow2": 3, "not_below_zero": 4, "positive": 5,
+             "interval": 6}
 
 
 def fp64_math_batch(op, a, b=None, c=None):

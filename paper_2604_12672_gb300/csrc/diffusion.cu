@@ -156,9 +156,7 @@ __global__ void k_diff_init(DevGeo G, Box box, const double *__restrict__ U, con
     const double by = Bf[pl + ps] + Bf[pl + ps + G.sy];
     const double bz = Bf[2 * pl + ps] + Bf[2 * pl + ps + G.sz];
     e = (U[4 * pl + ps] - 0.5 * ((mx * mx + my * my + mz * mz) * ir + 0.25 * (bx * bx + by * by + bz * bz))) * ir;
-    if (!positive(r) || !positive(e)) {   // false for infinities and NaN too
-      if (!(r > 0.0) || !(e > 0.0)) atomicOr(dflag, FLAG_NEG);
-    }
+    if (!positive(r) || !positive(e)) atomicOr(dflag, FLAG_NEG);
     kr = p.k0 * powi_dev(ir, p.nR);
     if (MX) {   // kp and a as raw floats, rescaled once the maxima are known
       M.Y0d[q] = e;

@@ -33,9 +33,15 @@ __device__ __forceinline__ bool below_normal(double x) {
   return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x00100000u;
 }
 
-// x > 0 without an FP64 compare (those run on the FP64 pipe): true for
-// positive finite values from 2^-1042 up; false for NaN and infinity too.
-__device__ __forceinline__ bool positive(double x) { return (unsigned)__double2hiint(x) - 1u < 0x7fefffffu; }
+// x > 0 without an FP64 compare (those run on the FP64 pipe): positive doubles
+// order as their bits, 0 wraps to the top.  The second form is false for
+// infinity too.
+__device__ __forceinline__ bool positive(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool positive_finite(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7fefffffffffffffull;
+}
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
 // lo < x < hi for positive lo, hi: positive doubles order as their bits (false
 // for NaN, no FP64 compare)

@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(SPT, 2) k_sph_prims_st(SphDev D, SphWork<R> Wk
     if (it < 0) atomicOr(D.dflag, FLAG_NEWTON);
     D.T[c] = T;
     const double P = o.P * D.ip_u;
-    if (!positive(rho) || !positive(P)) {   // false for infinities and NaN too
+    if (!positive_finite(rho) || !positive_finite(P)) {
       if (!(rho > 0.0) || !(P > 0.0)) atomicOr(D.dflag, FLAG_NEG);
       if (!isfinite(rho) || !isfinite(P)) atomicOr(D.dflag, FLAG_NAN);
     }

@@ -88,6 +88,7 @@ __global__ void k_fp64_math(long n, int op, const double *a, const double *b, co
       case 2: r0 = between_pos(x, b[t], c[t]); r1 = below_normal(x); break;
       case 3: r0 = below_pow2<10>(x); r1 = below_pow2<18>(x); break;
       case 4: r0 = not_below_zero(x); break;
+      case 5: r0 = positive(x); r1 = positive_finite(x); break;
       default: { int i; r0 = interval(x, (int)b[t], i, r1) ? (double)i : -1.0; break; }
     }
     out[2 * t] = r0;
@@ -99,7 +100,7 @@ __global__ void k_fp64_math(long n, int op, const double *a, const double *b, co
 
 extern "C" phl_status phl_fp64_math_batch(long n, int op, const double *a, const double *b, const double *c,
                                           double *out) {
-  if (n < 0 || op < 0 || op > 5) return (phl_status)set_error(PHL_EINVAL, "phl_fp64_math_batch: bad n or op");
+  if (n < 0 || op < 0 || op > 6) return (phl_status)set_error(PHL_EINVAL, "phl_fp64_math_batch: bad n or op");
   if (n == 0) return PHL_OK;
   if (!a || !b || !c || !out) return (phl_status)set_error(PHL_EINVAL, "phl_fp64_math_batch: null argument");
   double *d = nullptr;

@@ -79,6 +79,8 @@ def test_bit_tests(P):
     with np.errstate(invalid="ignore"):
         got = P.fp64_math_batch("below_pow2", x)
         assert np.array_equal(got[:, 0], np.abs(x) < 2.0 ** -10) and np.array_equal(got[:, 1], np.abs(x) < 2.0 ** -18)
+        got = P.fp64_math_batch("positive", x)
+        assert np.array_equal(got[:, 0], x > 0) and np.array_equal(got[:, 1], (x > 0) & np.isfinite(x))
         got = P.fp64_math_batch("not_below_zero", x)[:, 0]
         assert np.array_equal(got, np.where(x < 0, 0.0, x), equal_nan=True)
         for lo, hi in ((1e7, 1e10), (5e-324, np.inf), (1.0, 1.0)):
