@@ -253,7 +253,7 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
       launch_eos_cells<double>(G, S.Uin, S.Bin, nullptr, nullptr, S.Tin, S.Tout, S.W, S.dflag, s, &nl, prof,
                                S.cfl_dmax, const_cast<double *>(S.dt));
     } else {
-      const unsigned t = tpb_for(b.n);
+      const unsigned t = tpb_for(G, b.n);
       PHL_LAUNCH(KC_PRIM, prof, s, k_prim<<<gridt(b, t), t, 0, s>>>(G, b, S.Uin, S.Bin, S.W, S.dflag, S.cfl_dmax, S.any));
       if (S.cfl_dmax) {
         PHL_LAUNCH(KC_DT, prof, s, k_dt_finalize<<<1, 1, 0, s>>>(G.cfl, S.cfl_dmax, const_cast<double *>(S.dt)));
@@ -280,12 +280,14 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
   }
   // one launch for all directions, and one for the EMFs and the cell update,
   // where a direction's faces are fewer than the GPU's threads in a wave (128
-  // x 128: 40 + 12 -> 28 + 8 us a stage, and two launches fewer)
+  // x 128: 40 + 12 -> 28 + 8 us a stage, and two launches fewer; a step in
+  // both forms: 128^2 177 and 236 us, 256^2 432 and 467, 32^3 442 and 466, and
+  // above the line 288^2 574 and 644, 56^3 1614 and 1723)
   // (a grid without an active axis has no faces: nothing to launch for them)
-  const bool small = most > 0 && most < 4L * 152 * 128 && G.recon == PHL_RECON_VANLEER;
+  const bool small = most > 0 && most < G.sms * 512L && G.recon == PHL_RECON_VANLEER;
   if (small) {
     FaceSet<double> A{};
-    const unsigned t = most < 152L * 128 ? 32u : 64u;
+    const unsigned t = most < G.sms * 128L ? 32u : 64u;
     unsigned blocks = 0;
     for (int D = 0; D < 3; ++D) {
       A.first[D] = ~0u;
@@ -310,11 +312,11 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
   // (4) edge EMFs
   const Box bs = site_box(G), bc = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
   if (small) {
-    const unsigned t = tpb_for(bs.n), nemf = gridt(bs, t).x;
+    const unsigned t = tpb_for(G, bs.n), nemf = gridt(bs, t).x;
     PHL_LAUNCH(KC_EMF, prof, s, k_emf_cells<<<nemf + gridt(bc, t).x, t, 0, s>>>(G, bs, bc, nemf, S));
     ++nl;
   } else {
-    const unsigned t = tpb_for(bs.n);
+    const unsigned t = tpb_for(G, bs.n);
     PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<double><<<gridt(bs, t), t, 0, s>>>(G, bs, S.W, S.F[0], S.F[1], S.F[2], S.E));
     PHL_LAUNCH(KC_UPDATE_CELLS, prof, s, k_update_cells<<<gridt(bc, t), t, 0, s>>>(G, bc, S));
     nl += 2;
@@ -322,7 +324,7 @@ void launch_stage_fp64(const DevGeo &G, const StageBufs &S, cudaStream_t s, int 
   // (5) face updates
   {
     const Box bu = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
-    const unsigned t = tpb_for(bu.n);
+    const unsigned t = tpb_for(G, bu.n);
     PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces<<<gridt(bu, t), t, 0, s>>>(G, bu, S));
     ++nl;
   }

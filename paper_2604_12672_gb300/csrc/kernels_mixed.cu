@@ -235,7 +235,7 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
   }
   if (!fused) {
     const Box bs = site_box(G);
-    const unsigned t = tpb_for(bs.n);
+    const unsigned t = tpb_for(G, bs.n);
     PHL_LAUNCH(KC_EMF, prof, s, k_emf_all<float><<<gridt(bs, t), t, 0, s>>>(G, bs, M.W, M.F[0], M.F[1], M.F[2], M.E));
     ++nl;
   }
@@ -250,7 +250,7 @@ void launch_stage_mixed(const DevGeo &G, const MixedBufs &M, int stage, int nsta
   }
   if (!fused) {
     const Box bf = make_box(0, G.n[0] + 1, 0, G.n[1] + 1, 0, G.n[2] + 1);
-    const unsigned t = tpb_for(bf.n);
+    const unsigned t = tpb_for(G, bf.n);
     PHL_LAUNCH(KC_UPDATE_FACES, prof, s, k_update_faces_mx<<<gridt(bf, t), t, 0, s>>>(G, bf, S));
     ++nl;
   }

@@ -33,6 +33,7 @@ struct phl_mlp {
   float b3 = 0.0f;
   float c[4] = {6.0f, 18.0f, 0.5f, 8.75f}, s[4] = {1.0f, 1.0f, 2.0f, 1.0f};
   long adam_t = 0;
+  int sms = phl::sm_count();
 };
 
 namespace phl {
@@ -388,7 +389,7 @@ cudaError_t launch_loss_grad(phl_mlp *M, long nb, const float *x, const float *t
   cudaMemsetAsync(M->grad, 0, NPARAM * sizeof(float), s);
   cudaMemsetAsync(loss, 0, sizeof(double), s);
   // three blocks fit an SM; a block's tiles share its weights and its sums
-  const unsigned grid = (unsigned)std::min<long>((nb + LG_S - 1) / LG_S, 3 * 152);
+  const unsigned grid = (unsigned)std::min<long>((nb + LG_S - 1) / LG_S, 3L * M->sms);
   k_loss_grad<<<grid, LG_T, LG_SMEM, s>>>(M->w, nb, x, t, 1.0f / (float)nb, M->grad, loss);
   return cudaGetLastError();
 }

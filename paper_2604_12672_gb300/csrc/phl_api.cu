@@ -55,6 +55,12 @@ int set_error(int st, const char *fmt, ...) {
   va_end(ap);
   return st;
 }
+int sm_count() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
 }  // namespace phl
 
 struct phl_grid {
@@ -400,6 +406,7 @@ phl_status phl_create_grid(const phl_grid_desc *d, phl_grid **out) {
   G.eps_sf = d->eps_sf;
   G.mach_thr = d->mach_thr;
   G.cfl = d->cfl;
+  G.sms = sm_count();
   {   // power-of-two unit scales of the mixed form's FP32 quantities
     double rho_ref = 1.0, p_ref = 1.0, dx_min = 0.0;
     if (d->bg_rho_c && d->bg_p_c) {

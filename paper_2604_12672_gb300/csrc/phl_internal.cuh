@@ -82,6 +82,7 @@ struct DevGeo {
   mlp::Dev mlp;
   unsigned long long *niter;   // Newton iterations summed over cells (device)
   double *pred;                // mixed stellar form: 8 planes, each cell's last inversion (eos::Pred)
+  int sms;                     // SMs of the grid's device (launch rules)
 };
 
 __host__ __device__ __forceinline__ long sidx(const DevGeo &G, int i, int j, int k) {
@@ -460,6 +461,8 @@ __host__ __device__ __forceinline__ double iusc(const DevGeo &G, int v) {
 // Records the calling thread's last-error message (phl_last_error) and
 // returns st (phl_api.cu).
 int set_error(int st, const char *fmt, ...);
+// SMs of the current device (phl_api.cu).
+int sm_count();
 
 // Device scratch of one call on host arrays, from the device's pool
 // (scratch.cu): given back to it in stream order when the call returns.

@@ -394,9 +394,12 @@ __global__ void __launch_bounds__(256) k_flag_box(DevGeo G, Box box, const uint8
 }
 
 // Block size of the one-thread-per-element kernels: 256, or 64 where 256
-// would leave SMs without a block (the FP64 kernels of a 128^2 grid: 65 blocks
-// on 152 SMs, each SM's FP64 pipe serving eight warps while others idle).
-inline unsigned tpb_for(long n) { return n < 2L * 152 * 256 ? 64u : 256u; }
+// would leave SMs without a block or with a second one here and there (the FP64
+// kernels of a 128^2 grid: 65 blocks on 152 SMs, each SM's FP64 pipe serving
+// eight warps while others idle).  FP64 step with 64 against 256: 16^3 168 and
+// 198 us, 128^2 177 and 186; above the line 320^2 702 and 720, 384^2 913 and
+// 916, and the mixed form's kernels 288^2 162 and 153.
+inline unsigned tpb_for(const DevGeo &G, long n) { return n < 2L * G.sms * 256 ? 64u : 256u; }
 inline dim3 gridt(const Box &b, unsigned t) { return dim3((unsigned)((b.n + t - 1) / t), 1, 1); }
 
 // Raw flags (W holds the stage input), then the flags of the cells the face
@@ -407,7 +410,7 @@ inline int launch_flags(const DevGeo &G, const R *W, uint8_t *raw, uint8_t *tmp,
                         Prof *prof, bool zeroed = false) {
   Box bi = make_box(0, G.n[0], 0, G.n[1], 0, G.n[2]);
   if (!zeroed) cudaMemsetAsync(any, 0, sizeof(unsigned int), s);
-  const unsigned t = tpb_for(bi.n);
+  const unsigned t = tpb_for(G, bi.n);
   PHL_LAUNCH(KC_FLAG_RAW, prof, s, k_flag_raw<R><<<gridt(bi, t), t, 0, s>>>(G, bi, W, raw, any));
   int l[3], h[3];
   for (int d = 0; d < 3; ++d) {
@@ -419,9 +422,9 @@ inline int launch_flags(const DevGeo &G, const R *W, uint8_t *raw, uint8_t *tmp,
     return 2;
   }
   const int ntx = (G.n[0] + DF - 1) / DF, nty = (G.n[1] + DF - 1) / DF, ntz = (G.n[2] + DF - 1) / DF;
-  const long nt = (long)ntx * nty * ntz;
+  const long nt = (long)ntx * nty * ntz, most = 8L * G.sms;
   PHL_LAUNCH(KC_FLAG_DILATE, prof, s,
-             k_flag_dilate3<<<(unsigned)(nt < 8L * 152 ? nt : 8L * 152), 256, 0, s>>>(G, raw, tmp, ntx, nty, any));
+             k_flag_dilate3<<<(unsigned)(nt < most ? nt : most), 256, 0, s>>>(G, raw, tmp, ntx, nty, any));
   PHL_LAUNCH(KC_FLAG_DILATE, prof, s, k_flag_expand<<<gridt(be, 256), 256, 0, s>>>(G, be, tmp, flag, any));
   return 3;
 }
@@ -729,13 +732,15 @@ inline void launch_flux(int D, const DevGeo &G, const Box &b, const R *W, const 
   // arithmetic, and strided loads cost more there (stellar box 128^3: 129-172
   // us a direction walking, 101-111 one face per thread)
   if (sizeof(R) == 8 && G.recon == PHL_RECON_VANLEER) {
-    // faces per thread: as many as leave several blocks per SM
+    // faces per thread: as many as leave several blocks per SM (FP64 step with
+    // 1, 2, 4 faces: 53^3 1547, 1555, 1508 us; 67^3 2849, 2759, 2829; 84^3 5388,
+    // 5079, 5083; 112^3 12286, 11463, 11192, and 11660 with 8)
     const int step = b.n >= 600000 ? 4 : (b.n >= 150000 ? 2 : 1);
     const int nD = b.hi[D];
     int h[3] = {b.hi[0], b.hi[1], b.hi[2]};
     h[D] = (nD + step - 1) / step;
     const Box bw = make_box(b.lo[0], h[0], b.lo[1], h[1], b.lo[2], h[2]);
-    const unsigned t = bw.n < 152L * 128 ? 32u : (bw.n < 4L * 152 * 128 ? 64u : 128u);
+    const unsigned t = bw.n < G.sms * 128L ? 32u : (bw.n < G.sms * 512L ? 64u : 128u);
 #define PHL_FLUX(DD, NN) \
   PHL_LAUNCH(kc, prof, s, (k_flux_walk<DD, R, NN><<<gridt(bw, t), t, 0, s>>>(G, bw, nD, step, W, Bf, dB, flag, F, dflag)))
     if (G.nspec == 0) {

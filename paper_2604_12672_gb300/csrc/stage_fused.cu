@@ -1303,8 +1303,10 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
   // at most one tile per SM: twice the threads per tile (one face each instead
   // of two), and the tile dilates the raw flags itself -- with one CTA per SM
   // a tile's own latency is the launch's time (32 x 32 x 48 with flags: 15.5 +
-  // 4.9 us in two launches -> 13.4 us in one)
-  const bool few = nb <= 152 && M.fused_variant == PHL_FUSED_DEFAULT;
+  // 4.9 us in two launches -> 13.4 us in one; a step with this form and the
+  // other: 96 tiles 122 and 146 us, 152 tiles 126 and 145; above the line 160
+  // tiles 155 and 163, 288 tiles 169 and 172, 320 tiles 201 and 196)
+  const bool few = nb <= G.sms && M.fused_variant == PHL_FUSED_DEFAULT;
   const uint8_t *dil = nullptr;
   const unsigned int *any = nullptr;
   int raw_mode = 0;
@@ -1326,7 +1328,7 @@ void launch_fused_tail(const DevGeo &G, const MixedBufs &M, bool first, bool las
       dil = M.raw;
       raw_mode = 1;
     } else {
-      const int nbd = std::min(nb, 8 * 152);   // eight 256-thread CTAs per SM
+      const int nbd = std::min(nb, 8 * G.sms);   // eight 256-thread CTAs per SM
       PHL_LAUNCH(KC_FLAG_DILATE, prof, s,
                  k_flag_dilate3<<<nbd, 256, 0, s>>>(G, M.raw, M.raw + ncell, ntx, nty, M.anyraw));
       dil = M.raw + ncell;
