@@ -150,7 +150,7 @@ phl_status phl_eos_table_create(double lrhoye_lo, double lrhoye_hi, int nrho, do
   t->t.dx = (lrhoye_hi - lrhoye_lo) * log(10.0) / (nrho - 1);
   t->t.y0 = lT_lo * log(10.0);
   t->t.dy = (lT_hi - lT_lo) * log(10.0) / (nT - 1);
-  t->t.x0f = (float)t->t.x0; t->t.dxf = (float)t->t.dx; t->t.y0f = (float)t->t.y0; t->t.dyf = (float)t->t.dy;
+  t->t.x0f = (float)t->t.x0; t->t.y0f = (float)t->t.y0;
   t->t.idx = 1.0 / t->t.dx; t->t.idy = 1.0 / t->t.dy;
   t->t.idxdy = t->t.idx * t->t.idy; t->t.idx2x2 = 2.0 * t->t.idx * t->t.idx; t->t.idy2x2 = 2.0 * t->t.idy * t->t.idy;
   t->t.idxdyf = (float)t->t.idxdy; t->t.idx2x2f = (float)t->t.idx2x2; t->t.idy2x2f = (float)t->t.idy2x2;
@@ -184,7 +184,6 @@ phl_status phl_eos_table_create(double lrhoye_lo, double lrhoye_hi, int nrho, do
     phl_eos_table_destroy(t);
     return (phl_status)set_error(e != cudaSuccess ? PHL_ECUDA : PHL_ENEWTON, "eos table: node solve failed");
   }
-  t->t.v = t->dv;
   t->t.c = t->dc;
   t->t.cf = t->dcf;
   *out = t;

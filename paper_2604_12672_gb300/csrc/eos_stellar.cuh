@@ -61,10 +61,9 @@ __host__ __device__ __forceinline__ int qslot(int p, int r) {
 struct Table {
   int nx, ny;
   double x0, dx, y0, dy;      // x = ln n_e, y = ln T
-  const double *v;            // [ny][nx][NQ] (device)
   const double *c;            // [ny-1][nx-1][NCF] polynomial coefficients in cell units
   const float *cf;            // FP32 copy
-  float x0f, dxf, y0f, dyf;
+  float x0f, y0f;
   double idx, idy;            // 1/dx, 1/dy
   float idxf, idyf;
   double idxdy, idx2x2, idy2x2;   // idx idy, 2 idx^2, 2 idy^2 (the second derivatives come halved)
