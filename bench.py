@@ -49,9 +49,10 @@ FP64_NOMINAL_TFLOPS = 1.25     # GB300 FP64 (profiling recipe's nominal table)
 # input (5 cell + 3 face doubles), read U^n for stages 2-3, write the output.
 BYTES_PER_CELL_STAGE = {1: 128.0, 2: 192.0, 3: 192.0}
 # FP64 flux kernel: FP64 operations per face (DADD + DMUL + 2 DFMA counted from
-# the ncu counters of k_flux_walk on the stratified box at 128 x 96 x 112, mean
-# of the three directions).
-FP64_FLOP_PER_FACE = 475.6
+# the ncu counters of k_flux_walk on the benchmark's stratified box at 128^3,
+# mean of the three directions; a flow in every cell, with no slope cut to
+# zero, takes 476).
+FP64_FLOP_PER_FACE = 399.7
 # Mixed flux kernel: FP32 operations per face (FADD + FMUL + 2 FFMA from the ncu
 # SASS counters of k_flux<0/1/2, float> on the stratified box at 160^3, per sweep
 # direction), and its DRAM bytes per face (dram__bytes_read + write, same capture;
@@ -66,11 +67,11 @@ FP32_NOMINAL_TFLOPS = 80.5
 # FMUL + 2 FFMA, the packed FP32x2 forms counted twice): 405 per face over the
 # 3.375 faces per cell an 8^3 tile evaluates; the algorithmic count is 3 faces
 # per cell x 405 = 1215.  DRAM
-# bytes per cell (160^3, W larger than L2): 111.8 (stage 1, no increment
-# to read), 144.6 (stage 2) and 205.3 (stage 3, which also reads and writes
-# the FP64 state), 153.9 on average over an RK3 step.
+# bytes per cell (160^3, W larger than L2): 112.0 (stage 1, no increment
+# to read), 144.4 (stage 2) and 206.4 (stage 3, which also reads and writes
+# the FP64 state), 154.3 on average over an RK3 step.
 FUSED_FLOP_PER_CELL = 3.0 * 405.1
-FUSED_DRAM_BYTES_PER_CELL = (111.8 + 144.6 + 205.3) / 3.0
+FUSED_DRAM_BYTES_PER_CELL = (112.0 + 144.4 + 206.4) / 3.0
 
 
 def read_peaks():
@@ -727,22 +728,22 @@ def ensemble_c4(P, steps, warmup, stream, ws):
 
 
 # Cubed-sphere shell (FP64): the flux kernel's FP64 operations per face
-# (DADD + DMUL + 2 DFMA from the ncu SASS counters of k_sph_flux on the
-# 6 x 64 x 64 x 96 shell: 5307.0 M over 7.102 M faces) and its DRAM bytes
-# per face on 6 x 64^3 (517.4 MB; the work arrays exceed L2 there).
-SPH_FP64_FLOP_PER_FACE = 747.3
-SPH_FLUX_DRAM_BYTES_PER_FACE = 109.1
+# (DADD + DMUL + 2 DFMA from the ncu counters of k_sph_flux on the ideal-gas
+# 6 x 64 x 64 x 96 shell: 5218.0 M over 7.102 M faces) and its DRAM bytes
+# per face there (786.8 MB; the work arrays exceed L2).
+SPH_FP64_FLOP_PER_FACE = 734.7
+SPH_FLUX_DRAM_BYTES_PER_FACE = 110.8
 # the mixed form's flux kernel: FP32 operations per face, FADD + FMUL + 2 FFMA
-# of the scalar solver on the same shell (2533.6 M over 4.743 M faces; the
+# of the scalar solver on 6 x 64^3 (2533.6 M over 4.743 M faces; the
 # packed-lane solver the kernel runs does the same arithmetic, partly as
 # f32x2 instructions those counters leave out), and its DRAM bytes per face
-# (241.0 MB in the capture of the packed-lane kernel)
+# on 6 x 64 x 64 x 96 (398.2 MB in the capture of the packed-lane kernel)
 SPH_FP32_FLOP_PER_FACE = 534.2
 # the stellar shell's mixed inversion (k_sph_prims_st<float>, recorded path): FP64 operations and
 # FP64-pipe instructions per cell-stage, ncu on the 6 x 64 x 64 x 96 stellar shell
 SPH_ST_FP64_FLOP_PER_CELL = 346.0
 SPH_ST_FP64_INST_PER_CELL = 210.0
-SPH_MX_FLUX_DRAM_BYTES_PER_FACE = 50.8
+SPH_MX_FLUX_DRAM_BYTES_PER_FACE = 56.1
 
 
 def cubed_sphere_c5(P, steps, warmup, stream, alu, hbm_peak, peak_kind, N=256, Nr=384, precision="fp64",
@@ -833,7 +834,7 @@ def cubed_sphere_c5(P, steps, warmup, stream, alu, hbm_peak, peak_kind, N=256, N
         roof.update({"bound": "alu", "achieved": tf, "peak": alu["fp64"], "unit": "TFLOP/s",
                      "frac": tf / alu["fp64"], "flop_per_face": SPH_FP64_FLOP_PER_FACE,
                      "traffic": faces * SPH_FLUX_DRAM_BYTES_PER_FACE,
-                     "traffic_note": "ncu DRAM bytes per face on the 6 x 64^3 shell x faces",
+                     "traffic_note": "ncu DRAM bytes per face on the 6 x 64 x 64 x 96 shell x faces",
                      "peak_kind": "measured FP64 DFMA rate (phl_probe_alu)"})
     elif name == "sph_flux":
         # mixed: FP32 work arrays; W read once per cell, phi (FP64) and dPhi
@@ -846,7 +847,7 @@ def cubed_sphere_c5(P, steps, warmup, stream, alu, hbm_peak, peak_kind, N=256, N
         roof.update({"bound": "alu", "achieved": tf, "peak": alu["fp32"], "unit": "TFLOP/s",
                      "frac": tf / alu["fp32"], "flop_per_face": SPH_FP32_FLOP_PER_FACE,
                      "traffic": faces * SPH_MX_FLUX_DRAM_BYTES_PER_FACE,
-                     "traffic_note": "ncu DRAM bytes per face on the 6 x 64^3 shell x faces",
+                     "traffic_note": "ncu DRAM bytes per face on the 6 x 64 x 64 x 96 shell x faces",
                      "peak_kind": "measured FP32 FFMA rate (phl_probe_alu)"})
     out["roofline"] = roof
     return out
