@@ -817,7 +817,7 @@ def cubed_sphere_c5(P, steps, warmup, stream, alu, hbm_peak, peak_kind, N=256, N
                      "fp64_pipe_inst_per_cell": SPH_ST_FP64_INST_PER_CELL,
                      "fp64_pipe_inst_rate_frac": inst / (alu["fp64"] / 2.0),
                      "traffic": None,
-                     "note": "DADD + DMUL + 2 DFMA per cell from ncu on the 6 x 64^3 stellar shell; the "
+                     "note": "DADD + DMUL + 2 DFMA per cell from ncu on the 6 x 64 x 64 x 96 stellar shell; the "
                              "instruction rate against the DFMA probe's (one FP64-pipe instruction per DFMA)",
                      "peak_kind": "measured FP64 DFMA rate (phl_probe_alu)"})
     elif eos == "stellar":

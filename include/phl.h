@@ -246,7 +246,9 @@ phl_status phl_diffuse(phl_grid *g, const phl_diffusion *p, double dt, int max_s
  *           faces of all three directions in shared memory and applies the
  *           cell update; the primitives, raw shock flags and their dilation
  *           before it and the Contact-CT EMFs and face updates after it run as
- *           one kernel each (six launches per stage).  Needs
+ *           one kernel each (six launches per stage; grids of at most one
+ *           tile per SM run 576 threads per tile instead of 288, which also
+ *           dilates the flags: five launches).  Needs
  *           precision = PHL_MIXED, an ideal gas, nspec = 0 and at least four
  *           cells along each of three active dimensions (PHL_EUNSUPPORTED
  *           otherwise).  Default where eligible.
@@ -255,7 +257,7 @@ phl_status phl_diffuse(phl_grid *g, const phl_diffusion *p, double dt, int max_s
  *           shared buffer; 5 to 7 evaluate two faces per thread on packed
  *           FP32x2 arithmetic; 8 and 9 pair the left and right states of
  *           each face on FP32x2 arithmetic), for tuning; 1 selects the
- *           default shape.
+ *           default shape, 8, with its small-grid form (so 8 does too).
  *   on = 201..209: shapes 1..9 with the stage in three launches: (i) the
  *           tile kernel, which dilates the raw shock flags of its tile in
  *           shared memory; (ii) Contact-CT: the edge EMFs an 8^3 tile of
@@ -269,7 +271,7 @@ phl_status phl_diffuse(phl_grid *g, const phl_diffusion *p, double dt, int max_s
  *           phl_set_state_prim, phl_diffuse, a host phl_get_state, an
  *           ensemble step, this call) forms the primitives, raw flags and
  *           CFL step in their own kernels first.  Ten launches per step
- *           instead of twenty, but slower per cell on this GPU (the flag
+ *           instead of eighteen (fifteen on small grids), but slower per cell on this GPU (the flag
  *           dilation no longer overlaps the tile's copy; the halo primitives
  *           and the small CT tiles cost more than they save).
  *   on = 0: one kernel per direction for the faces, then EMFs and updates.

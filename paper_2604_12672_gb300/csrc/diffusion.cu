@@ -328,8 +328,9 @@ struct Raw {
 };
 
 // p[cell] of a plane: the plane's start (block-uniform, 64-bit) plus a 32-bit
-// offset within it in units of 4 bytes.  (A plane's byte offsets fit: the state
-// of 2^28 cells alone exceeds the device.)
+// element offset within it, added to the 64-bit pointer.  (Four times a cell's
+// offset fits too: 2^30 cells of a mixed grid with its diffusion arrays take
+// more than 280 bytes each, more than the device has.)
 template <class T>
 __device__ __forceinline__ T pld(const T *p, long plane, unsigned off) {
   return __ldg(p + plane + off);
