@@ -184,7 +184,10 @@ phl_status phl_get_stats(phl_grid *g, phl_stats *st);
 /* Per-kernel device timing.  When enabled, every kernel launch of the grid is
  * bracketed by CUDA events on the grid's stream; phl_kernel_times folds the
  * recorded pairs (synchronising) into per-kernel totals since the last reset.
- * Kernel classes are named ("prim", "flux_x", "stage_mixed", ...). */
+ * Kernel classes are named ("prim", "flux_x", "stage_mixed", ...).  An FP64
+ * grid of less than one wave of faces runs the faces of all directions in one
+ * launch, counted as "flux_x", and the EMFs and the cell update in one,
+ * counted as "emf". */
 typedef struct {
   char name[32];
   long launches;
